@@ -458,6 +458,17 @@ int fire_selftest_tc_gemm(int64_t M, int32_t N, int32_t K, int32_t nc, const voi
  * iters < 1, blocks < 1 or out == NULL. */
 int fire_selftest_fma_rate(int32_t dtype, int64_t iters, int32_t blocks, void* out, void* stream);
 
+/* Diagnostic: the SIMT matrix product of the float32 and float64 forms on its
+ * own (dtype 0: float64, 1: float32).  For z < batch: C_z[M][N] (+)= A[M][K]
+ * op(B_z), op(B) = B[K][N] or, with transB, the transpose of B[N][K]; row
+ * strides lda, ldb, ldc; B_z = B + z sB, C_z = C + z sC (elements).  With
+ * accumulate the products are added to C.  The paper has no counterpart: this
+ * exists to test the kernel in isolation.  FIRE_ERR_INVALID_ARG on a bad
+ * dtype, a size below 1, a row stride shorter than its row or a NULL pointer. */
+int fire_selftest_simt_gemm(int32_t dtype, int64_t M, int32_t N, int32_t K, int32_t batch, int32_t transB,
+                            int32_t accumulate, const void* A, int64_t lda, const void* B, int64_t ldb,
+                            int64_t sB, void* C, int64_t ldc, int64_t sC, void* stream);
+
 /* Size of the workspace that fire_local_energy_static() owns (32 MiB). */
 #define FIRE_STATIC_WORKSPACE_BYTES (32u * 1024u * 1024u)
 

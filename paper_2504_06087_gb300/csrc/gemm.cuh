@@ -1,11 +1,16 @@
 // SIMT matrix product C = A * op(B) over row ranges of the forward-Laplacian
 // tensors, for the float32 and float64 forms.
 //
-// A is row-major [M][K] (lda), B row-major [K][N] (ldb) or, with TRANS_B,
+// A is row-major [M][K] (lda), B row-major [K][N] (ldb) or, with TB,
 // [N][K]; C row-major [M][N] (ldc).  The row range may live on the device
 // (m_range = {begin, end}), so a launch can be enqueued before the ragged row
 // counts are known; tiles past the end exit at once.  grid.z batches
-// independent products with element strides sA, sB, sC.
+// independent products with element strides sA, sB, sC.  Products of one A
+// with several B whose results lie side by side are one product whose
+// columns come from B in blocks of nb (element stride sB between blocks).
+//
+// Every output is one chain of fused multiply-adds over k in ascending order,
+// whatever the tile, so the result does not depend on the tile chosen.
 #pragma once
 
 #include "common.cuh"
@@ -22,15 +27,58 @@ struct GemmArgs {
   int64_t m_begin, m_end;        // used when m_range == nullptr
   const int64_t* m_range;        // device {begin, end} or nullptr
   int N, K;
+  int nb;                        // columns per block of B
   int accumulate;
+  int va, vb, vc;                // 16-byte loads of A and of B, 16-byte stores of C
 };
 
+// c += a * b for a pair of columns: one packed instruction for float32 (two
+// lanes, each rounded like fmaf), which leaves the issue slots of the other
+// half to the shared-memory loads.
+__device__ __forceinline__ void fma_pair(float& c0, float& c1, float a, float b0, float b1) {
+  asm("{\n .reg .b64 x, y, z;\n mov.b64 x, {%2, %2};\n mov.b64 y, {%3, %4};\n mov.b64 z, {%0, %1};\n"
+      " fma.rn.f32x2 z, x, y, z;\n mov.b64 {%0, %1}, z;\n}"
+      : "+f"(c0), "+f"(c1) : "f"(a), "f"(b0), "f"(b1));
+}
+__device__ __forceinline__ void fma_pair(double& c0, double& c1, double a, double b0, double b1) {
+  c0 = fma(a, b0, c0);
+  c1 = fma(a, b1, c1);
+}
+
+// VN consecutive elements, aligned to their size.
+template <typename T, int VN>
+__device__ __forceinline__ void ld_vec(T (&v)[VN], const T* p) {
+  constexpr int W = 16 / (int)sizeof(T) < VN ? 16 / (int)sizeof(T) : VN;
+  struct alignas(W * sizeof(T)) Vec { T x[W]; };
+#pragma unroll
+  for (int q = 0; q < VN; q += W) {
+    const Vec u = *reinterpret_cast<const Vec*>(p + q);
+#pragma unroll
+    for (int i = 0; i < W; ++i) v[q + i] = u.x[i];
+  }
+}
+
+// One BM x BN tile per CTA; a thread owns TM x TN outputs as groups of at most
+// four consecutive rows and columns, so a warp's shared loads are 128-bit
+// broadcasts without bank conflicts.  The next BK-deep slab is in registers
+// while the current one is multiplied.
 template <typename T, int BM, int BN, int BK, int TM, int TN, bool TB>
 __global__ void __launch_bounds__((BM / TM) * (BN / TN))
 gemm_kernel(GemmArgs<T> g) {
   constexpr int NT = (BM / TM) * (BN / TN);
-  __shared__ T As[2][BK][BM + 4];
-  __shared__ T Bs[2][BK][BN + 4];
+  constexpr int VE = 16 / (int)sizeof(T);          // elements of a 16-byte load
+  constexpr int GM = TM < 4 ? TM : 4, GN = TN < 4 ? TN : 4;
+  constexpr int RM = TM / GM, RN = TN / GN;        // row and column groups of a thread
+  constexpr int NX = BN / TN;                      // threads along the columns
+  constexpr int LX = NX < 8 ? NX : 8, LY = 32 / LX;   // warp: LY x LX threads
+  static_assert(NT % 32 == 0 && (BM / TM) % LY == 0 && NX % LX == 0, "warp layout");
+  constexpr int AC = BM * BK / VE / NT, KC = BK / VE;
+  static_assert(AC >= 1 && NT % KC == 0, "A slab");
+  constexpr int BC = BK * BN / VE / NT, NC = BN / VE;
+  static_assert(BC >= 1 && (TB ? NT % KC == 0 : NT % NC == 0 || NC % NT == 0), "B slab");
+  constexpr int PAD = 4;
+  __shared__ __align__(16) T As[2][BK][BM + PAD];
+  __shared__ __align__(16) T Bs[2][BK][BN + PAD];
   int64_t mb = g.m_begin, me = g.m_end;
   if (g.m_range) { mb = g.m_range[0]; me = g.m_range[1]; }
   const int64_t m0 = mb + (int64_t)blockIdx.x * BM;
@@ -40,9 +88,27 @@ gemm_kernel(GemmArgs<T> g) {
   const T* B = g.B + g.sB * blockIdx.z;
   T* C = g.C + g.sC * blockIdx.z;
   const int tid = threadIdx.x;
-  const int tx = tid % (BN / TN), ty = tid / (BN / TN);
-  constexpr int A_PER = BM * BK / NT, B_PER = BK * BN / NT;
-  T ra[A_PER], rb[B_PER];
+  const int wid = tid >> 5, lane = tid & 31;
+  const int tx = (wid % (NX / LX)) * LX + lane % LX, ty = (wid / (NX / LX)) * LY + lane / LX;
+  // A slab: thread loads VE elements of row ar + q (NT / KC) at column ak
+  const int ar = tid / KC, ak = (tid % KC) * VE;
+  const T* Ap = A + (m0 + ar) * g.lda + ak;
+  const int64_t mleft = me - m0 - ar;
+  // B slab: as rows k (VE columns) or, with TB, as rows n (VE k's)
+  const T* Bp[BC];
+  int bk[BC], bn[BC];
+  int bl[BC];   // columns left from this one on
+#pragma unroll
+  for (int q = 0; q < BC; ++q) {
+    const int e = tid + q * NT;
+    bk[q] = TB ? (e % KC) * VE : e / NC;
+    bn[q] = TB ? e / KC : (e % NC) * VE;
+    const int gn = n0 + bn[q];
+    bl[q] = g.N - gn;
+    const int z = gn / g.nb, c = gn - z * g.nb;
+    Bp[q] = B + (int64_t)z * g.sB + (TB ? (int64_t)c * g.ldb + bk[q] : (int64_t)bk[q] * g.ldb + c);
+  }
+  T ra[AC][VE], rb[BC][VE];
   T acc[TM][TN];
 #pragma unroll
   for (int i = 0; i < TM; ++i)
@@ -51,35 +117,60 @@ gemm_kernel(GemmArgs<T> g) {
 
   auto load = [&](int k0) {
 #pragma unroll
-    for (int q = 0; q < A_PER; ++q) {
-      int e = tid + q * NT;
-      int row = e / BK, col = e % BK;
-      int64_t gm = m0 + row;
-      int gk = k0 + col;
-      ra[q] = (gm < me && gk < g.K) ? A[gm * g.lda + gk] : T(0);
+    for (int q = 0; q < AC; ++q) {
+      const T* p = Ap + (int64_t)q * (NT / KC) * g.lda + k0;
+      const bool row = q * (NT / KC) < mleft;
+      if (g.va) {
+        if (row && k0 + ak < g.K) ld_vec<T, VE>(ra[q], p);
+        else
+#pragma unroll
+          for (int i = 0; i < VE; ++i) ra[q][i] = T(0);
+      } else {
+#pragma unroll
+        for (int i = 0; i < VE; ++i) ra[q][i] = (row && k0 + ak + i < g.K) ? p[i] : T(0);
+      }
     }
 #pragma unroll
-    for (int q = 0; q < B_PER; ++q) {
-      int e = tid + q * NT;
-      int gk, gn;
-      if (TB) { gn = n0 + e / BK; gk = k0 + e % BK; }
-      else { gk = k0 + e / BN; gn = n0 + e % BN; }
-      T v = T(0);
-      if (gk < g.K && gn < g.N) v = TB ? B[(int64_t)gn * g.ldb + gk] : B[(int64_t)gk * g.ldb + gn];
-      rb[q] = v;
+    for (int q = 0; q < BC; ++q) {
+      const T* p = Bp[q] + (TB ? (int64_t)k0 : (int64_t)k0 * g.ldb);
+      const bool in = TB ? bl[q] > 0 : k0 + bk[q] < g.K;
+      const int left = TB ? g.K - k0 - bk[q] : bl[q];   // elements along the load
+      if (g.vb) {
+        if (in && left > 0) ld_vec<T, VE>(rb[q], p);
+        else
+#pragma unroll
+          for (int i = 0; i < VE; ++i) rb[q][i] = T(0);
+      } else if (TB) {
+#pragma unroll
+        for (int i = 0; i < VE; ++i) rb[q][i] = (in && i < left) ? p[i] : T(0);
+      } else {
+        // columns may cross into the next block of B
+        int c = (n0 + bn[q]) % g.nb;
+#pragma unroll
+        for (int i = 0; i < VE; ++i) {
+          rb[q][i] = (in && i < left) ? *p : T(0);
+          ++p;
+          if (++c == g.nb) { c = 0; p += g.sB - g.nb; }
+        }
+      }
     }
   };
   auto store = [&](int buf) {
 #pragma unroll
-    for (int q = 0; q < A_PER; ++q) {
-      int e = tid + q * NT;
-      As[buf][e % BK][e / BK] = ra[q];
-    }
+    for (int q = 0; q < AC; ++q)
 #pragma unroll
-    for (int q = 0; q < B_PER; ++q) {
-      int e = tid + q * NT;
-      if (TB) Bs[buf][e % BK][e / BK] = rb[q];
-      else Bs[buf][e / BN][e % BN] = rb[q];
+      for (int i = 0; i < VE; ++i) As[buf][ak + i][ar + q * (NT / KC)] = ra[q][i];
+#pragma unroll
+    for (int q = 0; q < BC; ++q) {
+      if (TB) {
+#pragma unroll
+        for (int i = 0; i < VE; ++i) Bs[buf][bk[q] + i][bn[q]] = rb[q][i];
+      } else {
+        struct alignas(16) Vec { T x[VE]; } u;
+#pragma unroll
+        for (int i = 0; i < VE; ++i) u.x[i] = rb[q][i];
+        *reinterpret_cast<Vec*>(&Bs[buf][bk[q]][bn[q]]) = u;
+      }
     }
   };
 
@@ -92,15 +183,16 @@ gemm_kernel(GemmArgs<T> g) {
     if (more) load(k0 + BK);
 #pragma unroll
     for (int kk = 0; kk < BK; ++kk) {
-      T a[TM], b[TN];
+      T a[RM][GM], b[RN][GN];
 #pragma unroll
-      for (int i = 0; i < TM; ++i) a[i] = As[buf][kk][ty * TM + i];
+      for (int p = 0; p < RM; ++p) ld_vec<T, GM>(a[p], &As[buf][kk][p * (BM / RM) + ty * GM]);
 #pragma unroll
-      for (int j = 0; j < TN; ++j) b[j] = Bs[buf][kk][tx * TN + j];
+      for (int p = 0; p < RN; ++p) ld_vec<T, GN>(b[p], &Bs[buf][kk][p * (BN / RN) + tx * GN]);
 #pragma unroll
       for (int i = 0; i < TM; ++i)
 #pragma unroll
-        for (int j = 0; j < TN; ++j) acc[i][j] = fma(a[i], b[j], acc[i][j]);
+        for (int j = 0; j < TN; j += 2)
+          fma_pair(acc[i][j], acc[i][j + 1], a[i / GM][i % GM], b[j / GN][j % GN], b[j / GN][j % GN + 1]);
     }
     if (more) {
       store(buf ^ 1);
@@ -110,37 +202,92 @@ gemm_kernel(GemmArgs<T> g) {
   }
 #pragma unroll
   for (int i = 0; i < TM; ++i) {
-    int64_t gm = m0 + ty * TM + i;
-    if (gm >= me) break;
+    const int64_t gm = m0 + (i / GM) * (BM / RM) + ty * GM + i % GM;
+    if (gm >= me) continue;
 #pragma unroll
-    for (int j = 0; j < TN; ++j) {
-      int gn = n0 + tx * TN + j;
-      if (gn < g.N) {
-        T* p = C + gm * g.ldc + gn;
-        *p = g.accumulate ? (*p + acc[i][j]) : acc[i][j];
+    for (int p = 0; p < RN; ++p) {
+      const int gn = n0 + p * (BN / RN) + tx * GN;
+      T* o = C + gm * g.ldc + gn;
+      if (g.vc && gn + GN <= g.N) {
+        constexpr int W = VE < GN ? VE : GN;
+        struct alignas(W * sizeof(T)) Vec { T x[W]; };
+#pragma unroll
+        for (int q = 0; q < GN; q += W) {
+          Vec u;
+          if (g.accumulate) {
+            u = *reinterpret_cast<const Vec*>(o + q);
+#pragma unroll
+            for (int j = 0; j < W; ++j) u.x[j] = u.x[j] + acc[i][p * GN + q + j];
+          } else {
+#pragma unroll
+            for (int j = 0; j < W; ++j) u.x[j] = acc[i][p * GN + q + j];
+          }
+          *reinterpret_cast<Vec*>(o + q) = u;
+        }
+      } else {
+#pragma unroll
+        for (int j = 0; j < GN; ++j)
+          if (gn + j < g.N) o[j] = g.accumulate ? (o[j] + acc[i][p * GN + j]) : acc[i][p * GN + j];
       }
     }
   }
 }
 
+template <typename T, int BM, int BN, int BK, int TM, int TN>
+inline void gemm_launch(cudaStream_t s, const GemmArgs<T>& g, bool tb, int64_t m_cap, int batch) {
+  const dim3 grid((unsigned)((m_cap + BM - 1) / BM), (unsigned)((g.N + BN - 1) / BN), batch);
+  constexpr int NT = (BM / TM) * (BN / TN);
+  if (tb) gemm_kernel<T, BM, BN, BK, TM, TN, true><<<grid, NT, 0, s>>>(g);
+  else gemm_kernel<T, BM, BN, BK, TM, TN, false><<<grid, NT, 0, s>>>(g);
+}
+
 // Host launcher.  m_cap bounds end - begin (grid sizing).
+//
+// float32: tiles of 64 x 64 (64 threads, 8 x 8 outputs each, 168 registers)
+// reach 55-59 of the 77 TFLOP/s of plain multiply-adds once a few tiles per SM
+// exist: 400 k rows, K = N = 256 in 885 us, and N = 180 in 672 us (2200 and
+// 2064 us with one 128 x 128 tile of scalar loads and unpacked multiply-adds).
+// Larger tiles measured no faster (128 x 64: 905 us, 128 x 128 with 16 x 8
+// outputs: 1000 us).  32 x 32 tiles keep more SMs busy where there are few
+// outputs and a product is one chain of K dependent steps (128 x 256, K = 256:
+// 47 -> 9 us); 128 x 16 tiles avoid computing padding columns
+// (400 k rows, N = 16: 695 -> 138 us).
+// float64: every tile shape runs at the float64 pipe's rate (1.2 TFLOP/s), so
+// the smallest one, which pads least and spreads furthest, is the only one
+// (81920 rows, K = 64, N = 10: 578 -> 142 us; 256 rows: 70 -> 9 us).
 template <typename T>
 inline void gemm(cudaStream_t s, const T* A, int64_t lda, const T* B, int64_t ldb, bool transB,
                  T* C, int64_t ldc, int64_t m_begin, int64_t m_end, const int64_t* m_range,
                  int64_t m_cap, int N, int K, int batch = 1, int64_t sA = 0, int64_t sB = 0,
                  int64_t sC = 0, bool accumulate = false) {
   if (m_cap <= 0 || N <= 0 || K <= 0 || batch <= 0) return;
-  GemmArgs<T> g{A, B, C, lda, ldb, ldc, sA, sB, sC, m_begin, m_end, m_range, N, K, accumulate ? 1 : 0};
-  if constexpr (sizeof(T) == 4) {
-    constexpr int BM = 128, BN = 128, BK = 8;
-    dim3 grid((unsigned)((m_cap + BM - 1) / BM), (unsigned)((N + BN - 1) / BN), batch);
-    if (transB) gemm_kernel<T, BM, BN, BK, 8, 8, true><<<grid, 256, 0, s>>>(g);
-    else gemm_kernel<T, BM, BN, BK, 8, 8, false><<<grid, 256, 0, s>>>(g);
+  GemmArgs<T> g{A, B, C, lda, ldb, ldc, sA, sB, sC, m_begin, m_end, m_range, N, K, N, accumulate ? 1 : 0, 0, 0, 0};
+  if (batch > 1 && sA == 0 && sC == N) {   // side by side: one product of batch * N columns
+    g.N = N * batch;
+    batch = 1;
+  }
+  constexpr int VE = 16 / (int)sizeof(T);
+  auto al = [](const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; };
+  g.va = al(A) && lda % VE == 0 && K % VE == 0 && sA % VE == 0;
+  g.vb = al(B) && ldb % VE == 0 && sB % VE == 0 && (transB ? K : N) % VE == 0;
+  g.vc = al(C) && ldc % VE == 0 && sC % VE == 0;
+  if constexpr (sizeof(T) == 8) {
+    gemm_launch<T, 16, 16, 32, 1, 2>(s, g, transB, m_cap, batch);
   } else {
-    constexpr int BM = 64, BN = 64, BK = 8;
-    dim3 grid((unsigned)((m_cap + BM - 1) / BM), (unsigned)((N + BN - 1) / BN), batch);
-    if (transB) gemm_kernel<T, BM, BN, BK, 4, 4, true><<<grid, 256, 0, s>>>(g);
-    else gemm_kernel<T, BM, BN, BK, 4, 4, false><<<grid, 256, 0, s>>>(g);
+    // the tile of least estimated time: rounds of 152 SMs times the tile's
+    // outputs over its rate relative to the 64 x 64 tile's
+    struct Tile { int bm, bn; float eff; };
+    constexpr Tile t[] = {{64, 64, 1.f}, {32, 32, 0.38f}, {128, 16, 0.42f}};
+    int best = 0;
+    float cost = 3.4e38f;
+    for (int q = 0; q < 3; ++q) {
+      const int64_t tiles = ((m_cap + t[q].bm - 1) / t[q].bm) * ((g.N + t[q].bn - 1) / t[q].bn) * batch;
+      const float c = (float)((tiles + 151) / 152) * t[q].bm * t[q].bn / t[q].eff;
+      if (c < cost) { cost = c; best = q; }
+    }
+    if (best == 0) gemm_launch<T, 64, 64, 16, 8, 8>(s, g, transB, m_cap, batch);
+    else if (best == 1) gemm_launch<T, 32, 32, 32, 2, 4>(s, g, transB, m_cap, batch);
+    else gemm_launch<T, 128, 16, 32, 4, 4>(s, g, transB, m_cap, batch);
   }
 }
 

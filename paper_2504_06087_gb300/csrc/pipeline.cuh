@@ -994,11 +994,13 @@ struct Runner {
         // of up to 60 members; FIRE_CONTRACT=v1 keeps the 256-thread kernel
         // (diagnostic)
         const bool c2 = sizeof(T) == 4 && mcap <= kC2BigMax && !(cenv && strcmp(cenv, "v1") == 0);
-        // orbital rows of G determinants per product (BF16 form: one slice of
-        // the packed [D n][d] weights of a spin, so X is read D / G times)
-        int G = 1;
+        // orbital rows of G determinants per product: X is read D / G times.
+        // BF16 form: one slice of the packed [D n][d] weights of a spin; SIMT
+        // forms: the determinants' weights as column blocks of one product
+        // (float64, n = 10, 82 k rows: 142 -> 103 us per determinant, the
+        // 16-column tiles pad 40 columns less than 10)
         const __nv_bfloat16* WBo = wbm(3, pl.wb_orbv);
-        if (WBo && d % 64 == 0) G = (int)(pl.ld_big / n) < kOrbGroup ? (int)(pl.ld_big / n) : kOrbGroup;
+        int G = (int)(pl.ld_big / n) < kOrbGroup ? (int)(pl.ld_big / n) : kOrbGroup;
         if (G < 1) G = 1;
         for (int dd0 = 0; dd0 < D; dd0 += G) {
           const int g = D - dd0 < G ? D - dd0 : G;
@@ -1016,9 +1018,8 @@ struct Runner {
               }
             }
             if (!done)
-              for (int j = 0; j < g; ++j)
-                gemm<T>(s, X, d, p.orb_w + ((int64_t)sp * D + dd0 + j) * d * n, n, false, O + (int64_t)j * n, ldo,
-                        0, 0, rng + 2 * sp, cap, n, d);
+              gemm<T>(s, X, d, p.orb_w + ((int64_t)sp * D + dd0) * d * n, n, false, O, ldo, 0, 0, rng + 2 * sp, cap, n,
+                      d, g, 0, (int64_t)d * n, n);
           }
           if constexpr (sizeof(T) == 4) {
             if (ctc && c2 && hcount[0] > 0) {

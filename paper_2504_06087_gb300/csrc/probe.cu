@@ -1,4 +1,5 @@
-// FMA-rate probe of the SIMT pipes (float32 and float64).
+// Diagnostics of the SIMT pipes (float32 and float64): the matrix product on
+// its own, and the FMA-rate probe.
 //
 // The roofline fractions of the kernels that run on the FP32 or FP64 pipe
 // (the restricted log-det contraction, the Gauss-Jordan inverse, the float64
@@ -12,6 +13,7 @@
 #include <cuda_runtime.h>
 
 #include "../../include/fire.h"
+#include "gemm.cuh"
 
 namespace {
 
@@ -64,5 +66,21 @@ extern "C" int fire_selftest_fma_rate(int32_t dtype, int64_t iters, int32_t bloc
     fma_probe_kernel<double><<<blocks, 256, 0, s>>>((double*)out, rounds, 0.9999999, 1e-7);
   else
     fma_probe_kernel<float><<<blocks, 256, 0, s>>>((float*)out, rounds, 0.9999f, 1e-4f);
+  return cudaGetLastError() == cudaSuccess ? FIRE_OK : FIRE_ERR_CUDA;
+}
+
+extern "C" int fire_selftest_simt_gemm(int32_t dtype, int64_t M, int32_t N, int32_t K, int32_t batch, int32_t transB,
+                                       int32_t accumulate, const void* A, int64_t lda, const void* B, int64_t ldb,
+                                       int64_t sB, void* C, int64_t ldc, int64_t sC, void* stream) {
+  if ((dtype != 0 && dtype != 1) || M < 1 || N < 1 || K < 1 || batch < 1 || lda < K || ldb < (transB ? K : N) ||
+      ldc < N || sB < 0 || sC < 0 || !A || !B || !C)
+    return FIRE_ERR_INVALID_ARG;
+  cudaStream_t s = (cudaStream_t)stream;
+  if (dtype == 0)
+    fire::gemm<double>(s, (const double*)A, lda, (const double*)B, ldb, transB != 0, (double*)C, ldc, 0, M, nullptr,
+                       M, N, K, batch, 0, sB, sC, accumulate != 0);
+  else
+    fire::gemm<float>(s, (const float*)A, lda, (const float*)B, ldb, transB != 0, (float*)C, ldc, 0, M, nullptr, M, N,
+                      K, batch, 0, sB, sC, accumulate != 0);
   return cudaGetLastError() == cudaSuccess ? FIRE_OK : FIRE_ERR_CUDA;
 }
