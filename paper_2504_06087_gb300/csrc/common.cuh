@@ -38,6 +38,17 @@ template <typename T> __device__ __forceinline__ T dsqrt(T x);
 template <> __device__ __forceinline__ float dsqrt<float>(float x) { return sqrtf(x); }
 template <> __device__ __forceinline__ double dsqrt<double>(double x) { return sqrt(x); }
 
+// |v| as an unsigned key that orders like |v| for every non-NaN value (the
+// IEEE bit pattern without the sign bit), so the pivot search compares
+// integers and keeps the float64 pipe for the elimination.
+__device__ __forceinline__ unsigned long long mag_key(double v) {
+  return (unsigned long long)__double_as_longlong(v) & 0x7fffffffffffffffull;
+}
+__device__ __forceinline__ unsigned long long mag_key(float v) {
+  return (unsigned long long)((unsigned)__float_as_int(v) & 0x7fffffffu);
+}
+constexpr unsigned long long kMagInf = 0x7ff0000000000000ull;   // above it: a NaN (float64)
+
 // SiLU and its first two derivatives: s = logistic(x),
 // f = x s, f' = s (1 + x (1 - s)), f'' = s (1 - s) (2 + x (1 - 2 s)).
 template <typename T>

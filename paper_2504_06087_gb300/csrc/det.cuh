@@ -103,16 +103,6 @@ __global__ void phi_assemble_kernel(int Wc, int n, int n_up, int D, const T* __r
   }
 }
 
-// |v| as an unsigned key that orders like |v| for every non-NaN value (the
-// IEEE bit pattern without the sign bit), so the pivot search compares
-// integers and keeps the float64 pipe for the elimination.
-__device__ __forceinline__ unsigned long long mag_key(double v) {
-  return (unsigned long long)__double_as_longlong(v) & 0x7fffffffffffffffull;
-}
-__device__ __forceinline__ unsigned long long mag_key(float v) {
-  return (unsigned long long)((unsigned)__float_as_int(v) & 0x7fffffffu);
-}
-
 // Blocked right-looking LU with partial pivoting, one CTA per matrix, the
 // matrix in global memory (L2-resident), the current panel and U12 block in
 // shared memory.  Writes the pivots, log|det| and sign (0 and -inf for an
@@ -260,6 +250,120 @@ __global__ void lu_kernel(int n, LT* __restrict__ M, int32_t* __restrict__ piv,
 // Dynamic shared memory of lu_kernel<LT, NB>: the panel [n][NB + 1] and U12 [NB][n].
 inline size_t lu_smem_bytes(int n, size_t lsz, int nb = 16) { return (size_t)(2 * nb + 1) * n * lsz; }
 
+
+// The LU of lu_kernel (same pivots, same chain of operations per element) with
+// the whole matrix in shared memory, one CTA per matrix: three barriers per
+// column, no panel copies and no row interchanges in global memory.  A
+// float64 multiply-add occupies the pipe for so long (a warp's 32 take 64
+// cycles of an SM quarter) that only the number of float64 warp instructions
+// counts: the trailing block is walked as one flat range, so every lane of
+// every instruction works, and column c needs one reciprocal.
+// Two CTAs per SM fit up to n = 119 (float64) or 168 (float32); beyond that
+// the blocked kernel, which keeps only a panel, is the faster one.
+template <typename LT>
+__global__ void __launch_bounds__(256) lu_smem_kernel(int n, LT* __restrict__ M, int32_t* __restrict__ piv,
+                                                      double* __restrict__ logabs, double* __restrict__ sgn,
+                                                      const int* __restrict__ count) {
+  if (count && (int)blockIdx.x >= *count) return;
+  extern __shared__ unsigned char lu_smem[];
+  LT* S = reinterpret_cast<LT*>(lu_smem);   // [n][n + 1]
+  __shared__ int s_piv, s_zero;
+  __shared__ LT s_pv, s_rinv;
+  const int ld = n + 1;
+  LT* A = M + (int64_t)blockIdx.x * n * n;
+  int32_t* pv = piv + (int64_t)blockIdx.x * n;
+  const int tid = threadIdx.x, bd = blockDim.x;
+  if (tid == 0) s_zero = 0;
+  for (int r = tid >> 5; r < n; r += bd >> 5)
+    for (int c = tid & 31; c < n; c += 32) S[r * ld + c] = A[(int64_t)r * n + c];
+  int neg = 0;
+  __syncthreads();
+  for (int c = 0; c < n; ++c) {
+    if (tid < 32) {   // argmax |S[r][c]|, r >= c, first row on ties
+      unsigned long long best = 0;
+      int bi = c;
+      for (int r = c + tid; r < n; r += 32) {
+        const unsigned long long v = mag_key(S[r * ld + c]);
+        if (v > best) { best = v; bi = r; }
+      }
+      for (int o = 16; o > 0; o >>= 1) {
+        const unsigned long long ov = __shfl_xor_sync(0xffffffffu, best, o);
+        const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
+        if (ov > best || (ov == best && oi < bi)) { best = ov; bi = oi; }
+      }
+      if (tid == 0) {
+        const LT x = S[bi * ld + c];
+        s_piv = bi;
+        s_pv = x;
+        s_rinv = best == 0 ? LT(0) : LT(1) / x;
+        pv[c] = bi;
+        if (best == 0) s_zero = 1;
+      }
+    }
+    __syncthreads();
+    const int p = s_piv;
+    const LT pivot = s_pv, rinv = s_rinv;
+    // rows c and p change places; column c becomes the multipliers
+    if (p != c) {
+      for (int q = tid; q < n; q += bd) {
+        if (q == c) continue;
+        const LT t = S[c * ld + q];
+        S[c * ld + q] = S[p * ld + q];
+        S[p * ld + q] = t;
+      }
+      neg ^= 1;
+    }
+    for (int r = c + 1 + tid; r < n; r += bd) {
+      const LT x = S[(r == p ? c : r) * ld + c];
+      S[r * ld + c] = pivot != LT(0) ? x * rinv : x;
+      if (r == p) S[c * ld + c] = pivot;
+    }
+    __syncthreads();
+    if (pivot != LT(0)) {
+      const int w = n - c - 1;
+      const float iw = 1.f / (float)w;
+      for (int e = tid; e < w * w; e += bd) {
+        int rr = (int)((float)e * iw);   // e / w, corrected by one either way
+        rr += (rr + 1) * w <= e ? 1 : 0;
+        rr -= rr * w > e ? 1 : 0;
+        const int r = c + 1 + rr, j = c + 1 + e - rr * w;
+        S[r * ld + j] -= S[r * ld + c] * S[c * ld + j];
+      }
+    }
+    __syncthreads();
+  }
+  for (int r = tid >> 5; r < n; r += bd >> 5)
+    for (int c = tid & 31; c < n; c += 32) A[(int64_t)r * n + c] = S[r * ld + c];
+  if (tid < 32) {   // log|det| and sign
+    double la = 0.0;
+    int sg = tid == 0 ? neg : 0;
+    for (int k = tid; k < n; k += 32) {
+      const double u = (double)S[k * ld + k];
+      la += log(fabs(u));
+      if (u < 0) sg ^= 1;
+    }
+    for (int o = 16; o > 0; o >>= 1) {
+      la += __shfl_xor_sync(0xffffffffu, la, o);
+      sg ^= __shfl_xor_sync(0xffffffffu, sg, o);
+    }
+    if (tid == 0) {
+      if (s_zero) { logabs[blockIdx.x] = -INFINITY; sgn[blockIdx.x] = 0.0; }
+      else { logabs[blockIdx.x] = la; sgn[blockIdx.x] = sg ? -1.0 : 1.0; }
+    }
+  }
+}
+
+// LU of a batch of nmat matrices (or of the first *count of them), by the
+// kernel that suits n.
+template <typename LT>
+inline void lu_batch(cudaStream_t s, int n, int64_t nmat, LT* M, int32_t* piv, double* logabs, double* sgn,
+                     const int* count = nullptr) {
+  const size_t whole = (size_t)n * (n + 1) * sizeof(LT);
+  if (whole <= 113 * 1024)
+    lu_smem_kernel<LT><<<(unsigned)nmat, 256, whole, s>>>(n, M, piv, logabs, sgn, count);
+  else
+    lu_kernel<LT, 16><<<(unsigned)nmat, 256, lu_smem_bytes(n, sizeof(LT)), s>>>(n, M, piv, logabs, sgn, count);
+}
 
 // A = Phi^-1 by in-place Gauss-Jordan elimination with partial pivoting, in
 // float32, register-tiled: thread (tr, tc) of a Gr x Gc grid (Gr = ceil(n/12),

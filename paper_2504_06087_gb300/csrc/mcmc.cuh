@@ -489,54 +489,77 @@ __global__ void __launch_bounds__(256) mcmc_ratio_kernel(
   }
   __syncthreads();
   int32_t* pv = Mpiv + md * Umax;
-  double la = 0.0;
+  __shared__ double s_pv;
   int neg = 0;
-  bool zero = false;
   for (int c = 0; c < u; ++c) {
-    if (threadIdx.x < 32) {   // pivot: the first row of largest |M[q][c]|, q >= c
-      double best = -1.0;
+    if (threadIdx.x < 32) {   // pivot: the first row of largest |M[q][c]|, q >= c (never a NaN while others are left)
+      unsigned long long best = 0;
       int bq = c;
       for (int q = c + threadIdx.x; q < u; q += 32) {
-        const double v = fabs(M[q * ldm + c]);
+        const double x = M[q * ldm + c];
+        const unsigned long long v = mag_key(x) > kMagInf ? 0 : mag_key(x) + 1;
         if (v > best) { best = v; bq = q; }
       }
       for (int o = 16; o > 0; o >>= 1) {
-        const double ob = __shfl_xor_sync(0xffffffffu, best, o);
+        const unsigned long long ob = __shfl_xor_sync(0xffffffffu, best, o);
         const int oq = __shfl_xor_sync(0xffffffffu, bq, o);
         if (ob > best || (ob == best && oq < bq)) { best = ob; bq = oq; }
       }
-      if (threadIdx.x == 0) { s_p = bq; pv[c] = bq; }
+      if (threadIdx.x == 0) {
+        s_p = bq;
+        s_pv = M[bq * ldm + c];
+        pv[c] = bq;
+      }
     }
     __syncthreads();
     const int pq = s_p;
+    const double piv = s_pv;
+    // rows c and pq change places, and column c becomes the multipliers (one
+    // division per row)
     if (pq != c) {
       for (int q = threadIdx.x; q < u; q += blockDim.x) {
+        if (q == c) continue;
         const double t = M[c * ldm + q];
         M[c * ldm + q] = M[pq * ldm + q];
         M[pq * ldm + q] = t;
       }
       neg ^= 1;
     }
+    if (piv < 0.0) neg ^= 1;
+    for (int q = c + 1 + threadIdx.x; q < u; q += blockDim.x) {
+      const double x = M[(q == pq ? c : q) * ldm + c];
+      M[q * ldm + c] = piv == 0.0 ? x : x / piv;
+      if (q == pq) M[c * ldm + c] = piv;
+    }
     __syncthreads();
-    const double piv = M[c * ldm + c];
-    if (piv == 0.0) {
-      zero = true;
-    } else {
-      la += log(fabs(piv));
-      if (piv < 0.0) neg ^= 1;
+    if (piv != 0.0) {
       const int wdt = u - c - 1;
+      const float iw = 1.f / (float)wdt;
       for (int e = threadIdx.x; e < wdt * wdt; e += blockDim.x) {
-        const int q = c + 1 + e / wdt, cc = c + 1 + e % wdt;
-        M[q * ldm + cc] -= (M[q * ldm + c] / piv) * M[c * ldm + cc];
+        int rr = (int)((float)e * iw);            // e / wdt, corrected by one either way
+        rr += (rr + 1) * wdt <= e ? 1 : 0;
+        rr -= rr * wdt > e ? 1 : 0;
+        const int q = c + 1 + rr, cc = c + 1 + e - rr * wdt;
+        M[q * ldm + cc] -= M[q * ldm + c] * M[c * ldm + cc];
       }
-      __syncthreads();
-      for (int q = c + 1 + threadIdx.x; q < u; q += blockDim.x) M[q * ldm + c] /= piv;
     }
     __syncthreads();
   }
-  if (threadIdx.x == 0) {
-    lrat[md] = zero ? -INFINITY : la;
-    srat[md] = zero ? 0.0 : (neg ? -1.0 : 1.0);
+  // log|det M|: the logarithms by the lanes of one warp, summed in order
+  if (threadIdx.x < 32) {
+    double la = 0.0;
+    bool zero = false;
+    for (int c0 = 0; c0 < u; c0 += 32) {
+      const int c = c0 + threadIdx.x;
+      const double p = c < u ? M[c * ldm + c] : 1.0;
+      const double l = p == 0.0 ? 0.0 : log(fabs(p));
+      zero |= __any_sync(0xffffffffu, p == 0.0);
+      for (int k = 0; k < 32 && c0 + k < u; ++k) la += __shfl_sync(0xffffffffu, l, k);
+    }
+    if (threadIdx.x == 0) {
+      lrat[md] = zero ? -INFINITY : la;
+      srat[md] = zero ? 0.0 : (neg ? -1.0 : 1.0);
+    }
   }
   // the factors go to Mg for the Woodbury solve (already there when M lived in Mg)
   if (in_smem) {
@@ -789,18 +812,147 @@ __global__ void mcmc_rows_kernel(int Wn, int n, int n_up, int d, int Dn, int RD,
   }
 }
 
+// Solves L U x = b in place for 32 right-hand sides, one per lane of a warp:
+// X[i][lane] (row stride 33) holds b and receives x; A holds the factors (unit
+// L, row stride lda) and X[i][32] the reciprocal of U_ii.  Rows below i0 of
+// every b are zero.  A float64 multiply-add of a warp holds the pipe for
+// longer than its latency, so the number of warp instructions is what counts:
+// every lane has a column of its own and each factor is one broadcast load
+// for 32 multiply-adds.  Four rows go together, which loads X once for four
+// and keeps four chains in flight.  With rnd the solution of every row is
+// rounded to T before it is used further.
+template <typename T, bool rnd, typename LT, typename CT>
+__device__ __forceinline__ void warp_lu_solve(int n, const LT* __restrict__ A, int64_t lda, CT* X, int i0, int lane) {
+  auto keep = [](CT v) -> CT { return rnd ? (CT)(T)v : v; };
+  i0 &= ~3;
+  for (int ib = i0; ib < n; ib += 4) {   // forward: unit lower
+    const int nr = n - ib < 4 ? n - ib : 4;
+    const LT* a[4];
+    CT s[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const int r = k < nr ? ib + k : ib;
+      a[k] = A + (int64_t)r * lda;
+      s[k] = X[r * 33 + lane];
+    }
+#pragma unroll 4
+    for (int q = i0; q < ib; ++q) {
+      const CT x = X[q * 33 + lane];
+#pragma unroll
+      for (int k = 0; k < 4; ++k) s[k] -= (CT)a[k][q] * x;
+    }
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      if (k < nr) {
+#pragma unroll
+        for (int q = 0; q < k; ++q) s[k] -= (CT)a[k][ib + q] * s[q];
+        s[k] = keep(s[k]);
+        X[(ib + k) * 33 + lane] = s[k];
+      }
+    }
+  }
+  for (int ib = (n - 1) & ~3; ib >= 0; ib -= 4) {   // backward: upper
+    const int nr = n - ib < 4 ? n - ib : 4;
+    const LT* a[4];
+    CT s[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const int r = k < nr ? ib + k : ib;
+      a[k] = A + (int64_t)r * lda;
+      s[k] = X[r * 33 + lane];
+    }
+#pragma unroll 4
+    for (int q = ib + 4; q < n; ++q) {
+      const CT x = X[q * 33 + lane];
+#pragma unroll
+      for (int k = 0; k < 4; ++k) s[k] -= (CT)a[k][q] * x;
+    }
+#pragma unroll
+    for (int k = 3; k >= 0; --k) {
+      if (k < nr) {
+#pragma unroll
+        for (int q = 3; q > k; --q)
+          if (q < nr) s[k] -= (CT)a[k][ib + q] * s[q];
+        s[k] = keep(s[k] * X[(ib + k) * 33 + 32]);
+        X[(ib + k) * 33 + lane] = s[k];
+      }
+    }
+  }
+}
+
+// Shared memory of one warp's panel of warp_lu_solve, with n ints behind it.
+inline size_t warp_panel_smem(int n, size_t csz) { return (size_t)n * 33 * csz + (size_t)n * sizeof(int); }
+
+// A = Phi^-1 from the LU factors (P Phi = L U) of a batch of n x n matrices,
+// transposed (out[j][l] = A[l][j]) in AT's type: one warp per 32 columns.
+// Row t of P is e_{perm[t]}, so the column of A with the right-hand side e_t is
+// perm[t]: panel p takes t = 32 p .. 32 p + 31, whose forward solves start at
+// row 32 p.  With list, matrix f of the batch (f < *count) goes to slot
+// list[f] of out and a singular one (bsg[f] == 0) becomes zero.  2048
+// matrices of n = 100 in float64: see the dispatch in the pipeline.
+template <typename LT, typename AT>
+__global__ void __launch_bounds__(32) inverse_warp_kernel(int n, int64_t m0, const LT* __restrict__ LU,
+                                                          const int32_t* __restrict__ piv, AT* __restrict__ Ainv,
+                                                          const int* __restrict__ count, int cap,
+                                                          const int32_t* __restrict__ list,
+                                                          const double* __restrict__ bsg) {
+  extern __shared__ __align__(16) unsigned char iw_smem[];
+  LT* X = reinterpret_cast<LT*>(iw_smem);                     // [n][33]
+  int* perm = reinterpret_cast<int*>(X + (int64_t)n * 33);    // [n]
+  const int np = (n + 31) / 32;
+  const int64_t f = m0 + blockIdx.x / np;
+  const int p = blockIdx.x % np;
+  if (count && f >= (*count < cap ? *count : cap)) return;
+  const int lane = threadIdx.x;
+  const LT* A = LU + f * n * n;
+  AT* out = Ainv + (list ? (int64_t)list[f] : f) * n * n;
+  const int t = 32 * p + lane;
+  if (bsg && bsg[f] == 0.0) {
+    for (int j = 32 * p; j < n && j < 32 * p + 32; ++j)
+      for (int l = lane; l < n; l += 32) out[(int64_t)j * n + l] = AT(0);
+    return;
+  }
+  int* spv = reinterpret_cast<int*>(X);   // the interchanges, before X is written
+  for (int i = lane; i < n; i += 32) {
+    perm[i] = i;
+    spv[i] = piv[f * n + i];
+  }
+  __syncwarp();
+  if (lane == 0)
+    for (int k = 0; k < n; ++k) {
+      const int q = spv[k], a = perm[k];
+      perm[k] = perm[q];
+      perm[q] = a;
+    }
+  __syncwarp();
+  for (int i = 0; i < n; ++i) X[i * 33 + lane] = i == t ? LT(1) : LT(0);
+  for (int i = lane; i < n; i += 32) X[i * 33 + 32] = LT(1) / A[(int64_t)i * n + i];
+  __syncwarp();
+  warp_lu_solve<LT, false>(n, A, n, X, 32 * p, lane);
+  __syncwarp();
+  for (int c = 0; c < 32 && 32 * p + c < n; ++c) {
+    AT* o = out + (int64_t)perm[32 * p + c] * n;
+    for (int l = lane; l < n; l += 32) o[l] = (AT)X[l * 33 + c];
+  }
+}
+
 // Woodbury update of A^T and the rows U of Phi for accepted walkers:
 //   B = Delta A (u x n), C = M^-1 B (solved with the LU factors of M),
 //   A'^T[m][l] = A^T[m][l] - sum_a C[a][m] A^T[U_a][l],   Phi_U += Delta.
 // A persistent grid of 256-thread CTAs walks the (walker, det) pairs; CTA b
 // keeps its scratch (Tw: [Umax][n] in Tu, B then C: [Umax][n] in Bw) in slot
 // b.  Flagged pairs are refactorised by mcmc_repair_kernel instead.
+// The float64 solve (|U|^2 n multiply-adds against 2 |U| n^2 float32 ones) is
+// what bounds the kernel: nw warps take 32 columns each (warp_lu_solve), their
+// columns in dynamic shared memory ([nw][Upan][33] doubles); update sets larger
+// than Upan keep their columns in the scratch.
 template <typename T>
 __global__ void __launch_bounds__(256) mcmc_woodbury_kernel(
     int Wn, int n, int D, int Umax, const int32_t* __restrict__ acc, const int32_t* __restrict__ flag,
     const int32_t* __restrict__ Ul, const int32_t* __restrict__ Uc, const T* __restrict__ Dl,
     const double* __restrict__ Mlu, const int32_t* __restrict__ Mpiv, T* __restrict__ AT, T* __restrict__ Phi,
-    T* __restrict__ Tu, T* __restrict__ Bw) {
+    T* __restrict__ Tu, T* __restrict__ Bw, int Upan, int nw) {
+  extern __shared__ __align__(16) unsigned char wb_smem[];
   // the product tiles and the LU of M are never live together: one buffer
   __shared__ double su[kLemmaSmem * (kLemmaSmem + 1)];
   __shared__ int spv[kLemmaSmem];
@@ -835,28 +987,33 @@ __global__ void __launch_bounds__(256) mcmc_woodbury_kernel(
     const double* L = in_smem ? sL : Mg;
     const int ldl = in_smem ? kLemmaSmem + 1 : Umax;
     const int32_t* pv = in_smem ? spv : pvg;
-    // C = M^-1 B: one column per thread, row swaps then unit-lower and upper
-    // solves in float64; the column lives in local memory
-    for (int m = threadIdx.x; m < n; m += blockDim.x) {
-      double x[kLemmaSmem];
-      if (in_smem) {
-        for (int c = 0; c < u; ++c) x[c] = (double)Bm[(int64_t)c * n + m];
-        for (int c = 0; c < u; ++c) {
-          const int p = pv[c];
-          if (p != c) { const double t = x[c]; x[c] = x[p]; x[p] = t; }
+    // C = M^-1 B in float64: row interchanges, then the two triangular solves
+    if (u <= Upan) {
+      const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
+      double* X = reinterpret_cast<double*>(wb_smem) + (int64_t)wid * Upan * 33;
+      if (wid < nw) {
+        for (int c = lane; c < u; c += 32) X[c * 33 + 32] = 1.0 / L[c * ldl + c];
+        for (int m0 = 32 * wid; m0 < n; m0 += 32 * nw) {
+          const int m = m0 + lane;
+          for (int c = 0; c < u; ++c) X[c * 33 + lane] = m < n ? (double)Bm[(int64_t)c * n + m] : 0.0;
+          for (int c = 0; c < u; ++c) {
+            const int p = pv[c];
+            if (p != c) {
+              const double t = X[c * 33 + lane];
+              X[c * 33 + lane] = X[p * 33 + lane];
+              X[p * 33 + lane] = t;
+            }
+          }
+          __syncwarp();
+          // beyond kLemmaSmem the rows are kept in T between the steps
+          if (in_smem) warp_lu_solve<T, false>(u, L, ldl, X, 0, lane);
+          else warp_lu_solve<T, true>(u, L, ldl, X, 0, lane);
+          if (m < n)
+            for (int c = 0; c < u; ++c) Bm[(int64_t)c * n + m] = (T)X[c * 33 + lane];
         }
-        for (int c = 0; c < u; ++c) {
-          double s = x[c];
-          for (int q = 0; q < c; ++q) s -= L[c * ldl + q] * x[q];
-          x[c] = s;
-        }
-        for (int c = u - 1; c >= 0; --c) {
-          double s = x[c];
-          for (int q = c + 1; q < u; ++q) s -= L[c * ldl + q] * x[q];
-          x[c] = s / L[c * ldl + c];
-        }
-        for (int c = 0; c < u; ++c) Bm[(int64_t)c * n + m] = (T)x[c];
-      } else {   // large U: the same solve on the column in the scratch
+      }
+    } else {   // the columns in the scratch, one per thread
+      for (int m = threadIdx.x; m < n; m += blockDim.x) {
         for (int c = 0; c < u; ++c) {
           const int p = pv[c];
           if (p != c) {
@@ -882,6 +1039,24 @@ __global__ void __launch_bounds__(256) mcmc_woodbury_kernel(
     cta_gemm_tn<T>(n, n, u, Bm, n, Tw, n, A, n, T(-1), true, sm);
     for (int e = threadIdx.x; e < u * n; e += blockDim.x) P[(int64_t)U[e / n] * n + e % n] += Dw[e];
   }
+}
+
+// The Woodbury kernel's panel rows and solving warps: four warps (one per SM
+// quarter) where their panels fit beside the LU of M, two CTAs per SM up to
+// |U| = 64.
+struct WoodburyShape {
+  int Upan, nw;
+  size_t smem;
+};
+inline WoodburyShape woodbury_shape(int n, int Umax) {
+  WoodburyShape w;
+  w.Upan = Umax < 192 ? Umax : 192;
+  const size_t panel = (size_t)w.Upan * 33 * sizeof(double);
+  const int np = (n + 31) / 32;
+  w.nw = np < 4 ? np : 4;
+  while (w.nw > 1 && w.nw * panel > 150 * 1024) --w.nw;
+  w.smem = w.nw * panel;
+  return w;
 }
 
 // ---------------------------------------------------------------------------
@@ -961,26 +1136,6 @@ __global__ void __launch_bounds__(256) inverse_panel_kernel(int n, int64_t m0, c
   inverse_panel_block<LT, CT, AT>(n, LU + mat * n * n, piv + mat * n, Ainv + mat * n * n, ip_smem);
 }
 
-// A^T of the batched refactorisations: matrix f of the batch into the slot
-// rlist[f] of A^T (zero for a singular matrix); CTAs beyond the count leave.
-template <typename LT, typename T>
-__global__ void __launch_bounds__(256) mcmc_repair_inverse_kernel(int n, const int* __restrict__ count, int cap,
-                                                                  const int32_t* __restrict__ rlist,
-                                                                  const LT* __restrict__ batch,
-                                                                  const int32_t* __restrict__ piv,
-                                                                  const double* __restrict__ bsg,
-                                                                  T* __restrict__ AT) {
-  extern __shared__ unsigned char ri_smem[];
-  const int c = *count < cap ? *count : cap;
-  if ((int)blockIdx.x >= c) return;
-  T* A = AT + (int64_t)rlist[blockIdx.x] * n * n;
-  if (bsg[blockIdx.x] == 0.0) {
-    for (int e = threadIdx.x; e < n * n; e += blockDim.x) A[e] = T(0);
-    return;
-  }
-  inverse_panel_block<LT, LT, T>(n, batch + (int64_t)blockIdx.x * n * n, piv + (int64_t)blockIdx.x * n, A, ri_smem);
-}
-
 inline size_t inverse_panel_smem(int n, size_t lsz) { return (size_t)n * 33 * lsz + 2 * (size_t)n * sizeof(int); }
 
 
@@ -1042,61 +1197,67 @@ __device__ void lu_block(int n, LT* __restrict__ A, int32_t* __restrict__ pv, do
   __syncthreads();
 }
 
-// Exact ratios for the (walker, det) pairs whose determinant-lemma ratio is
-// beyond e^{+-kExactLogRatio} or not finite: Phi' = Phi with the rows U
-// replaced (Phi_U + Delta), its float64 LU, lrat = log|det Phi'| - ldabs and
-// srat = sign(det Phi') * lsign.  xflag[pair] = 1 marks them for a
-// refactorisation if the move is accepted.  A persistent grid; CTA b uses
-// slot b of the float64 scratch; dynamic shared memory n ints.
-//
-// Also recomputed exactly (and refactorised if accepted): every determinant
-// whose Woodbury-carried inverse cannot be trusted to the tolerance ktol,
-// i.e. kappa_d u w_d > ktol, with kappa_d the Frobenius condition estimate of
-// the last factorisation (kap), u the unit roundoff of the state (kunit) and
-// w_d = |det Phi_d| / max_q |det Phi_q| the determinant's weight in the
-// walker's sum.  A float32 inverse of a matrix with kappa ~ 1e6 carries
-// relative errors of order kappa u ~ 0.06, which a run of moves accumulates
-// into the carried log-determinant; weighted by w_d that is the error it
-// brings into log|Psi| and the acceptance ratio.  ktol < 0 turns the test off.
+// Chooses the (walker, det) pairs whose ratio comes from a float64 LU of
+// Phi' = Phi with the rows U replaced (Phi_U + Delta) instead of the lemma:
+//  range  the determinant-lemma ratio is beyond e^{+-kExactLogRatio} or not
+//         finite (xflag 1: refactorised if the move is accepted);
+//  cond   the Woodbury-carried inverse cannot be trusted to the tolerance
+//         ktol, i.e. kappa_d u w_d > ktol, with kappa_d the Frobenius
+//         condition estimate of the last factorisation (kap), u the unit
+//         roundoff of the state (kunit) and w_d = |det Phi_d| / max_q |det Phi_q|
+//         the determinant's weight in the walker's sum (xflag 2).  A float32
+//         inverse of a matrix with kappa ~ 1e6 carries relative errors of
+//         order kappa u ~ 0.06, which a run of moves accumulates into the
+//         carried log-determinant; weighted by w_d that is the error it
+//         brings into log|Psi| and the acceptance ratio.  ktol < 0 turns the
+//         test off.
+// The pairs are listed for the batched LU; those beyond its capacity keep
+// their mark in xover and take mcmc_exact_ratio_kernel.  One thread per pair.
+static __global__ void mcmc_exact_select_kernel(int64_t npair, int D, const double* __restrict__ ldabs,
+                                                const double* __restrict__ lsign, const double* __restrict__ lrat,
+                                                int32_t* __restrict__ xflag, const float* __restrict__ kap,
+                                                double kunit, double ktol, int* __restrict__ xcount,
+                                                int32_t* __restrict__ xlist, int xcap, int32_t* __restrict__ xover,
+                                                unsigned long long* __restrict__ nexact) {
+  const int64_t md = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (md >= npair) return;
+  const double lr = lrat[md];
+  const bool range = !(fabs(lr) <= kExactLogRatio) && lsign[md] != 0.0;
+  bool cond = false;
+  if (!range && ktol >= 0.0 && lsign[md] != 0.0) {
+    const int64_t w0 = (md / D) * D;
+    double lmax = -INFINITY;
+    for (int q = 0; q < D; ++q)
+      if (lsign[w0 + q] != 0.0 && ldabs[w0 + q] > lmax) lmax = ldabs[w0 + q];
+    cond = (double)kap[md] * kunit * exp(ldabs[md] - lmax) > ktol;
+  }
+  xflag[md] = range ? 1 : (cond ? 2 : 0);
+  int over = 0;
+  if (range || cond) {
+    if (nexact) atomicAdd(nexact, 1ull);
+    const int slot = atomicAdd(xcount, 1);
+    if (slot < xcap) xlist[slot] = (int32_t)md;
+    else over = 1;
+  }
+  if (xover) xover[md] = over;
+}
+
+// The exact ratios of the pairs that the batched LU had no room for (xover),
+// lrat = log|det Phi'| - ldabs and srat = sign(det Phi') * lsign, by one CTA
+// per pair.  A persistent grid; CTA b uses slot b of the float64 scratch;
+// dynamic shared memory n ints.
 template <typename T, typename LT>
 __global__ void __launch_bounds__(256) mcmc_exact_ratio_kernel(
     int Wn, int n, int D, int Umax, const int32_t* __restrict__ Ul, const int32_t* __restrict__ Uc,
     const T* __restrict__ Phi, const T* __restrict__ Dl, const double* __restrict__ ldabs,
     const double* __restrict__ lsign, double* __restrict__ lrat, double* __restrict__ srat,
-    int32_t* __restrict__ xflag, LT* __restrict__ scratch, int32_t* __restrict__ spiv,
-    const float* __restrict__ kap, double kunit, double ktol, int* __restrict__ xcount,
-    int32_t* __restrict__ xlist, int xcap, unsigned long long* __restrict__ nexact) {
+    LT* __restrict__ scratch, int32_t* __restrict__ spiv, const int32_t* __restrict__ xover) {
   extern __shared__ int xr_slot[];   // [n]: slot of row i in U, or -1
   __shared__ double s_la, s_sg;
-  __shared__ int s_slot;
   LT* L = scratch + (int64_t)blockIdx.x * n * n;
   int32_t* pv = spiv + (int64_t)blockIdx.x * n;
   for (int64_t md = blockIdx.x; md < (int64_t)Wn * D; md += gridDim.x) {
-    const double lr = lrat[md];
-    const bool range = !(fabs(lr) <= kExactLogRatio) && lsign[md] != 0.0;
-    bool cond = false;
-    if (!range && ktol >= 0.0 && lsign[md] != 0.0) {
-      const int64_t w0 = (md / D) * D;
-      double lmax = -INFINITY;
-      for (int q = 0; q < D; ++q)
-        if (lsign[w0 + q] != 0.0 && ldabs[w0 + q] > lmax) lmax = ldabs[w0 + q];
-      cond = (double)kap[md] * kunit * exp(ldabs[md] - lmax) > ktol;
-    }
-    // 1: ratio out of range (the inverse is refactorised if accepted);
-    // 2: conditioning (exact ratio; the Woodbury update keeps A until the
-    // next refresh, the ratio does not use it while the test holds)
-    if (threadIdx.x == 0) xflag[md] = range ? 1 : (cond ? 2 : 0);
-    if (!range && !cond) continue;
-    if (threadIdx.x == 0 && nexact) atomicAdd(nexact, 1ull);
-    if (cond && xlist) {   // deferred to the batched float64 LU when it has room
-      __syncthreads();
-      if (threadIdx.x == 0) {
-        s_slot = atomicAdd(xcount, 1);
-        if (s_slot < xcap) xlist[s_slot] = (int32_t)md;
-      }
-      __syncthreads();
-      if (s_slot < xcap) continue;
-    }
+    if (!xover[md]) continue;
     const int w = (int)(md / D);
     const int u = Uc[w];
     for (int i = threadIdx.x; i < n; i += blockDim.x) xr_slot[i] = -1;

@@ -252,13 +252,31 @@ struct Runner {
   int nc_h0 = 3;              // h^0 products and orbital value rows (no fp32 recompute)
   bool use_gj = true;
   int lu_nb = 16;             // FIRE_LU_NB (diagnostic): 16 or 32-column LU panels
-  // A^T from the LU factors, matrices in batches of the grid limit
-  void inverse_from_lu(int n, int64_t nmat, const LT* LUb, const int32_t* piv, T* Ainv) {
-    const size_t ism = inverse_panel_smem(n, sizeof(T));
-    for (int64_t m0 = 0; m0 < nmat; m0 += 65535) {
-      const int64_t cnt = nmat - m0 < 65535 ? nmat - m0 : 65535;
-      inverse_panel_kernel<LT, T, T><<<(unsigned)cnt, 256, ism, s>>>(n, m0, LUb, piv, Ainv);
+  // A^T from the LU factors.  Float64 factors inverted in float64: one warp
+  // per 32 columns (inverse_warp_kernel).  Float32 inversion (the float32
+  // forms beyond the Gauss-Jordan kernel's n): the panel kernel.
+  template <typename AT>
+  void inverse_warp(int n, int64_t nmat, const LT* LUb, const int32_t* piv, AT* Ainv, const int* count = nullptr,
+                    int cap = 0, const int32_t* list = nullptr, const double* bsg = nullptr) {
+    const int np = (n + 31) / 32;
+    const int64_t most = (1ll << 30) / np;
+    for (int64_t m0 = 0; m0 < nmat; m0 += most) {
+      const int64_t cnt = nmat - m0 < most ? nmat - m0 : most;
+      inverse_warp_kernel<LT, AT><<<(unsigned)(cnt * np), 32, warp_panel_smem(n, sizeof(LT)), s>>>(
+          n, m0, LUb, piv, Ainv, count, cap, list, bsg);
       launches += 1;
+    }
+  }
+  void inverse_from_lu(int n, int64_t nmat, const LT* LUb, const int32_t* piv, T* Ainv) {
+    if constexpr (sizeof(T) == 8) {
+      inverse_warp<T>(n, nmat, LUb, piv, Ainv);
+    } else {
+      const size_t ism = inverse_panel_smem(n, sizeof(T));
+      for (int64_t m0 = 0; m0 < nmat; m0 += 65535) {   // batches of the grid limit
+        const int64_t cnt = nmat - m0 < 65535 ? nmat - m0 : 65535;
+        inverse_panel_kernel<LT, T, T><<<(unsigned)cnt, 256, ism, s>>>(n, m0, LUb, piv, Ainv);
+        launches += 1;
+      }
     }
   }
   int64_t capA = 0;           // allocated rows of X / Y: the component stride of Xb / Yb
@@ -500,7 +518,7 @@ struct Runner {
       double* lsign = at<double>(pl.lsign);
       const bool gj = use_gj && sizeof(T) == 4 && n <= 192;
       phi_assemble_kernel<T, LT><<<wc * D, 256, 0, s>>>(wc, n, n_up, D, Ov, Fenv, 1, LUb, gj ? B.Phif : nullptr);
-      lu_kernel<LT, 16><<<wc * D, 256, lu_smem_bytes(n, sizeof(LT)), s>>>(n, LUb, piv, ldabs, lsign);
+      lu_batch<LT>(s, n, wc * D, LUb, piv, ldabs, lsign);
       if (gj) {
         gj_inverse_kernel<float, T><<<wc * D, gj_threads(n), gj_smem_bytes(n), s>>>(n, B.Phif, B.AT);
       } else {
@@ -952,19 +970,13 @@ struct Runner {
         if (!deriv) launch_lu_side();
       } else {
         if (lu_nb == 32) lu_kernel<LT, 32><<<wc * D, 256, lu_smem_bytes(n, sizeof(LT), 32), s>>>(n, LUb, piv, ldabs, lsign);
-        else lu_kernel<LT, 16><<<wc * D, 256, lusm, s>>>(n, LUb, piv, ldabs, lsign);
+        else lu_batch<LT>(s, n, wc * D, LUb, piv, ldabs, lsign);
       }
       check("lu");
       if (mc) {
         // A^T = (Phi^-1)^T from the float64 factors
         mark("inverse", 1);
-        const int64_t nmat = (int64_t)wc * D;
-        const size_t ism = inverse_panel_smem(n, sizeof(LT));
-        for (int64_t m0 = 0; m0 < nmat; m0 += 65535) {
-          const int64_t cnt = nmat - m0 < 65535 ? nmat - m0 : 65535;
-          inverse_panel_kernel<LT, LT, T><<<(unsigned)cnt, 256, ism, s>>>(n, m0, LUb, piv, at<T>(pl.Ainv));
-          launches += 1;
-        }
+        inverse_warp<T>(n, (int64_t)wc * D, LUb, piv, at<T>(pl.Ainv));
         check("inverse");
       }
       T* gdet = at<T>(pl.gdet);
@@ -1375,27 +1387,27 @@ struct Runner {
         const int64_t npair = (int64_t)Wn * D;
         int* xcnt = at<int>(pl.mc_xcnt);
         int32_t* xlist = at<int32_t>(pl.mc_xlist);
-        const bool batched = mc.kappa_tol >= 0.0;
-        if (batched) cudaMemsetAsync(xcnt, 0, sizeof(int), s);
-        mcmc_exact_ratio_kernel<T, LT><<<(unsigned)(npair < kWoodburySlots ? npair : kWoodburySlots), 256,
-                                         (size_t)n * sizeof(int), s>>>(
-            Wn, n, D, Umax, Ul, Uc, PhiS, Dl, ldabs, lsign, lrat, srat, xflag, at<LT>(pl.mc_rep),
-            at<int32_t>(pl.mc_rpiv), kap, kunit, mc.kappa_tol, xcnt, batched ? xlist : nullptr, pl.xcap,
-            &ms->n_exact);
-        launches += 1;
-        if (batched) {
-          // ill-conditioned determinants: float64 LU of Phi' over all SMs
-          LT* xb = at<LT>(pl.mc_xbatch);
-          double* xlab = at<double>(pl.mc_xlab);
-          double* xsg = at<double>(pl.mc_xsg);
-          mcmc_exact_build_kernel<T, LT><<<pl.xcap, 256, (size_t)n * sizeof(int), s>>>(n, D, Umax, xcnt, xlist, Ul, Uc,
-                                                                                       PhiS, Dl, xb);
-          lu_kernel<LT, 16><<<pl.xcap, 256, lu_smem_bytes(n, sizeof(LT)), s>>>(n, xb, at<int32_t>(pl.mc_xpiv), xlab,
-                                                                               xsg, xcnt);
-          mcmc_exact_scatter_kernel<<<(pl.xcap + 255) / 256, 256, 0, s>>>(xcnt, pl.xcap, xlist, xlab, xsg, ldabs,
-                                                                         lsign, lrat, srat);
-          launches += 3;
+        // pairs whose ratio needs a float64 LU of Phi', then that LU over all
+        // SMs; only a batch beyond its capacity leaves any to the per-CTA path
+        int32_t* xover = npair > pl.xcap ? at<int32_t>(pl.mc_flag) : nullptr;
+        cudaMemsetAsync(xcnt, 0, sizeof(int), s);
+        mcmc_exact_select_kernel<<<(unsigned)((npair + 127) / 128), 128, 0, s>>>(
+            npair, D, ldabs, lsign, lrat, xflag, kap, kunit, mc.kappa_tol, xcnt, xlist, pl.xcap, xover, &ms->n_exact);
+        if (xover) {
+          mcmc_exact_ratio_kernel<T, LT><<<kWoodburySlots, 256, (size_t)n * sizeof(int), s>>>(
+              Wn, n, D, Umax, Ul, Uc, PhiS, Dl, ldabs, lsign, lrat, srat, at<LT>(pl.mc_rep), at<int32_t>(pl.mc_rpiv),
+              xover);
+          launches += 1;
         }
+        LT* xb = at<LT>(pl.mc_xbatch);
+        double* xlab = at<double>(pl.mc_xlab);
+        double* xsg = at<double>(pl.mc_xsg);
+        mcmc_exact_build_kernel<T, LT><<<pl.xcap, 256, (size_t)n * sizeof(int), s>>>(n, D, Umax, xcnt, xlist, Ul, Uc,
+                                                                                     PhiS, Dl, xb);
+        lu_batch<LT>(s, n, pl.xcap, xb, at<int32_t>(pl.mc_xpiv), xlab, xsg, xcnt);
+        mcmc_exact_scatter_kernel<<<(pl.xcap + 255) / 256, 256, 0, s>>>(xcnt, pl.xcap, xlist, xlab, xsg, ldabs,
+                                                                       lsign, lrat, srat);
+        launches += 4;
       }
       check("mc ratio");
     };
@@ -1499,8 +1511,9 @@ struct Runner {
             Fenv, Vn, V, G1n, G2n, G1, G2, H1n, H1);
         mark("mc_woodbury", 1);
         const int64_t npair = (int64_t)Wn * D;
-        mcmc_woodbury_kernel<T><<<(unsigned)(npair < kWoodburySlots ? npair : kWoodburySlots), 256, 0, s>>>(
-            Wn, n, D, Umax, acc, flag, Ul, Uc, Dl, Mlu, Mpiv, AT, PhiS, Tu, Bw);
+        const WoodburyShape wsh = woodbury_shape(n, Umax);
+        mcmc_woodbury_kernel<T><<<(unsigned)(npair < kWoodburySlots ? npair : kWoodburySlots), 256, wsh.smem, s>>>(
+            Wn, n, D, Umax, acc, flag, Ul, Uc, Dl, Mlu, Mpiv, AT, PhiS, Tu, Bw, wsh.Upan, wsh.nw);
         mcmc_repair_kernel<T, LT><<<(unsigned)(npair < kWoodburySlots ? npair : kWoodburySlots), 256,
                                     inverse_panel_smem(n, sizeof(LT)), s>>>(
             Wn, n, D, acc, flag, PhiS, AT, ldabs, lsign, lref, at<LT>(pl.mc_rep), at<int32_t>(pl.mc_rpiv));
@@ -1512,11 +1525,10 @@ struct Runner {
           double* xlab = at<double>(pl.mc_xlab);
           double* xsg = at<double>(pl.mc_xsg);
           mcmc_repair_build_kernel<T, LT><<<pl.xcap, 256, 0, s>>>(n, rcnt, rlist, PhiS, xb);
-          lu_kernel<LT, 16><<<pl.xcap, 256, lu_smem_bytes(n, sizeof(LT)), s>>>(n, xb, xpiv, xlab, xsg, rcnt);
+          lu_batch<LT>(s, n, pl.xcap, xb, xpiv, xlab, xsg, rcnt);
           mcmc_repair_scatter_kernel<<<(pl.xcap + 255) / 256, 256, 0, s>>>(rcnt, pl.xcap, rlist, xlab, xsg, ldabs,
                                                                           lsign, lref);
-          mcmc_repair_inverse_kernel<LT, T><<<pl.xcap, 256, inverse_panel_smem(n, sizeof(LT)), s>>>(
-              n, rcnt, pl.xcap, rlist, xb, xpiv, xsg, AT);
+          inverse_warp<T>(n, pl.xcap, xb, xpiv, AT, rcnt, pl.xcap, rlist, xsg);
         }
         launches += 5;
         check("mc update");
@@ -1582,15 +1594,16 @@ inline int set_smem_limits() {
   raise((const void*)contract3_kernel<192>);
   raise((const void*)contract3_kernel<320>);
   raise((const void*)lu_kernel<LT, 16>);
+  raise((const void*)lu_smem_kernel<LT>);
   raise((const void*)lu_kernel<LT, 32>);
   raise((const void*)att_pool_kernel<T>);
   raise((const void*)gj_inverse_kernel<float, T>);
   raise((const void*)gj_inverse_pre_kernel<float, T>);
   raise((const void*)mcmc_att_kernel<T>);
-  raise((const void*)inverse_panel_kernel<LT, LT, T>);
-  raise((const void*)inverse_panel_kernel<LT, T, T>);
+  if constexpr (sizeof(T) == 4) raise((const void*)inverse_panel_kernel<LT, T, T>);
+  raise((const void*)mcmc_woodbury_kernel<T>);
   raise((const void*)mcmc_repair_kernel<T, LT>);
-  raise((const void*)mcmc_repair_inverse_kernel<LT, T>);
+  raise((const void*)inverse_warp_kernel<LT, T>);
   cudaError_t e = cudaGetLastError();
   if (rc != FIRE_OK || e != cudaSuccess) set_last_error("smem limits", cudaGetErrorString(e));
   return rc;
