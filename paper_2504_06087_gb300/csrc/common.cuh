@@ -49,6 +49,19 @@ __device__ __forceinline__ unsigned long long mag_key(float v) {
 }
 constexpr unsigned long long kMagInf = 0x7ff0000000000000ull;   // above it: a NaN (float64)
 
+// VN consecutive elements, aligned to 16 bytes (or to their whole size).
+template <typename T, int VN>
+__device__ __forceinline__ void ld_vec(T (&v)[VN], const T* p) {
+  constexpr int W = 16 / (int)sizeof(T) < VN ? 16 / (int)sizeof(T) : VN;
+  struct alignas(W * sizeof(T)) Vec { T x[W]; };
+#pragma unroll
+  for (int q = 0; q < VN; q += W) {
+    const Vec u = *reinterpret_cast<const Vec*>(p + q);
+#pragma unroll
+    for (int i = 0; i < W; ++i) v[q + i] = u.x[i];
+  }
+}
+
 // SiLU and its first two derivatives: s = logistic(x),
 // f = x s, f' = s (1 + x (1 - s)), f'' = s (1 - s) (2 + x (1 - 2 s)).
 template <typename T>

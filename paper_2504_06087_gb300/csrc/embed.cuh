@@ -60,14 +60,67 @@ __device__ __forceinline__ FL3<T> pair_feature(int k, const T dv[3], T r, const 
 constexpr int kPairBatch = 16;
 // Largest nucleus count of the batched electron-nucleus filter.
 constexpr int kMaxNuc = 512;
+// Widest CTA (one thread per column) whose registers the filter kernels have
+// to fit: 128 a thread in float32, 255 in float64.
+template <typename T>
+constexpr int kFilterThreads = sizeof(T) == 4 ? 512 : 256;
+// Filter features of a pair, hidden units first, then Gaussians, then e-bar.
+constexpr int kPairFeat = kEdgeHidden + kGauss + 4;
+
+// Features of one pair in shared memory.  NC = 1: the values, so a thread
+// reads four features with one 128-bit broadcast.  NC = 5: value, Laplacian
+// and three tangents of a feature side by side (an array per component, read
+// four features at a time, measured 2-6 % slower: the sums issue as many
+// multiply-adds, and the loads are not what bounds them).
+template <typename T, int NC>
+struct alignas(16) PairFeat {
+  T f[kPairFeat][NC];
+};
+template <int NC, typename T>
+__device__ __forceinline__ void put_feature(PairFeat<T, NC>& o, int k, const FL3<T>& v) {
+  o.f[k][0] = v.v;
+  if constexpr (NC == 5) {
+    o.f[k][1] = v.l;
+#pragma unroll
+    for (int t = 0; t < 3; ++t) o.f[k][2 + t] = v.t[t];
+  }
+}
+// acc[c] += sum_k f[k][c] w[k] over COUNT features from k0 on, in order.
+template <int COUNT, int NC, typename T>
+__device__ __forceinline__ void feat_dot(const PairFeat<T, NC>& q, int k0, const T* w, T (&acc)[NC]) {
+  if constexpr (NC == 1) {
+#pragma unroll
+    for (int k = 0; k < COUNT; k += 4) {
+      T v[4];
+      ld_vec<T, 4>(v, &q.f[k0 + k][0]);
+#pragma unroll
+      for (int i = 0; i < 4; ++i) acc[0] += v[i] * w[k + i];
+    }
+  } else {
+#pragma unroll
+    for (int k = 0; k < COUNT; ++k)
+#pragma unroll
+      for (int c = 0; c < NC; ++c) acc[c] += q.f[k0 + k][c] * w[k];
+  }
+}
+template <typename T>
+__device__ __forceinline__ FL3<T> as_fl3(const T (&a)[5]) {
+  FL3<T> o;
+  o.v = a[0];
+  o.l = a[1];
+#pragma unroll
+  for (int t = 0; t < 3; ++t) o.t[t] = a[2 + t];
+  return o;
+}
 
 // One CTA per electron (w, i), blockDim == d.  Writes the filter sum
-// s_i = sum_m Gamma_m * (h^nuc_m + e-bar W) as R5 rows of S.
-template <typename T, typename W>
-__global__ void en_filter_kernel(int Wc, int n, int n_up, int N, int d, const double* __restrict__ r,
+// s_i = sum_m Gamma_m * (h^nuc_m + e-bar W) as R5 rows of S (NC = 5 components
+// for R5 = 5, the value alone for R5 = 1).
+template <typename T, typename W, int NC>
+__global__ void __launch_bounds__(kFilterThreads<T>) en_filter_kernel(int Wc, int n, int n_up, int N, int d, const double* __restrict__ r,
                                  const double* __restrict__ R, double cnuc, Params<W> p,
-                                 T* __restrict__ S, int R5) {
-  constexpr int H = kEdgeHidden, G = kGauss;
+                                 T* __restrict__ S) {
+  constexpr int H = kEdgeHidden, G = kGauss, R5 = NC;
   const int blk = blockIdx.x;
   const int w = blk / n, i = blk % n;
   const int c = threadIdx.x;
@@ -83,7 +136,7 @@ __global__ void en_filter_kernel(int Wc, int n, int n_up, int N, int d, const do
   acc.t[0] = acc.t[1] = acc.t[2] = T(0);
   const double* ri = r + ((int64_t)w * n + i) * 3;
   // nuclei within c_n (Gamma_m vanishes identically beyond), ascending
-  __shared__ FL3<T> featb[kPairBatch][H + G + 4];
+  __shared__ PairFeat<T, NC> featb[kPairBatch];
   __shared__ T s_dv[kPairBatch][3], s_r[kPairBatch];
   __shared__ int s_m[kPairBatch];
   __shared__ int s_list[kMaxNuc];
@@ -118,58 +171,39 @@ __global__ void en_filter_kernel(int Wc, int n, int n_up, int N, int d, const do
       s_m[threadIdx.x] = m;
     }
     __syncthreads();
-    for (int e = threadIdx.x; e < nbat * (H + G + 4); e += blockDim.x) {
-      const int q = e / (H + G + 4), k = e - q * (H + G + 4);
+    for (int e = threadIdx.x; e < nbat * kPairFeat; e += blockDim.x) {
+      const int q = e / kPairFeat, k = e - q * kPairFeat;
       const int m = s_m[q];
-      featb[q][k] = pair_feature<T, W>(k, s_dv[q], s_r[q], p.en_w1 + (int64_t)m * 4 * H, p.en_b1 + (int64_t)m * H,
-                                       p.en_sigma, T(cnuc));
+      put_feature<NC, T>(featb[q], k,
+                         pair_feature<T, W>(k, s_dv[q], s_r[q], p.en_w1 + (int64_t)m * 4 * H,
+                                            p.en_b1 + (int64_t)m * H, p.en_sigma, T(cnuc)));
     }
     __syncthreads();
     for (int q = 0; q < nbat; ++q) {
       const int m = s_m[q];
-      const FL3<T>* feat = featb[q];
-    FL3<T> gv, ev, fv;
-    gv.v = gv.l = ev.v = ev.l = T(0);
-    fv.v = T(p.nuc_emb[(int64_t)m * d + c]);
-    fv.l = T(0);
+      T gv[NC], ev[NC], fv[NC];
 #pragma unroll
-    for (int t = 0; t < 3; ++t) gv.t[t] = ev.t[t] = fv.t[t] = T(0);
+      for (int t = 0; t < NC; ++t) gv[t] = ev[t] = fv[t] = T(0);
+      fv[0] = T(p.nuc_emb[(int64_t)m * d + c]);
+      feat_dot<H, NC, T>(featb[q], 0, w2, gv);
+      feat_dot<G, NC, T>(featb[q], H, we, ev);
+      feat_dot<4, NC, T>(featb[q], H + G, wf, fv);
+      if constexpr (NC == 5) {
+        FL3<T> gam, term;
+        fl3_mul(as_fl3(gv), as_fl3(ev), gam);
+        fl3_mul(gam, as_fl3(fv), term);
+        acc.v += term.v;
+        acc.l += term.l;
 #pragma unroll
-    for (int h = 0; h < H; ++h) {
-      const FL3<T> a = feat[h];
-      gv.v += a.v * w2[h];
-      gv.l += a.l * w2[h];
-#pragma unroll
-      for (int t = 0; t < 3; ++t) gv.t[t] += a.t[t] * w2[h];
-    }
-#pragma unroll
-    for (int g = 0; g < G; ++g) {
-      const FL3<T> a = feat[H + g];
-      ev.v += a.v * we[g];
-      ev.l += a.l * we[g];
-#pragma unroll
-      for (int t = 0; t < 3; ++t) ev.t[t] += a.t[t] * we[g];
-    }
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      const FL3<T> a = feat[H + G + k];
-      fv.v += a.v * wf[k];
-      fv.l += a.l * wf[k];
-#pragma unroll
-      for (int t = 0; t < 3; ++t) fv.t[t] += a.t[t] * wf[k];
-    }
-    FL3<T> gam, term;
-    fl3_mul(gv, ev, gam);
-    fl3_mul(gam, fv, term);
-    acc.v += term.v;
-    acc.l += term.l;
-#pragma unroll
-    for (int t = 0; t < 3; ++t) acc.t[t] += term.t[t];
+        for (int t = 0; t < 3; ++t) acc.t[t] += term.t[t];
+      } else {
+        acc.v += (gv[0] * ev[0]) * fv[0];
+      }
     }
   }
   const int64_t row = (int64_t)block_index(w, i, Wc, n, n_up) * R5;
   S[row * d + c] = acc.v;
-  if (R5 > 1) {
+  if constexpr (NC == 5) {
     S[(row + 1) * d + c] = acc.l;
 #pragma unroll
     for (int t = 0; t < 3; ++t) S[(row + 2 + t) * d + c] = acc.t[t];
@@ -293,13 +327,16 @@ __global__ void split_rows_kernel(int64_t rows, int ncol, const T* __restrict__ 
 // Message passing step.  One CTA per electron (w, i), blockDim == d.
 // H0 [Wc*n*R5][d]; PQ [Wc*n*R5][4d] = [h0 W^par_a | h0 W^anti_a | h0 W^par_b |
 // h0 W^anti_b]; X receives the block of h^1_i (value, Laplacian, tangents).
-template <typename T, typename W>
-__global__ void msg_kernel(int Wc, int n, int n_up, int d, int K, const double* __restrict__ r,
+// With NC = 5 the blocks are value, Laplacian and tangents; with NC = 1 the
+// value row alone.
+template <typename T, typename W, int NC>
+__global__ void __launch_bounds__(kFilterThreads<T>) msg_kernel(int Wc, int n, int n_up, int d, int K, const double* __restrict__ r,
                            double cut, Params<W> p, const int32_t* __restrict__ idx,
                            const int32_t* __restrict__ cnt, const int64_t* __restrict__ blk_off,
                            const T* __restrict__ H0, const T* __restrict__ PQ, T* __restrict__ X,
-                           __nv_bfloat16* __restrict__ Xb, int xnc, int64_t xcs, int deriv) {
+                           __nv_bfloat16* __restrict__ Xb, int xnc, int64_t xcs) {
   constexpr int H = kEdgeHidden, G = kGauss;
+  constexpr bool deriv = NC == 5;
   const int blk = blockIdx.x;
   const int w = blk / n, i = blk % n;
   const int c = threadIdx.x;
@@ -339,7 +376,7 @@ __global__ void msg_kernel(int Wc, int n, int n_up, int d, int K, const double* 
   const int cpar = cnt[((int64_t)w * n + i) * 2], ctot = cpar + cnt[((int64_t)w * n + i) * 2 + 1];
   const double* rw = r + (int64_t)w * n * 3;
   const int32_t* li = idx + ((int64_t)w * n + i) * K;
-  __shared__ FL3<T> featb[kPairBatch][H + G + 4];
+  __shared__ PairFeat<T, NC> featb[kPairBatch];
   __shared__ T s_dv[kPairBatch][3], s_r[kPairBatch];
   for (int b0 = 0; b0 < ctot; b0 += kPairBatch) {
     const int nbat = min(kPairBatch, ctot - b0);
@@ -353,56 +390,39 @@ __global__ void msg_kernel(int Wc, int n, int n_up, int d, int K, const double* 
       s_r[threadIdx.x] = T(sqrt(dd[0] * dd[0] + dd[1] * dd[1] + dd[2] * dd[2]));
     }
     __syncthreads();
-    for (int e = threadIdx.x; e < nbat * (H + G + 4); e += blockDim.x) {
-      const int q = e / (H + G + 4), k = e - q * (H + G + 4);
-      featb[q][k] = pair_feature<T, W>(k, s_dv[q], s_r[q], p.ee_w1, p.ee_b1, p.ee_sigma, T(cut));
+    for (int e = threadIdx.x; e < nbat * kPairFeat; e += blockDim.x) {
+      const int q = e / kPairFeat, k = e - q * kPairFeat;
+      put_feature<NC, T>(featb[q], k, pair_feature<T, W>(k, s_dv[q], s_r[q], p.ee_w1, p.ee_b1, p.ee_sigma, T(cut)));
     }
     __syncthreads();
   for (int s = b0; s < b0 + nbat; ++s) {
     const int j = li[s];
     const int a = (s < cpar) ? 0 : 1;
-    const FL3<T>* feat = featb[s - b0];
+    const PairFeat<T, NC>& feat = featb[s - b0];
     // Gamma(e_ij) in delta-space (delta = r_i - r_j)
-    FL3<T> gv, ev, gam;
-    gv.v = gv.l = ev.v = ev.l = T(0);
+    T gc[NC], ec[NC], bc[NC];
 #pragma unroll
-    for (int t = 0; t < 3; ++t) gv.t[t] = ev.t[t] = T(0);
-#pragma unroll
-    for (int h = 0; h < H; ++h) {
-      const FL3<T> q = feat[h];
-      gv.v += q.v * w2[h];
-      gv.l += q.l * w2[h];
-#pragma unroll
-      for (int t = 0; t < 3; ++t) gv.t[t] += q.t[t] * w2[h];
-    }
-#pragma unroll
-    for (int g = 0; g < G; ++g) {
-      const FL3<T> q = feat[H + g];
-      ev.v += q.v * we[g];
-      ev.l += q.l * we[g];
-#pragma unroll
-      for (int t = 0; t < 3; ++t) ev.t[t] += q.t[t] * we[g];
-    }
-    fl3_mul(gv, ev, gam);
+    for (int t = 0; t < NC; ++t) gc[t] = ec[t] = bc[t] = T(0);
+    feat_dot<H, NC, T>(feat, 0, w2, gc);
+    feat_dot<G, NC, T>(feat, H, we, ec);
+    FL3<T> gam;
+    if constexpr (deriv) fl3_mul(as_fl3(gc), as_fl3(ec), gam);
+    else gam.v = gc[0] * ec[0];
     // z = P_i + Q_j + e-bar_ij W_c + b ; tangents in r_i and r_j
     const int bj = block_index(w, j, Wc, n, n_up);
     const int64_t prow = hrow, qrow = (int64_t)bj * R5;
     const int64_t pcol = (int64_t)a * d + c, qcol = 2 * (int64_t)d + (int64_t)a * d + c;
-    T ebv = T(0), ebt[3] = {T(0), T(0), T(0)}, ebl = T(0);
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      const FL3<T> q = feat[H + G + k];
-      ebv += q.v * wc[a][k];
-      ebl += q.l * wc[a][k];
-#pragma unroll
-      for (int t = 0; t < 3; ++t) ebt[t] += q.t[t] * wc[a][k];
-    }
+    if (a) feat_dot<4, NC, T>(feat, H + G, wc[1], bc);
+    else feat_dot<4, NC, T>(feat, H + G, wc[0], bc);
+    const T ebv = bc[0];
     T zv = (a ? pv[1] : pv[0]) + PQ[qrow * ld4 + qcol] + ebv + bb[a];
     T f, f1, f2;
     silu3<T>(zv, f, f1, f2);
     const T mv = gam.v * f;
     acc.v += mv;
-    if (deriv) {
+    if constexpr (deriv) {
+      const T ebl = bc[1];
+      const T ebt[3] = {bc[2], bc[3], bc[4]};
       T zi[3], zj[3], sq = T(0);
 #pragma unroll
       for (int t = 0; t < 3; ++t) {

@@ -45,19 +45,6 @@ __device__ __forceinline__ void fma_pair(double& c0, double& c1, double a, doubl
   c1 = fma(a, b1, c1);
 }
 
-// VN consecutive elements, aligned to their size.
-template <typename T, int VN>
-__device__ __forceinline__ void ld_vec(T (&v)[VN], const T* p) {
-  constexpr int W = 16 / (int)sizeof(T) < VN ? 16 / (int)sizeof(T) : VN;
-  struct alignas(W * sizeof(T)) Vec { T x[W]; };
-#pragma unroll
-  for (int q = 0; q < VN; q += W) {
-    const Vec u = *reinterpret_cast<const Vec*>(p + q);
-#pragma unroll
-    for (int i = 0; i < W; ++i) v[q + i] = u.x[i];
-  }
-}
-
 // One BM x BN tile per CTA; a thread owns TM x TN outputs as groups of at most
 // four consecutive rows and columns, so a warp's shared loads are 128-bit
 // broadcasts without bank conflicts.  The next BK-deep slab is in registers

@@ -18,6 +18,7 @@
 #pragma once
 
 #include "common.cuh"
+#include "embed.cuh"
 #include "philox.cuh"
 
 namespace fire {
@@ -295,118 +296,210 @@ static __global__ void __launch_bounds__(1024) mcmc_scan_kernel(int W, int Umax,
   }
 }
 
+// Message terms (value only) of the update set of a move or a swap,
+//   Gamma(delta) SiLU(P_i^a + Q_j^a + e-bar W_c^a + b^a),
+// by CTAs of d threads, one column each.  A CTA's weights (58 a thread) and the
+// two barriers of a batch of filter features serve up to 32 pairs at a time:
+// with a CTA per member, which has two to four terms, loading the weights and
+// computing derivatives of features nobody reads took most of the time
+// (C14H16, 128 walkers: see mcmc_msg_kernel).
+constexpr int kMsgPairs = 32;
+
+// Columns c of the message weights.
+template <typename T, typename W>
+struct MsgWeights {
+  T w2[kEdgeHidden], we[kGauss], wc[2][4], bb[2];
+  __device__ __forceinline__ MsgWeights(const Params<W>& p, int d, int c) {
+#pragma unroll
+    for (int h = 0; h < kEdgeHidden; ++h) w2[h] = T(p.ee_w2[h * d + c]);
+#pragma unroll
+    for (int g = 0; g < kGauss; ++g) we[g] = T(p.ee_wenv[g * d + c]);
+#pragma unroll
+    for (int a = 0; a < 2; ++a) {
+      bb[a] = T(p.msg_b[a * d + c]);
+#pragma unroll
+      for (int q = 0; q < 4; ++q) wc[a][q] = T(p.msg_w[((int64_t)a * (2 * d + 4) + 2 * d + q) * d + c]);
+    }
+  }
+  // filter value and SiLU factor of one pair
+  __device__ __forceinline__ void term(const PairFeat<T, 1>& feat, const T* Pi, const T* Qj, int a, int d, int c,
+                                       T& gam, T& f) const {
+    T gv[1] = {T(0)}, ev[1] = {T(0)}, eb[1] = {T(0)};
+    feat_dot<kEdgeHidden, 1, T>(feat, 0, w2, gv);
+    feat_dot<kGauss, 1, T>(feat, kEdgeHidden, we, ev);
+    if (a) feat_dot<4, 1, T>(feat, kEdgeHidden + kGauss, wc[1], eb);
+    else feat_dot<4, 1, T>(feat, kEdgeHidden + kGauss, wc[0], eb);
+    const T z = Pi[(int64_t)a * d + c] + Qj[2 * (int64_t)d + (int64_t)a * d + c] + eb[0] + (a ? bb[1] : bb[0]);
+    T f1, f2;
+    silu3<T>(z, f, f1, f2);
+    gam = gv[0] * ev[0];
+  }
+};
+
+// A batch of pairs of one CTA: pair vectors and distances, the row of Q of the
+// partner (< 0: no such pair), the spin channel, and the filter features.
+template <typename T>
+struct MsgBatch {
+  PairFeat<T, 1> feat[kMsgPairs];
+  T dv[kMsgPairs][3], r[kMsgPairs];
+  const T* Q[kMsgPairs];
+  int ch[kMsgPairs];
+  __device__ __forceinline__ void put(int s, const double dd[3], const T* q, int a) {
+    dv[s][0] = T(dd[0]);
+    dv[s][1] = T(dd[1]);
+    dv[s][2] = T(dd[2]);
+    r[s] = T(sqrt(dd[0] * dd[0] + dd[1] * dd[1] + dd[2] * dd[2]));
+    Q[s] = q;
+    ch[s] = a;
+  }
+  // between two barriers of the caller
+  template <typename W>
+  __device__ __forceinline__ void features(int cnt, const Params<W>& p, double cut) {
+    for (int e = threadIdx.x; e < cnt * kPairFeat; e += blockDim.x) {
+      const int q = e / kPairFeat, k = e - q * kPairFeat;
+      if (Q[q]) feat[q].f[k][0] = pair_feature<T, W>(k, dv[q], r[q], p.ee_w1, p.ee_b1, p.ee_sigma, T(cut)).v;
+    }
+  }
+};
+
+// Neighbours of electron i at the positions pos(j, t): same spin ascending,
+// then the opposite spin; cnt[0] of the same spin, cnt[1] in all.  One warp.
+template <typename Pos>
+__device__ __forceinline__ void warp_neighbours(int n, int n_up, int i, double cut, const Pos& pos, int* nbr,
+                                                int* cnt) {
+  const int lane = threadIdx.x;
+  const bool up = i < n_up;
+  int cntN = 0;
+  for (int pass = 0; pass < 2; ++pass) {
+    const bool same = pass == 0;
+    const int lo = (up == same) ? 0 : n_up, hi = (up == same) ? n_up : n;
+    for (int j0 = lo; j0 < hi; j0 += 32) {
+      const int j = j0 + lane;
+      bool in = false;
+      if (j < hi && j != i) {
+        double a2 = 0.0;
+        for (int t = 0; t < 3; ++t) {
+          const double dd = pos(i, t) - pos(j, t);
+          a2 += dd * dd;
+        }
+        in = a2 <= cut * cut;
+      }
+      const unsigned m = __ballot_sync(0xffffffffu, in);
+      if (in) nbr[cntN + __popc(m & ((1u << lane) - 1u))] = j;
+      cntN += __popc(m);
+    }
+    if (lane == 0) cnt[pass] = cntN;
+  }
+}
+
+// The moved electron i: every term, over its neighbours at the new positions
+// (nbr, cnt built), with the projections Pi and those of qrow(j).
+template <typename T, typename W, typename Pos, typename Row>
+__device__ __forceinline__ T msg_of_moved(const MsgWeights<T, W>& mw, MsgBatch<T>& B, const Params<W>& p, int i, int d,
+                                          double cut, const Pos& pos, const Row& qrow, const T* Pi, const int* nbr,
+                                          const int* cnt, T acc) {
+  const int c = threadIdx.x, cpar = cnt[0], ctot = cnt[1];
+  for (int b0 = 0; b0 < ctot; b0 += kMsgPairs) {
+    const int nb = min(kMsgPairs, ctot - b0);
+    __syncthreads();   // the previous batch is consumed
+    if (c < nb) {
+      const int j = nbr[b0 + c];
+      const double dd[3] = {pos(i, 0) - pos(j, 0), pos(i, 1) - pos(j, 1), pos(i, 2) - pos(j, 2)};
+      B.put(c, dd, qrow(j), b0 + c < cpar ? 0 : 1);
+    }
+    __syncthreads();
+    B.features(nb, p, cut);
+    __syncthreads();
+    for (int s = 0; s < nb; ++s) {
+      T gam, f;
+      mw.term(B.feat[s], Pi, B.Q[s], B.ch[s], d, c, gam, f);
+      acc += gam * f;
+    }
+  }
+  return acc;
+}
+
 // h^1 of every member i of U under the proposed positions (value only),
 //   h^1_i = h^0_i + sum_{j in N_i} Gamma(e_ij) SiLU(h^0_i W^a + h^0_j W^a' + e-bar_ij W^a_c + b^a).
 // For i = k every term changes: the neighbour list is rebuilt on the fly
 // (same spin ascending, then the opposite spin) with h^0 and projections of
 // k from h0k / PQk.  For i != k only the term of the pair (i, k) changes:
 // h^1_i = cached h^1_i - [old (i, k) term] + [new (i, k) term], each present
-// when that distance is within c.  One CTA per (walker, slot), blockDim == d;
-// dynamic shared memory n ints.  Writes h^1 to X (overwritten by the MLP) and
-// to H1n (kept for the cache).
+// when that distance is within c.  CTA 0 of a walker takes electron k, the
+// others 16 members each; blockDim == d, dynamic shared memory n ints.
+// Writes h^1 to X (overwritten by the MLP) and to H1n (kept for the cache).
+// 128 walkers of C14H16: 272 -> 50 us a move.
 template <typename T, typename W>
-__global__ void mcmc_msg_kernel(int Wn, int n, int n_up, int d, int k, int Umax, const double* __restrict__ r,
-                                const double* __restrict__ rk, double cut, Params<W> p,
-                                const int32_t* __restrict__ Ul, const int32_t* __restrict__ Uc,
-                                const int32_t* __restrict__ Urow, const T* __restrict__ H0,
-                                const T* __restrict__ PQ, const T* __restrict__ H1, const T* __restrict__ h0k,
-                                const T* __restrict__ PQk, T* __restrict__ X, T* __restrict__ H1n) {
-  constexpr int H = kEdgeHidden, G = kGauss;
-  __shared__ FL3<T> feat[H + G + 4];
+__global__ void __launch_bounds__(kFilterThreads<T>) mcmc_msg_kernel(
+    int Wn, int n, int n_up, int d, int k, int Umax, const double* __restrict__ r, const double* __restrict__ rk,
+    double cut, Params<W> p, const int32_t* __restrict__ Ul, const int32_t* __restrict__ Uc,
+    const int32_t* __restrict__ Urow, const T* __restrict__ H0, const T* __restrict__ PQ, const T* __restrict__ H1,
+    const T* __restrict__ h0k, const T* __restrict__ PQk, T* __restrict__ X, T* __restrict__ H1n) {
+  constexpr int GM = kMsgPairs / 2;   // members of a CTA: two terms each
+  __shared__ MsgBatch<T> B;
   extern __shared__ int mm_nbr[];
-  __shared__ int s_cnt[2];
-  const int w = blockIdx.x / Umax, u = blockIdx.x % Umax;
-  if (u >= Uc[w]) return;
-  const int i = Ul[(int64_t)w * Umax + u];
+  __shared__ int s_cnt[2], s_u;
+  const int groups = 1 + (Umax + GM - 1) / GM;
+  const int w = blockIdx.x / groups, g = blockIdx.x % groups;
+  const int uc = Uc[w], u0 = (g - 1) * GM;
+  if (uc == 0 || (g > 0 && u0 >= uc)) return;
   const int c = threadIdx.x;
   const int64_t ld4 = 4 * (int64_t)d;
   const double* rw = r + (int64_t)w * n * 3;
   const double* rkw = rk + (int64_t)w * 3;
-  T w2[H], we[G], wc[2][4], bb[2];
-#pragma unroll
-  for (int h = 0; h < H; ++h) w2[h] = T(p.ee_w2[h * d + c]);
-#pragma unroll
-  for (int g = 0; g < G; ++g) we[g] = T(p.ee_wenv[g * d + c]);
-#pragma unroll
-  for (int a = 0; a < 2; ++a) {
-    bb[a] = T(p.msg_b[a * d + c]);
-#pragma unroll
-    for (int q = 0; q < 4; ++q) wc[a][q] = T(p.msg_w[((int64_t)a * (2 * d + 4) + 2 * d + q) * d + c]);
-  }
-  // one message term: Gamma(delta) SiLU(Pi^a + Qj^a + e-bar W_c^a + b^a)
-  auto term = [&](const double ddv[3], const T* Pi, const T* Qj, int a) -> T {
-    const double rr = sqrt(ddv[0] * ddv[0] + ddv[1] * ddv[1] + ddv[2] * ddv[2]);
-    T dv[3] = {T(ddv[0]), T(ddv[1]), T(ddv[2])};
-    __syncthreads();
-    pair_features_to_smem<T, W>(dv, T(rr), p.ee_w1, p.ee_b1, p.ee_sigma, T(cut), feat);
-    __syncthreads();
-    T gv = T(0), ev = T(0), eb = T(0);
-#pragma unroll
-    for (int h = 0; h < H; ++h) gv += feat[h].v * w2[h];
-#pragma unroll
-    for (int g = 0; g < G; ++g) ev += feat[H + g].v * we[g];
-#pragma unroll
-    for (int q = 0; q < 4; ++q) eb += feat[H + G + q].v * wc[a][q];
-    const T z = Pi[(int64_t)a * d + c] + Qj[2 * (int64_t)d + (int64_t)a * d + c] + eb + bb[a];
-    T f, f1, f2;
-    silu3<T>(z, f, f1, f2);
-    return (gv * ev) * f;
-  };
-  T acc;
-  if (i == k) {
+  const int32_t* U = Ul + (int64_t)w * Umax;
+  const int32_t* rows = Urow + (int64_t)w * Umax;
+  const MsgWeights<T, W> mw(p, d, c);
+  if (g == 0) {
     auto pos = [&](int j, int t) -> double { return j == k ? rkw[t] : rw[3 * j + t]; };
-    if (threadIdx.x < 32) {
-      const int lane = threadIdx.x;
-      const bool up = i < n_up;
-      int cntN = 0;
-      for (int pass = 0; pass < 2; ++pass) {
-        const bool same = pass == 0;
-        const int lo = (up == same) ? 0 : n_up, hi = (up == same) ? n_up : n;
-        for (int j0 = lo; j0 < hi; j0 += 32) {
-          const int j = j0 + lane;
-          bool in = false;
-          if (j < hi && j != i) {
-            double a2 = 0.0;
-            for (int t = 0; t < 3; ++t) {
-              const double dd = pos(i, t) - pos(j, t);
-              a2 += dd * dd;
-            }
-            in = a2 <= cut * cut;
-          }
-          const unsigned m = __ballot_sync(0xffffffffu, in);
-          if (in) mm_nbr[cntN + __popc(m & ((1u << lane) - 1u))] = j;
-          cntN += __popc(m);
-        }
-        if (lane == 0) s_cnt[pass] = cntN;
-      }
-    }
+    auto qrow = [&](int j) { return PQ + (int64_t)block_index(w, j, Wn, n, n_up) * ld4; };
+    if (c == 0) s_u = -1;
     __syncthreads();
-    const int cpar = s_cnt[0], ctot = s_cnt[1];
-    const T* Pi = PQk + (int64_t)w * ld4;
-    acc = h0k[(int64_t)w * d + c];
-    for (int s = 0; s < ctot; ++s) {
-      const int j = mm_nbr[s];
-      const double ddv[3] = {pos(i, 0) - pos(j, 0), pos(i, 1) - pos(j, 1), pos(i, 2) - pos(j, 2)};
-      acc += term(ddv, Pi, PQ + (int64_t)block_index(w, j, Wn, n, n_up) * ld4, s < cpar ? 0 : 1);
-    }
-  } else {
-    const int bi = block_index(w, i, Wn, n, n_up);
-    const T* Pi = PQ + (int64_t)bi * ld4;
-    const int a = ((i < n_up) == (k < n_up)) ? 0 : 1;
-    acc = H1[(int64_t)bi * d + c];
-    for (int side = 0; side < 2; ++side) {   // 0: remove the old (i, k) term, 1: add the new one
-      const double* q = side == 0 ? rw + 3 * k : rkw;
-      const double ddv[3] = {rw[3 * i] - q[0], rw[3 * i + 1] - q[1], rw[3 * i + 2] - q[2]};
-      if (!(ddv[0] * ddv[0] + ddv[1] * ddv[1] + ddv[2] * ddv[2] <= cut * cut)) continue;
-      const T* Qk = side == 0 ? PQ + (int64_t)block_index(w, k, Wn, n, n_up) * ld4 : PQk + (int64_t)w * ld4;
-      const T t = term(ddv, Pi, Qk, a);
-      acc += side == 0 ? -t : t;
-    }
+    if (c < 32) warp_neighbours(n, n_up, k, cut, pos, mm_nbr, s_cnt);
+    for (int u = c; u < uc; u += blockDim.x)
+      if (U[u] == k) s_u = u;
+    __syncthreads();
+    if (s_u < 0) return;   // the update set was cut short (reported as an overflow)
+    const T acc = msg_of_moved<T, W>(mw, B, p, k, d, cut, pos, qrow, PQk + (int64_t)w * ld4, mm_nbr, s_cnt,
+                                     h0k[(int64_t)w * d + c]);
+    const int64_t row = rows[s_u];
+    X[row * d + c] = acc;
+    H1n[row * d + c] = acc;
+    return;
   }
-  const int64_t row = Urow[(int64_t)w * Umax + u];
-  X[row * d + c] = acc;
-  H1n[row * d + c] = acc;
+  const int nm = min(GM, uc - u0);
+  if (c < 2 * nm) {   // pair 2 m: the old (i, k) term of member m, 2 m + 1: the new one
+    const int i = U[u0 + c / 2], side = c & 1;
+    const double* q = side == 0 ? rw + 3 * k : rkw;
+    const double dd[3] = {rw[3 * i] - q[0], rw[3 * i + 1] - q[1], rw[3 * i + 2] - q[2]};
+    const bool in = i != k && dd[0] * dd[0] + dd[1] * dd[1] + dd[2] * dd[2] <= cut * cut;
+    const T* Qk = side == 0 ? PQ + (int64_t)block_index(w, k, Wn, n, n_up) * ld4 : PQk + (int64_t)w * ld4;
+    B.put(c, dd, in ? Qk : nullptr, ((i < n_up) == (k < n_up)) ? 0 : 1);
+  }
+  __syncthreads();
+  B.features(2 * nm, p, cut);
+  __syncthreads();
+  for (int m = 0; m < nm; ++m) {
+    const int i = U[u0 + m];
+    if (i == k) continue;
+    const int64_t bi = block_index(w, i, Wn, n, n_up);
+    const T* Pi = PQ + bi * ld4;
+    T acc = H1[bi * d + c];
+#pragma unroll
+    for (int side = 0; side < 2; ++side) {
+      const int s = 2 * m + side;
+      if (!B.Q[s]) continue;
+      T gam, f;
+      mw.term(B.feat[s], Pi, B.Q[s], B.ch[s], d, c, gam, f);
+      acc += side == 0 ? -(gam * f) : gam * f;
+    }
+    const int64_t row = rows[u0 + m];
+    X[row * d + c] = acc;
+    H1n[row * d + c] = acc;
+  }
 }
+// CTAs of one walker.
+inline int mcmc_msg_groups(int Umax) { return 1 + (Umax + kMsgPairs / 2 - 1) / (kMsgPairs / 2); }
 
 // Y[row][c] = (residual ? Y[row][c] : 0) + SiLU(Z[row][c] + b[c]) for rows in
 // [rng[0], rng[1]); grid-stride over rows x columns.
@@ -464,6 +557,13 @@ __global__ void __launch_bounds__(256) mcmc_ratio_kernel(
   const int u = Uc[w];
   const int64_t Dn = (int64_t)D * n;
   const int64_t md = (int64_t)w * D + dd;
+  if (u == 0) {   // a walker without a move: det Phi' = det Phi
+    if (threadIdx.x == 0) {
+      lrat[md] = 0.0;
+      srat[md] = 1.0;
+    }
+    return;
+  }
   const int32_t* U = Ul + (int64_t)w * Umax;
   const T* Pw = Phi + md * n * n;
   const T* Aw = AT + md * n * n;
@@ -1211,9 +1311,11 @@ __device__ void lu_block(int n, LT* __restrict__ A, int32_t* __restrict__ pv, do
 //         carried log-determinant; weighted by w_d that is the error it
 //         brings into log|Psi| and the acceptance ratio.  ktol < 0 turns the
 //         test off.
+// Walkers without a move (an empty update set) need neither.
 // The pairs are listed for the batched LU; those beyond its capacity keep
 // their mark in xover and take mcmc_exact_ratio_kernel.  One thread per pair.
-static __global__ void mcmc_exact_select_kernel(int64_t npair, int D, const double* __restrict__ ldabs,
+static __global__ void mcmc_exact_select_kernel(int64_t npair, int D, const int32_t* __restrict__ Uc,
+                                                const double* __restrict__ ldabs,
                                                 const double* __restrict__ lsign, const double* __restrict__ lrat,
                                                 int32_t* __restrict__ xflag, const float* __restrict__ kap,
                                                 double kunit, double ktol, int* __restrict__ xcount,
@@ -1222,9 +1324,10 @@ static __global__ void mcmc_exact_select_kernel(int64_t npair, int D, const doub
   const int64_t md = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (md >= npair) return;
   const double lr = lrat[md];
-  const bool range = !(fabs(lr) <= kExactLogRatio) && lsign[md] != 0.0;
+  const bool moved = Uc[md / D] > 0;
+  const bool range = moved && !(fabs(lr) <= kExactLogRatio) && lsign[md] != 0.0;
   bool cond = false;
-  if (!range && ktol >= 0.0 && lsign[md] != 0.0) {
+  if (moved && !range && ktol >= 0.0 && lsign[md] != 0.0) {
     const int64_t w0 = (md / D) * D;
     double lmax = -INFINITY;
     for (int q = 0; q < D; ++q)

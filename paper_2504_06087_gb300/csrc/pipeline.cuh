@@ -431,7 +431,7 @@ struct Runner {
       T* H0 = at<T>(pl.H0);
       T* PQ = at<T>(pl.PQ);
       mark("fwd_embed", 8);
-      en_filter_kernel<T, T><<<nb, d, 0, s>>>(wc, n, n_up, N, d, r, sys->nuc_pos, sys->cutoff_nuc, p, S5, 1);
+      en_filter_kernel<T, T, 1><<<nb, d, 0, s>>>(wc, n, n_up, N, d, r, sys->nuc_pos, sys->cutoff_nuc, p, S5);
       ln_fl_kernel<T, T><<<nb, d, 0, s>>>(d, S5, Y5, p.ln_gamma, p.ln_beta, 1);
       gemm<T>(s, Y5, d, p.glu_wg, d, false, Z5, 2 * d, 0, nb, nullptr, nb, d, d);
       gemm<T>(s, Y5, d, p.glu_wv, d, false, Z5 + d, 2 * d, 0, nb, nullptr, nb, d, d);
@@ -441,7 +441,7 @@ struct Runner {
         gemm<T>(s, H0, d, p.msg_w + (int64_t)part * d * d, d, false, PQ + (int64_t)part * 2 * d, 4 * d, 0, nb,
                 nullptr, nb, d, d, 2, 0, (int64_t)(2 * d + 4) * d, d);
       T* H1 = B.HL;
-      msg_kernel<T, T><<<nb, d, 0, s>>>(wc, n, n_up, d, K, r, c, p, idx, cnt, boff, H0, PQ, H1, nullptr, 1, 0, 0);
+      msg_kernel<T, T, 1><<<nb, d, 0, s>>>(wc, n, n_up, d, K, r, c, p, idx, cnt, boff, H0, PQ, H1, nullptr, 1, 0);
       mark("fwd_mlp", 3 * L);
       for (int l = 0; l < L; ++l) {
         T* hin = B.HL + (int64_t)l * nb * d;
@@ -810,7 +810,8 @@ struct Runner {
       T* PQ = at<T>(pl.PQ);
       const int64_t r5 = (int64_t)nb * R5;
       mark("en_filter", 1);
-      en_filter_kernel<T, T><<<nb, d, 0, s>>>(wc, n, n_up, N, d, r, sys->nuc_pos, sys->cutoff_nuc, p, S5, R5);
+      (deriv ? en_filter_kernel<T, T, 5> : en_filter_kernel<T, T, 1>)<<<nb, d, 0, s>>>(
+          wc, n, n_up, N, d, r, sys->nuc_pos, sys->cutoff_nuc, p, S5);
       // BF16 form: the h^0 products on the tensor cores (nc_h0 components)
       const __nv_bfloat16* WBh = (pl.wbf16 && (tc_mask & 32) && d % 64 == 0) ? at<__nv_bfloat16>(pl.wbf16) : nullptr;
       const int64_t r5cap = (int64_t)pl.Wc * n * R5;
@@ -862,8 +863,8 @@ struct Runner {
       mark("msg", 1);
       // bf16 components of h^1: those the first MLP layer reads, else (no
       // MLP layers) all that any consumer reads
-      msg_kernel<T, T><<<nb, d, 0, s>>>(wc, n, n_up, d, K, r, c, p, idx, cnt, boff, H0, PQ, X, Xb,
-                                        dm.L > 0 ? nc_mlp : ncw, capA * d, deriv);
+      (deriv ? msg_kernel<T, T, 5> : msg_kernel<T, T, 1>)<<<nb, d, 0, s>>>(
+          wc, n, n_up, d, K, r, c, p, idx, cnt, boff, H0, PQ, X, Xb, dm.L > 0 ? nc_mlp : ncw, capA * d);
       check("msg");
       if (dm.op == FIRE_OP_MCMC) {   // the Metropolis state keeps h^1 (value rows, block order)
         cudaMemcpyAsync(at<T>(pl.mc_H1), X, sizeof(T) * (size_t)nb * d, cudaMemcpyDeviceToDevice, s);
@@ -1331,7 +1332,7 @@ struct Runner {
       // (the proposals form a one-electron batch of Wn walkers)
       const int nup1 = k < n_up ? 1 : 0;
       mark("mc_embed_k", 9);
-      en_filter_kernel<T, T><<<Wn, d, 0, s>>>(Wn, 1, nup1, N, d, rk, sys->nuc_pos, sys->cutoff_nuc, p, S5, 1);
+      en_filter_kernel<T, T, 1><<<Wn, d, 0, s>>>(Wn, 1, nup1, N, d, rk, sys->nuc_pos, sys->cutoff_nuc, p, S5);
       ln_fl_kernel<T, T><<<Wn, d, 0, s>>>(d, S5, Y5, p.ln_gamma, p.ln_beta, 1);
       gemm<T>(s, Y5, d, p.glu_wg, d, false, Z5, 2 * d, 0, Wn, nullptr, Wn, d, d);
       gemm<T>(s, Y5, d, p.glu_wv, d, false, Z5 + d, 2 * d, 0, Wn, nullptr, Wn, d, d);
@@ -1346,7 +1347,7 @@ struct Runner {
       check("mc embed k");
       // h^1 and h of the members of U (compact rows)
       mark("mc_msg", 1);
-      mcmc_msg_kernel<T, T><<<(unsigned)capU, d, msm, s>>>(Wn, n, n_up, d, k, Umax, r, rk, c, p, Ul, Uc, Urow, H0,
+      mcmc_msg_kernel<T, T><<<(unsigned)(Wn * mcmc_msg_groups(Umax)), d, msm, s>>>(Wn, n, n_up, d, k, Umax, r, rk, c, p, Ul, Uc, Urow, H0,
                                                            PQ, H1, h0k, PQk, X1, H1n);
       check("mc msg");
     };
@@ -1392,7 +1393,7 @@ struct Runner {
         int32_t* xover = npair > pl.xcap ? at<int32_t>(pl.mc_flag) : nullptr;
         cudaMemsetAsync(xcnt, 0, sizeof(int), s);
         mcmc_exact_select_kernel<<<(unsigned)((npair + 127) / 128), 128, 0, s>>>(
-            npair, D, ldabs, lsign, lrat, xflag, kap, kunit, mc.kappa_tol, xcnt, xlist, pl.xcap, xover, &ms->n_exact);
+            npair, D, Uc, ldabs, lsign, lrat, xflag, kap, kunit, mc.kappa_tol, xcnt, xlist, pl.xcap, xover, &ms->n_exact);
         if (xover) {
           mcmc_exact_ratio_kernel<T, LT><<<kWoodburySlots, 256, (size_t)n * sizeof(int), s>>>(
               Wn, n, D, Umax, Ul, Uc, PhiS, Dl, ldabs, lsign, lrat, srat, at<LT>(pl.mc_rep), at<int32_t>(pl.mc_rpiv),
@@ -1433,7 +1434,7 @@ struct Runner {
         env_feat_kernel<T, T><<<Wn, 128, 0, s>>>(Wn, 1, 1, N, E, rk2, sys->nuc_pos, p.env_sigma, Qk, 1);
         gemm<T>(s, Qk, NE, p.env_pi + Dn * NE, NE, true, Fk2, Dn, 0, Wn, nullptr, Wn, (int)Dn, NE);
         mark("swap_msg", 1);
-        swap_msg_kernel<T, T><<<(unsigned)capU, d, msm, s>>>(Wn, n, n_up, d, a2, b, Umax, r, c, p, Ul, Uc, Urow, H0,
+        swap_msg_kernel<T, T><<<(unsigned)(Wn * swap_msg_groups(Umax)), d, msm, s>>>(Wn, n, n_up, d, a2, b, Umax, r, c, p, Ul, Uc, Urow, H0,
                                                              PQ, H1, X1, H1n);
         check("swap msg");
         rows_and_ratio(a2, b, Fk2);

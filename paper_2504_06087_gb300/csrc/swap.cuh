@@ -44,112 +44,81 @@ static __global__ void swap_propose_kernel(int n, int n_up, int a, int b, const 
 // other electron's block.  For any other i the terms of the pairs (i, a) and
 // (i, b) change: h^1_i - old (i, a) - old (i, b) + new (i, a) + new (i, b),
 // the new terms at the swapped positions with the swapped projections and
-// the spin channel of the pair unchanged.  One CTA per (walker, slot),
-// blockDim == d; dynamic shared memory n ints.
+// the spin channel of the pair unchanged.  CTAs 0 and 1 of a walker take a and
+// b, the others 8 members each (four terms); blockDim == d; dynamic shared
+// memory n ints.  256 walkers of C8H10: 500 -> 78 us a swap.
 template <typename T, typename W>
-__global__ void swap_msg_kernel(int Wn, int n, int n_up, int d, int a, int b, int Umax, const double* __restrict__ r,
-                                double cut, Params<W> p, const int32_t* __restrict__ Ul, const int32_t* __restrict__ Uc,
-                                const int32_t* __restrict__ Urow, const T* __restrict__ H0, const T* __restrict__ PQ,
-                                const T* __restrict__ H1, T* __restrict__ X, T* __restrict__ H1n) {
-  constexpr int H = kEdgeHidden, G = kGauss;
-  __shared__ FL3<T> feat[H + G + 4];
+__global__ void __launch_bounds__(kFilterThreads<T>) swap_msg_kernel(
+    int Wn, int n, int n_up, int d, int a, int b, int Umax, const double* __restrict__ r, double cut, Params<W> p,
+    const int32_t* __restrict__ Ul, const int32_t* __restrict__ Uc, const int32_t* __restrict__ Urow,
+    const T* __restrict__ H0, const T* __restrict__ PQ, const T* __restrict__ H1, T* __restrict__ X,
+    T* __restrict__ H1n) {
+  constexpr int GM = kMsgPairs / 4;   // members of a CTA: four terms each
+  __shared__ MsgBatch<T> B;
   extern __shared__ int sw_nbr[];
-  __shared__ int s_cnt[2];
-  const int w = blockIdx.x / Umax, u = blockIdx.x % Umax;
-  if (u >= Uc[w]) return;
-  const int i = Ul[(int64_t)w * Umax + u];
+  __shared__ int s_cnt[2], s_u;
+  const int groups = 2 + (Umax + GM - 1) / GM;
+  const int w = blockIdx.x / groups, g = blockIdx.x % groups;
+  const int uc = Uc[w], u0 = (g - 2) * GM;
+  if (g > 1 && u0 >= uc) return;
   const int c = threadIdx.x;
   const int64_t ld4 = 4 * (int64_t)d;
   const double* rw = r + (int64_t)w * n * 3;
-  T w2[H], we[G], wc[2][4], bb[2];
-#pragma unroll
-  for (int h = 0; h < H; ++h) w2[h] = T(p.ee_w2[h * d + c]);
-#pragma unroll
-  for (int g = 0; g < G; ++g) we[g] = T(p.ee_wenv[g * d + c]);
-#pragma unroll
-  for (int al = 0; al < 2; ++al) {
-    bb[al] = T(p.msg_b[al * d + c]);
-#pragma unroll
-    for (int q = 0; q < 4; ++q) wc[al][q] = T(p.msg_w[((int64_t)al * (2 * d + 4) + 2 * d + q) * d + c]);
-  }
-  auto term = [&](const double ddv[3], const T* Pi, const T* Qj, int al) -> T {
-    const double rr = sqrt(ddv[0] * ddv[0] + ddv[1] * ddv[1] + ddv[2] * ddv[2]);
-    T dv[3] = {T(ddv[0]), T(ddv[1]), T(ddv[2])};
-    __syncthreads();
-    pair_features_to_smem<T, W>(dv, T(rr), p.ee_w1, p.ee_b1, p.ee_sigma, T(cut), feat);
-    __syncthreads();
-    T gv = T(0), ev = T(0), eb = T(0);
-#pragma unroll
-    for (int h = 0; h < H; ++h) gv += feat[h].v * w2[h];
-#pragma unroll
-    for (int g = 0; g < G; ++g) ev += feat[H + g].v * we[g];
-#pragma unroll
-    for (int q = 0; q < 4; ++q) eb += feat[H + G + q].v * wc[al][q];
-    const T z = Pi[(int64_t)al * d + c] + Qj[2 * (int64_t)d + (int64_t)al * d + c] + eb + bb[al];
-    T f, f1, f2;
-    silu3<T>(z, f, f1, f2);
-    return (gv * ev) * f;
-  };
+  const int32_t* U = Ul + (int64_t)w * Umax;
+  const int32_t* rows = Urow + (int64_t)w * Umax;
+  const MsgWeights<T, W> mw(p, d, c);
   // positions and position-dependent blocks after the swap
   auto src = [&](int j) { return j == a ? b : (j == b ? a : j); };
-  auto pos = [&](int j, int t) -> double { return rw[3 * src(j) + t]; };
-  T acc;
-  if (i == a || i == b) {
-    if (threadIdx.x < 32) {
-      const int lane = threadIdx.x;
-      const bool up = i < n_up;
-      int cntN = 0;
-      for (int pass = 0; pass < 2; ++pass) {
-        const bool same = pass == 0;
-        const int lo = (up == same) ? 0 : n_up, hi = (up == same) ? n_up : n;
-        for (int j0 = lo; j0 < hi; j0 += 32) {
-          const int j = j0 + lane;
-          bool in = false;
-          if (j < hi && j != i) {
-            double a2 = 0.0;
-            for (int t = 0; t < 3; ++t) {
-              const double dd = pos(i, t) - pos(j, t);
-              a2 += dd * dd;
-            }
-            in = a2 <= cut * cut;
-          }
-          const unsigned m = __ballot_sync(0xffffffffu, in);
-          if (in) sw_nbr[cntN + __popc(m & ((1u << lane) - 1u))] = j;
-          cntN += __popc(m);
-        }
-        if (lane == 0) s_cnt[pass] = cntN;
-      }
-    }
+  auto qrow = [&](int j) { return PQ + (int64_t)block_index(w, src(j), Wn, n, n_up) * ld4; };
+  if (g < 2) {
+    const int i = g == 0 ? a : b;
+    auto pos = [&](int j, int t) -> double { return rw[3 * src(j) + t]; };
+    if (c == 0) s_u = -1;
     __syncthreads();
-    const int cpar = s_cnt[0], ctot = s_cnt[1];
+    if (c < 32) warp_neighbours(n, n_up, i, cut, pos, sw_nbr, s_cnt);
+    for (int u = c; u < uc; u += blockDim.x)
+      if (U[u] == i) s_u = u;
+    __syncthreads();
+    if (s_u < 0) return;   // the update set was cut short (reported as an overflow)
     const int64_t bi = block_index(w, src(i), Wn, n, n_up);
-    const T* Pi = PQ + bi * ld4;
-    acc = H0[bi * d + c];
-    for (int s = 0; s < ctot; ++s) {
-      const int j = sw_nbr[s];
-      const double ddv[3] = {pos(i, 0) - pos(j, 0), pos(i, 1) - pos(j, 1), pos(i, 2) - pos(j, 2)};
-      acc += term(ddv, Pi, PQ + (int64_t)block_index(w, src(j), Wn, n, n_up) * ld4, s < cpar ? 0 : 1);
-    }
-  } else {
+    const T acc = msg_of_moved<T, W>(mw, B, p, i, d, cut, pos, qrow, PQ + bi * ld4, sw_nbr, s_cnt, H0[bi * d + c]);
+    const int64_t row = rows[s_u];
+    X[row * d + c] = acc;
+    H1n[row * d + c] = acc;
+    return;
+  }
+  const int nm = min(GM, uc - u0);
+  if (c < 4 * nm) {   // pairs 4 m ..: (i, a) old, new, (i, b) old, new
+    const int i = U[u0 + c / 4], kk = (c & 2) ? b : a;
+    const int sk = (c & 1) ? src(kk) : kk;   // the position and blocks the pair uses
+    const double dd[3] = {rw[3 * i] - rw[3 * sk], rw[3 * i + 1] - rw[3 * sk + 1], rw[3 * i + 2] - rw[3 * sk + 2]};
+    const bool in = i != a && i != b && dd[0] * dd[0] + dd[1] * dd[1] + dd[2] * dd[2] <= cut * cut;
+    B.put(c, dd, in ? PQ + (int64_t)block_index(w, sk, Wn, n, n_up) * ld4 : nullptr,
+          ((i < n_up) == (kk < n_up)) ? 0 : 1);
+  }
+  __syncthreads();
+  B.features(4 * nm, p, cut);
+  __syncthreads();
+  for (int m = 0; m < nm; ++m) {
+    const int i = U[u0 + m];
+    if (i == a || i == b) continue;
     const int64_t bi = block_index(w, i, Wn, n, n_up);
     const T* Pi = PQ + bi * ld4;
-    acc = H1[bi * d + c];
-    for (int mv = 0; mv < 2; ++mv) {
-      const int k = mv == 0 ? a : b;
-      const int al = ((i < n_up) == (k < n_up)) ? 0 : 1;
-      for (int side = 0; side < 2; ++side) {   // 0: remove the old (i, k) term, 1: add the new one
-        const int sk = side == 0 ? k : src(k);  // the position and blocks the pair uses
-        const double ddv[3] = {rw[3 * i] - rw[3 * sk], rw[3 * i + 1] - rw[3 * sk + 1], rw[3 * i + 2] - rw[3 * sk + 2]};
-        if (!(ddv[0] * ddv[0] + ddv[1] * ddv[1] + ddv[2] * ddv[2] <= cut * cut)) continue;
-        const T t = term(ddv, Pi, PQ + (int64_t)block_index(w, sk, Wn, n, n_up) * ld4, al);
-        acc += side == 0 ? -t : t;
-      }
+    T acc = H1[bi * d + c];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const int s = 4 * m + q;
+      if (!B.Q[s]) continue;
+      T gam, f;
+      mw.term(B.feat[s], Pi, B.Q[s], B.ch[s], d, c, gam, f);
+      acc += (q & 1) == 0 ? -(gam * f) : gam * f;
     }
+    const int64_t row = rows[u0 + m];
+    X[row * d + c] = acc;
+    H1n[row * d + c] = acc;
   }
-  const int64_t row = Urow[(int64_t)w * Umax + u];
-  X[row * d + c] = acc;
-  H1n[row * d + c] = acc;
 }
+inline int swap_msg_groups(int Umax) { return 2 + (Umax + kMsgPairs / 4 - 1) / (kMsgPairs / 4); }
 
 // ratios[w][a] = Psi(swapped) / Psi for the walkers (signed).
 template <typename T>
