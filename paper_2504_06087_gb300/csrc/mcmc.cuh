@@ -913,16 +913,17 @@ __global__ void mcmc_rows_kernel(int Wn, int n, int n_up, int d, int Dn, int RD,
 }
 
 // Solves L U x = b in place for 32 right-hand sides, one per lane of a warp:
-// X[i][lane] (row stride 33) holds b and receives x; A holds the factors (unit
-// L, row stride lda) and X[i][32] the reciprocal of U_ii.  Rows below i0 of
-// every b are zero.  A float64 multiply-add of a warp holds the pipe for
+// x[i ldx] (the lane's column) holds b and receives x; A holds the factors
+// (unit L, row stride lda) and rinv[i rs] the reciprocal of U_ii.  Rows below
+// i0 of every b are zero.  A float64 multiply-add of a warp holds the pipe for
 // longer than its latency, so the number of warp instructions is what counts:
 // every lane has a column of its own and each factor is one broadcast load
-// for 32 multiply-adds.  Four rows go together, which loads X once for four
+// for 32 multiply-adds.  Four rows go together, which loads x once for four
 // and keeps four chains in flight.  With rnd the solution of every row is
 // rounded to T before it is used further.
 template <typename T, bool rnd, typename LT, typename CT>
-__device__ __forceinline__ void warp_lu_solve(int n, const LT* __restrict__ A, int64_t lda, CT* X, int i0, int lane) {
+__device__ __forceinline__ void warp_lu_solve(int n, const LT* __restrict__ A, int64_t lda, CT* x, int ldx,
+                                              const CT* rinv, int rs, int i0) {
   auto keep = [](CT v) -> CT { return rnd ? (CT)(T)v : v; };
   i0 &= ~3;
   for (int ib = i0; ib < n; ib += 4) {   // forward: unit lower
@@ -933,13 +934,13 @@ __device__ __forceinline__ void warp_lu_solve(int n, const LT* __restrict__ A, i
     for (int k = 0; k < 4; ++k) {
       const int r = k < nr ? ib + k : ib;
       a[k] = A + (int64_t)r * lda;
-      s[k] = X[r * 33 + lane];
+      s[k] = x[r * ldx];
     }
 #pragma unroll 4
     for (int q = i0; q < ib; ++q) {
-      const CT x = X[q * 33 + lane];
+      const CT v = x[q * ldx];
 #pragma unroll
-      for (int k = 0; k < 4; ++k) s[k] -= (CT)a[k][q] * x;
+      for (int k = 0; k < 4; ++k) s[k] -= (CT)a[k][q] * v;
     }
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
@@ -947,7 +948,7 @@ __device__ __forceinline__ void warp_lu_solve(int n, const LT* __restrict__ A, i
 #pragma unroll
         for (int q = 0; q < k; ++q) s[k] -= (CT)a[k][ib + q] * s[q];
         s[k] = keep(s[k]);
-        X[(ib + k) * 33 + lane] = s[k];
+        x[(ib + k) * ldx] = s[k];
       }
     }
   }
@@ -959,13 +960,13 @@ __device__ __forceinline__ void warp_lu_solve(int n, const LT* __restrict__ A, i
     for (int k = 0; k < 4; ++k) {
       const int r = k < nr ? ib + k : ib;
       a[k] = A + (int64_t)r * lda;
-      s[k] = X[r * 33 + lane];
+      s[k] = x[r * ldx];
     }
 #pragma unroll 4
     for (int q = ib + 4; q < n; ++q) {
-      const CT x = X[q * 33 + lane];
+      const CT v = x[q * ldx];
 #pragma unroll
-      for (int k = 0; k < 4; ++k) s[k] -= (CT)a[k][q] * x;
+      for (int k = 0; k < 4; ++k) s[k] -= (CT)a[k][q] * v;
     }
 #pragma unroll
     for (int k = 3; k >= 0; --k) {
@@ -973,8 +974,8 @@ __device__ __forceinline__ void warp_lu_solve(int n, const LT* __restrict__ A, i
 #pragma unroll
         for (int q = 3; q > k; --q)
           if (q < nr) s[k] -= (CT)a[k][ib + q] * s[q];
-        s[k] = keep(s[k] * X[(ib + k) * 33 + 32]);
-        X[(ib + k) * 33 + lane] = s[k];
+        s[k] = keep(s[k] * rinv[(ib + k) * rs]);
+        x[(ib + k) * ldx] = s[k];
       }
     }
   }
@@ -988,8 +989,8 @@ inline size_t warp_panel_smem(int n, size_t csz) { return (size_t)n * 33 * csz +
 // Row t of P is e_{perm[t]}, so the column of A with the right-hand side e_t is
 // perm[t]: panel p takes t = 32 p .. 32 p + 31, whose forward solves start at
 // row 32 p.  With list, matrix f of the batch (f < *count) goes to slot
-// list[f] of out and a singular one (bsg[f] == 0) becomes zero.  2048
-// matrices of n = 100 in float64: see the dispatch in the pipeline.
+// list[f] of out and a singular one (bsg[f] == 0) becomes zero.  A sweep's
+// refactorisations of C14H16 (n = 100, 128 walkers): 2930 -> 930 us a move.
 template <typename LT, typename AT>
 __global__ void __launch_bounds__(32) inverse_warp_kernel(int n, int64_t m0, const LT* __restrict__ LU,
                                                           const int32_t* __restrict__ piv, AT* __restrict__ Ainv,
@@ -1028,7 +1029,7 @@ __global__ void __launch_bounds__(32) inverse_warp_kernel(int n, int64_t m0, con
   for (int i = 0; i < n; ++i) X[i * 33 + lane] = i == t ? LT(1) : LT(0);
   for (int i = lane; i < n; i += 32) X[i * 33 + 32] = LT(1) / A[(int64_t)i * n + i];
   __syncwarp();
-  warp_lu_solve<LT, false>(n, A, n, X, 32 * p, lane);
+  warp_lu_solve<LT, false>(n, A, n, X + lane, 33, X + 32, 33, 32 * p);
   __syncwarp();
   for (int c = 0; c < 32 && 32 * p + c < n; ++c) {
     AT* o = out + (int64_t)perm[32 * p + c] * n;
@@ -1039,19 +1040,19 @@ __global__ void __launch_bounds__(32) inverse_warp_kernel(int n, int64_t m0, con
 // Woodbury update of A^T and the rows U of Phi for accepted walkers:
 //   B = Delta A (u x n), C = M^-1 B (solved with the LU factors of M),
 //   A'^T[m][l] = A^T[m][l] - sum_a C[a][m] A^T[U_a][l],   Phi_U += Delta.
-// A persistent grid of 256-thread CTAs walks the (walker, det) pairs; CTA b
-// keeps its scratch (Tw: [Umax][n] in Tu, B then C: [Umax][n] in Bw) in slot
-// b.  Flagged pairs are refactorised by mcmc_repair_kernel instead.
-// The float64 solve (|U|^2 n multiply-adds against 2 |U| n^2 float32 ones) is
-// what bounds the kernel: nw warps take 32 columns each (warp_lu_solve), their
-// columns in dynamic shared memory ([nw][Upan][33] doubles); update sets larger
-// than Upan keep their columns in the scratch.
+// This form takes what mcmc_woodbury_panel_kernel does not (umin: the smallest
+// |U| of its share).  A persistent grid of 256-thread CTAs walks the (walker,
+// det) pairs; CTA b keeps its scratch (Tw: [Umax][n] in Tu, B then C: [Umax][n]
+// in Bw) in slot b.  Flagged pairs are refactorised by mcmc_repair_kernel
+// instead.  nw warps take 32 columns each of the float64 solve, their columns
+// in dynamic shared memory ([nw][Upan][33] doubles); update sets larger than
+// Upan keep their columns in the scratch.
 template <typename T>
 __global__ void __launch_bounds__(256) mcmc_woodbury_kernel(
     int Wn, int n, int D, int Umax, const int32_t* __restrict__ acc, const int32_t* __restrict__ flag,
     const int32_t* __restrict__ Ul, const int32_t* __restrict__ Uc, const T* __restrict__ Dl,
     const double* __restrict__ Mlu, const int32_t* __restrict__ Mpiv, T* __restrict__ AT, T* __restrict__ Phi,
-    T* __restrict__ Tu, T* __restrict__ Bw, int Upan, int nw) {
+    T* __restrict__ Tu, T* __restrict__ Bw, int Upan, int nw, int umin) {
   extern __shared__ __align__(16) unsigned char wb_smem[];
   // the product tiles and the LU of M are never live together: one buffer
   __shared__ double su[kLemmaSmem * (kLemmaSmem + 1)];
@@ -1064,6 +1065,7 @@ __global__ void __launch_bounds__(256) mcmc_woodbury_kernel(
     const int w = (int)(md / D);
     if (!acc[w]) continue;
     const int u = Uc[w];
+    if (u < umin) continue;
     const int32_t* U = Ul + (int64_t)w * Umax;
     T* A = AT + md * n * n;
     const T* Dw = Dl + md * Umax * n;
@@ -1106,8 +1108,8 @@ __global__ void __launch_bounds__(256) mcmc_woodbury_kernel(
           }
           __syncwarp();
           // beyond kLemmaSmem the rows are kept in T between the steps
-          if (in_smem) warp_lu_solve<T, false>(u, L, ldl, X, 0, lane);
-          else warp_lu_solve<T, true>(u, L, ldl, X, 0, lane);
+          if (in_smem) warp_lu_solve<T, false>(u, L, ldl, X + lane, 33, X + 32, 33, 0);
+          else warp_lu_solve<T, true>(u, L, ldl, X + lane, 33, X + 32, 33, 0);
           if (m < n)
             for (int c = 0; c < u; ++c) Bm[(int64_t)c * n + m] = (T)X[c * 33 + lane];
         }
@@ -1141,9 +1143,7 @@ __global__ void __launch_bounds__(256) mcmc_woodbury_kernel(
   }
 }
 
-// The Woodbury kernel's panel rows and solving warps: four warps (one per SM
-// quarter) where their panels fit beside the LU of M, two CTAs per SM up to
-// |U| = 64.
+// The general Woodbury kernel's panel rows and solving warps.
 struct WoodburyShape {
   int Upan, nw;
   size_t smem;
@@ -1158,6 +1158,198 @@ inline WoodburyShape woodbury_shape(int n, int Umax) {
   w.smem = w.nw * panel;
   return w;
 }
+
+// The Woodbury update for |U| <= kLemmaSmem and n <= 192, one CTA per (walker,
+// det) with everything but A^T and Delta in shared memory:
+//   1. B = Delta A: Delta and A^T pass through in chunks of 128 bytes of a row,
+//      copied one chunk ahead; a thread owns rows a = ta + 16 i and columns
+//      m = tm + 16 j.
+//   2. C = M^-1 B in float64, one column per lane (warp_lu_solve): |U|^2 n
+//      multiply-adds on the float64 pipe, the bound of the kernel (n = 100,
+//      |U| = 45: 100 k cycles of an SM against 12 k for the float32 products).
+//   3. A^T -= C^T Tw with the old rows U of A^T (Tw) staged before any is
+//      written; 64 x 64 tiles, 4 x 4 outputs per thread.
+// Every output keeps the chain of multiply-adds of the tiled products of the
+// general kernel.  C14H16, 128 walkers, a move:
+// 795 -> 413 us.
+template <typename T, int NJ>
+__global__ void __launch_bounds__(256) mcmc_woodbury_panel_kernel(
+    int n, int D, int Umax, const int32_t* __restrict__ acc, const int32_t* __restrict__ flag,
+    const int32_t* __restrict__ Ul, const int32_t* __restrict__ Uc, const T* __restrict__ Dl,
+    const double* __restrict__ Mlu, const int32_t* __restrict__ Mpiv, T* __restrict__ AT, T* __restrict__ Phi,
+    size_t r1_bytes) {
+  constexpr int LC = 128 / (int)sizeof(T), LS = LC + 16 / (int)sizeof(T);   // chunk and its padded row stride
+  constexpr int VE = 16 / (int)sizeof(T);
+  extern __shared__ __align__(16) unsigned char wp_smem[];
+  __shared__ double s_rinv[kLemmaSmem], s_dump[32];
+  __shared__ int s_pv[kLemmaSmem], s_U[kLemmaSmem];
+  const int64_t md = blockIdx.x;
+  const int w = (int)(md / D);
+  if (!acc[w]) return;
+  const int u = Uc[w];
+  if (u > kLemmaSmem) return;
+  const int tid = threadIdx.x;
+  T* A = AT + md * n * n;
+  const T* Dw = Dl + md * Umax * n;
+  T* P = Phi + md * n * n;
+  if (tid < u) s_U[tid] = Ul[(int64_t)w * Umax + tid];
+  __syncthreads();
+  for (int a = tid >> 5; a < u; a += 8)   // Phi_U += Delta
+    for (int l = tid & 31; l < n; l += 32) P[(int64_t)s_U[a] * n + l] += Dw[(int64_t)a * n + l];
+  if (flag[md]) return;                   // refactorised from Phi instead
+  T* R1 = reinterpret_cast<T*>(wp_smem);
+  double* X = reinterpret_cast<double*>(wp_smem + r1_bytes);   // [u][n]
+  // 1. B = Delta A
+  const int tm = tid & 15, ta = tid >> 4;
+  T b[4][NJ];
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+#pragma unroll
+    for (int j = 0; j < NJ; ++j) b[i][j] = T(0);
+  T* stage[2] = {R1, R1 + (int64_t)(n + kLemmaSmem) * LS};   // [n rows of A^T | u rows of Delta][LS]
+  auto fetch = [&](int l0, T* to) {
+    for (int e = tid; e < (n + u) * LC; e += 256) {
+      const int row = e / LC, c = e % LC, l = l0 + c;
+      const T* src = row < n ? A + (int64_t)row * n : Dw + (int64_t)(row - n) * n;
+      const uint32_t dst = (uint32_t)__cvta_generic_to_shared(to + (int64_t)row * LS + c);
+      const int bytes = l < n ? (int)sizeof(T) : 0;
+      asm volatile("cp.async.ca.shared.global [%0], [%1], %2, %3;" ::"r"(dst), "l"(src + (l < n ? l : 0)),
+                   "n"((int)sizeof(T)), "r"(bytes));
+    }
+    asm volatile("cp.async.commit_group;");
+  };
+  fetch(0, stage[0]);
+  int buf = 0;
+  for (int l0 = 0; l0 < n; l0 += LC) {
+    if (l0 + LC < n) {
+      fetch(l0 + LC, stage[buf ^ 1]);
+      asm volatile("cp.async.wait_group 1;");
+    } else {
+      asm volatile("cp.async.wait_group 0;");
+    }
+    __syncthreads();
+    const T* sa = stage[buf];
+    const T* sd = sa + (int64_t)n * LS;
+#pragma unroll 2
+    for (int c = 0; c < LC; c += VE) {
+      T d[4][VE];
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+        if (16 * i < u) ld_vec<T, VE>(d[i], sd + (int64_t)(ta + 16 * i < u ? ta + 16 * i : u - 1) * LS + c);
+#pragma unroll
+      for (int j = 0; j < NJ; ++j) {
+        if (16 * j < n) {
+          T x[VE];
+          ld_vec<T, VE>(x, sa + (int64_t)(tm + 16 * j < n ? tm + 16 * j : n - 1) * LS + c);
+#pragma unroll
+          for (int i = 0; i < 4; ++i)
+            if (16 * i < u) {
+#pragma unroll
+              for (int v = 0; v < VE; ++v) b[i][j] = fma(d[i][v], x[v], b[i][j]);
+            }
+        }
+      }
+    }
+    __syncthreads();
+    buf ^= 1;
+  }
+  // 2. C = M^-1 B
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+#pragma unroll
+    for (int j = 0; j < NJ; ++j) {
+      const int a = ta + 16 * i, m = tm + 16 * j;
+      if (a < u && m < n) X[a * n + m] = (double)b[i][j];
+    }
+  double* M = reinterpret_cast<double*>(R1);   // [u][u]
+  const double* Mg = Mlu + md * Umax * Umax;
+  for (int e = tid; e < u * u; e += 256) M[e] = Mg[(int64_t)(e / u) * Umax + e % u];
+  if (tid < u) {
+    s_rinv[tid] = 1.0 / Mg[(int64_t)tid * Umax + tid];
+    s_pv[tid] = Mpiv[md * Umax + tid];
+  }
+  __syncthreads();
+  const int lane = tid & 31;
+  for (int m0 = 32 * (tid >> 5); m0 < n; m0 += 256) {
+    const bool in = m0 + lane < n;
+    double* x = in ? X + m0 + lane : s_dump + lane;   // lanes past n work on a value of their own
+    const int ldx = in ? n : 0;
+    for (int c = 0; c < u; ++c) {
+      const int p = s_pv[c];
+      if (p != c) {
+        const double t = x[c * ldx];
+        x[c * ldx] = x[p * ldx];
+        x[p * ldx] = t;
+      }
+    }
+    warp_lu_solve<T, false>(u, M, u, x, ldx, s_rinv, 1, 0);
+  }
+  __syncthreads();
+  // 3. A^T[m][l] -= sum_a C[a][m] Tw[a][l]
+  const int nc = (n + 3) & ~3;
+  T *Cs, *Tw;
+  int ldc;
+  if constexpr (sizeof(T) == 4) {   // C rounded into R1, Tw over the solved columns
+    Cs = R1;
+    ldc = nc;
+    for (int a = tid >> 5; a < u; a += 8)
+      for (int m = lane; m < n; m += 32) Cs[a * nc + m] = (T)X[a * n + m];
+    __syncthreads();
+    Tw = reinterpret_cast<T*>(X);
+  } else {
+    Cs = reinterpret_cast<T*>(X);
+    ldc = n;
+    Tw = R1;
+  }
+  for (int a = tid >> 5; a < u; a += 8)
+    for (int l = lane; l < n; l += 32) Tw[a * nc + l] = A[(int64_t)s_U[a] * n + l];
+  __syncthreads();
+  for (int m0 = 4 * ta; m0 < n; m0 += 64)
+    for (int l0 = 4 * tm; l0 < n; l0 += 64) {
+      T o[4][4];
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) o[i][j] = T(0);
+#pragma unroll 4
+      for (int a = 0; a < u; ++a) {
+        T cv[4], tv[4];
+        if constexpr (sizeof(T) == 4) {
+          ld_vec<T, 4>(cv, Cs + a * ldc + m0);
+          ld_vec<T, 4>(tv, Tw + a * nc + l0);
+        } else {
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            cv[i] = m0 + i < n ? Cs[a * ldc + m0 + i] : T(0);
+            tv[i] = Tw[a * nc + l0 + i];
+          }
+        }
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+#pragma unroll
+          for (int j = 0; j < 4; ++j) o[i][j] = fma(cv[i], tv[j], o[i][j]);
+      }
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+          if (m0 + i < n && l0 + j < n) {
+            T* q = A + (int64_t)(m0 + i) * n + l0 + j;
+            *q = *q - o[i][j];
+          }
+    }
+}
+// Bytes of the first shared region (staging chunks, then M, then C or Tw) and
+// in all.
+template <typename T>
+inline size_t woodbury_panel_r1(int n) {
+  const size_t stage = 2 * (size_t)(n + kLemmaSmem) * 144, lu = (size_t)kLemmaSmem * kLemmaSmem * 8;
+  const size_t prod = (size_t)kLemmaSmem * ((n + 3) & ~3) * sizeof(T);
+  size_t r = stage > lu ? stage : lu;
+  r = r > prod ? r : prod;
+  return (r + 15) & ~(size_t)15;
+}
+inline size_t woodbury_panel_x(int n) { return (size_t)kLemmaSmem * ((n + 3) & ~3) * 8; }
 
 // ---------------------------------------------------------------------------
 // Refresh helpers

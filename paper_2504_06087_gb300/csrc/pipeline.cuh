@@ -1510,11 +1510,26 @@ struct Runner {
             Wn, n, n_up, d, (int)Dn, RD, k, Umax, pl.ld_big, RD1, (dm.flags & FIRE_J_MLP) ? 1 : 0,
             (dm.flags & FIRE_J_ATT) ? 1 : 0, acc, Ul, Uc, Urow, F1n, F2n, F1, F2, SUn, SU, h0k, H0, PQk, PQ, Fk,
             Fenv, Vn, V, G1n, G2n, G1, G2, H1n, H1);
-        mark("mc_woodbury", 1);
+        mark("mc_woodbury", 0);
         const int64_t npair = (int64_t)Wn * D;
-        const WoodburyShape wsh = woodbury_shape(n, Umax);
-        mcmc_woodbury_kernel<T><<<(unsigned)(npair < kWoodburySlots ? npair : kWoodburySlots), 256, wsh.smem, s>>>(
-            Wn, n, D, Umax, acc, flag, Ul, Uc, Dl, Mlu, Mpiv, AT, PhiS, Tu, Bw, wsh.Upan, wsh.nw);
+        // update sets of up to kLemmaSmem members (nearly all) in the panel
+        // kernel, the rest in the general one
+        const bool wpanel = n <= 192;
+        if (wpanel) {
+          const size_t r1 = woodbury_panel_r1<T>(n);
+          auto kern = n <= 64 ? mcmc_woodbury_panel_kernel<T, 4>
+                              : (n <= 128 ? mcmc_woodbury_panel_kernel<T, 8> : mcmc_woodbury_panel_kernel<T, 12>);
+          kern<<<(unsigned)npair, 256, r1 + woodbury_panel_x(n), s>>>(n, D, Umax, acc, flag, Ul, Uc, Dl, Mlu, Mpiv, AT,
+                                                                     PhiS, r1);
+          launches += 1;
+        }
+        if (!wpanel || Umax > kLemmaSmem) {
+          const WoodburyShape wsh = woodbury_shape(n, Umax);
+          mcmc_woodbury_kernel<T><<<(unsigned)(npair < kWoodburySlots ? npair : kWoodburySlots), 256, wsh.smem, s>>>(
+              Wn, n, D, Umax, acc, flag, Ul, Uc, Dl, Mlu, Mpiv, AT, PhiS, Tu, Bw, wsh.Upan, wsh.nw,
+              wpanel ? kLemmaSmem + 1 : 0);
+          launches += 1;
+        }
         mcmc_repair_kernel<T, LT><<<(unsigned)(npair < kWoodburySlots ? npair : kWoodburySlots), 256,
                                     inverse_panel_smem(n, sizeof(LT)), s>>>(
             Wn, n, D, acc, flag, PhiS, AT, ldabs, lsign, lref, at<LT>(pl.mc_rep), at<int32_t>(pl.mc_rpiv));
@@ -1603,6 +1618,9 @@ inline int set_smem_limits() {
   raise((const void*)mcmc_att_kernel<T>);
   if constexpr (sizeof(T) == 4) raise((const void*)inverse_panel_kernel<LT, T, T>);
   raise((const void*)mcmc_woodbury_kernel<T>);
+  raise((const void*)mcmc_woodbury_panel_kernel<T, 4>);
+  raise((const void*)mcmc_woodbury_panel_kernel<T, 8>);
+  raise((const void*)mcmc_woodbury_panel_kernel<T, 12>);
   raise((const void*)mcmc_repair_kernel<T, LT>);
   raise((const void*)inverse_warp_kernel<LT, T>);
   cudaError_t e = cudaGetLastError();
