@@ -550,7 +550,7 @@ __global__ void __launch_bounds__(256) mcmc_ratio_kernel(
     const int32_t* __restrict__ Urow, const T* __restrict__ On, const T* __restrict__ Fenv, const T* __restrict__ Fk,
     const T* __restrict__ Phi, const T* __restrict__ AT, T* __restrict__ Dl, T* __restrict__ Mt,
     double* __restrict__ Mg, int32_t* __restrict__ Mpiv, double* __restrict__ lrat, double* __restrict__ srat,
-    int k2 = -1, const T* __restrict__ Fk2 = nullptr) {
+    const int32_t* __restrict__ xflag, int k2 = -1, const T* __restrict__ Fk2 = nullptr) {
   __shared__ double su[kLemmaSmem * (kLemmaSmem + 1)];   // the product tiles, then M
   __shared__ int s_p;
   const int w = blockIdx.x / D, dd = blockIdx.x % D;
@@ -577,6 +577,7 @@ __global__ void __launch_bounds__(256) mcmc_ratio_kernel(
                              : Fenv[(int64_t)block_index(w, i, Wn, n, n_up) * Dn + dd * n + l];
     Dw[(int64_t)aa * n + l] = o * ph - Pw[(int64_t)i * n + l];
   }
+  if (xflag[md]) return;   // its ratio comes from a float64 LU: only Delta is needed
   // Delta A[:, U] = Delta (u x n) times the rows U of A^T
   T* Mw = Mt + md * Umax * Umax;
   cta_gemm_nt<T>(u, u, n, Dw, n, Aw, n, U, Mw, Umax, T(1), false, reinterpret_cast<T*>(su));
@@ -989,7 +990,7 @@ inline size_t warp_panel_smem(int n, size_t csz) { return (size_t)n * 33 * csz +
 // Row t of P is e_{perm[t]}, so the column of A with the right-hand side e_t is
 // perm[t]: panel p takes t = 32 p .. 32 p + 31, whose forward solves start at
 // row 32 p.  With list, matrix f of the batch (f < *count) goes to slot
-// list[f] of out and a singular one (bsg[f] == 0) becomes zero.  A sweep's
+// list[f] of out (-1: nowhere) and a singular one (bsg[f] == 0) becomes zero.  A sweep's
 // refactorisations of C14H16 (n = 100, 128 walkers): 2930 -> 930 us a move.
 template <typename LT, typename AT>
 __global__ void __launch_bounds__(32) inverse_warp_kernel(int n, int64_t m0, const LT* __restrict__ LU,
@@ -1004,6 +1005,7 @@ __global__ void __launch_bounds__(32) inverse_warp_kernel(int n, int64_t m0, con
   const int64_t f = m0 + blockIdx.x / np;
   const int p = blockIdx.x % np;
   if (count && f >= (*count < cap ? *count : cap)) return;
+  if (list && list[f] < 0) return;
   const int lane = threadIdx.x;
   const LT* A = LU + f * n * n;
   AT* out = Ainv + (list ? (int64_t)list[f] : f) * n * n;
@@ -1489,46 +1491,71 @@ __device__ void lu_block(int n, LT* __restrict__ A, int32_t* __restrict__ pv, do
   __syncthreads();
 }
 
-// Chooses the (walker, det) pairs whose ratio comes from a float64 LU of
-// Phi' = Phi with the rows U replaced (Phi_U + Delta) instead of the lemma:
-//  range  the determinant-lemma ratio is beyond e^{+-kExactLogRatio} or not
-//         finite (xflag 1: refactorised if the move is accepted);
-//  cond   the Woodbury-carried inverse cannot be trusted to the tolerance
-//         ktol, i.e. kappa_d u w_d > ktol, with kappa_d the Frobenius
-//         condition estimate of the last factorisation (kap), u the unit
-//         roundoff of the state (kunit) and w_d = |det Phi_d| / max_q |det Phi_q|
-//         the determinant's weight in the walker's sum (xflag 2).  A float32
-//         inverse of a matrix with kappa ~ 1e6 carries relative errors of
-//         order kappa u ~ 0.06, which a run of moves accumulates into the
-//         carried log-determinant; weighted by w_d that is the error it
-//         brings into log|Psi| and the acceptance ratio.  ktol < 0 turns the
-//         test off.
-// Walkers without a move (an empty update set) need neither.
-// The pairs are listed for the batched LU; those beyond its capacity keep
-// their mark in xover and take mcmc_exact_ratio_kernel.  One thread per pair.
+// The conditioning test of one (walker, det) pair: true when its Woodbury-carried
+// inverse cannot be trusted to the tolerance ktol, i.e. kappa_d u w_d > ktol,
+// with kappa_d the Frobenius condition estimate of the last factorisation
+// (kap), u the unit roundoff of the state (kunit) and w_d = |det Phi_d| /
+// max_q |det Phi_q| the determinant's weight in the walker's sum.  A
+// float32 inverse of a matrix with kappa ~ 1e6 carries relative errors of
+// order kappa u ~ 0.06, which a run of moves accumulates into the carried
+// log-determinant; weighted by w_d that is the error it brings into log|Psi|
+// and the acceptance ratio.  ktol < 0 turns the test off.
+__device__ __forceinline__ bool untrusted(int64_t md, int D, const double* __restrict__ ldabs,
+                                          const double* __restrict__ lsign, const float* __restrict__ kap,
+                                          double kunit, double ktol) {
+  if (!(ktol >= 0.0) || lsign[md] == 0.0) return false;
+  const int64_t w0 = (md / D) * D;
+  double lmax = -INFINITY;
+  for (int q = 0; q < D; ++q)
+    if (lsign[w0 + q] != 0.0 && ldabs[w0 + q] > lmax) lmax = ldabs[w0 + q];
+  return (double)kap[md] * kunit * exp(ldabs[md] - lmax) > ktol;
+}
+
+// Before a move: xflag = 2 for the pairs under the conditioning test, else 0
+// (walkers without a move, i.e. with an empty update set, are not tested).  A
+// determinant refactorised under the test has no inverse (stale): while it
+// stays there its ratios come from float64 LUs, which need none, and an
+// accepted move refactorises it again.  One that the lemma is going to use
+// after all gets its inverse now: it is listed, and marked in over where the
+// list (cap) is full.
+// One thread per pair.
+static __global__ void mcmc_exact_test_kernel(int64_t npair, int D, const int32_t* __restrict__ Uc,
+                                              const double* __restrict__ ldabs, const double* __restrict__ lsign,
+                                              const float* __restrict__ kap, double kunit, double ktol,
+                                              int32_t* __restrict__ xflag, int32_t* __restrict__ stale,
+                                              int* __restrict__ scount, int32_t* __restrict__ slist, int cap,
+                                              int32_t* __restrict__ over) {
+  const int64_t md = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (md >= npair) return;
+  const bool cond = Uc[md / D] > 0 && untrusted(md, D, ldabs, lsign, kap, kunit, ktol);
+  xflag[md] = cond ? 2 : 0;
+  int full = 0;
+  if (stale && stale[md] && !cond) {
+    stale[md] = 0;
+    const int slot = atomicAdd(scount, 1);
+    if (slot < cap) slist[slot] = (int32_t)md;
+    else full = 1;
+  }
+  if (over) over[md] = full;
+}
+
+// Lists the pairs whose ratio comes from a float64 LU of Phi' = Phi with the
+// rows U replaced (Phi_U + Delta): those under the conditioning test (xflag 2)
+// and those whose determinant-lemma ratio is beyond e^{+-kExactLogRatio} or
+// not finite (xflag 1).  Pairs beyond the list's capacity are marked in xover
+// and take mcmc_exact_ratio_kernel.  One thread per pair.
 static __global__ void mcmc_exact_select_kernel(int64_t npair, int D, const int32_t* __restrict__ Uc,
-                                                const double* __restrict__ ldabs,
                                                 const double* __restrict__ lsign, const double* __restrict__ lrat,
-                                                int32_t* __restrict__ xflag, const float* __restrict__ kap,
-                                                double kunit, double ktol, int* __restrict__ xcount,
+                                                int32_t* __restrict__ xflag, int* __restrict__ xcount,
                                                 int32_t* __restrict__ xlist, int xcap, int32_t* __restrict__ xover,
                                                 unsigned long long* __restrict__ nexact) {
   const int64_t md = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (md >= npair) return;
-  const double lr = lrat[md];
-  const bool moved = Uc[md / D] > 0;
-  const bool range = moved && !(fabs(lr) <= kExactLogRatio) && lsign[md] != 0.0;
-  bool cond = false;
-  if (moved && !range && ktol >= 0.0 && lsign[md] != 0.0) {
-    const int64_t w0 = (md / D) * D;
-    double lmax = -INFINITY;
-    for (int q = 0; q < D; ++q)
-      if (lsign[w0 + q] != 0.0 && ldabs[w0 + q] > lmax) lmax = ldabs[w0 + q];
-    cond = (double)kap[md] * kunit * exp(ldabs[md] - lmax) > ktol;
-  }
-  xflag[md] = range ? 1 : (cond ? 2 : 0);
+  const bool cond = xflag[md] != 0;
+  const bool range = !cond && Uc[md / D] > 0 && !(fabs(lrat[md]) <= kExactLogRatio) && lsign[md] != 0.0;
   int over = 0;
   if (range || cond) {
+    if (range) xflag[md] = 1;
     if (nexact) atomicAdd(nexact, 1ull);
     const int slot = atomicAdd(xcount, 1);
     if (slot < xcap) xlist[slot] = (int32_t)md;
@@ -1618,15 +1645,16 @@ static __global__ void mcmc_exact_scatter_kernel(const int* __restrict__ count, 
 }
 
 // Batched refactorisation of the determinants in rlist[0 .. *count) (flag
-// 2): a float64 copy of the cached Phi (already updated by the move) for
-// lu_kernel, then log|det|, sign and the reference log|det| of the new
-// factors, then A^T from them (zero for a singular matrix).  CTAs beyond the
-// count leave.
+// 2): a float64 copy of the cached Phi (already updated by the move) for the
+// LU, then log|det|, sign and the reference log|det| of the new factors, then
+// A^T from them, but not for those that the next move takes under the
+// conditioning test (mcmc_repair_choose_kernel).  The same copy and LU serve
+// the inverses formed later.  CTAs beyond the count leave.
 template <typename T, typename LT>
 __global__ void __launch_bounds__(256) mcmc_repair_build_kernel(int n, const int* __restrict__ count,
                                                                 const int32_t* __restrict__ rlist,
                                                                 const T* __restrict__ Phi, LT* __restrict__ batch) {
-  if ((int)blockIdx.x >= *count) return;
+  if ((int)blockIdx.x >= *count) return;   // (the grid is the list's capacity)
   const T* P = Phi + (int64_t)rlist[blockIdx.x] * n * n;
   LT* L = batch + (int64_t)blockIdx.x * n * n;
   for (int e = threadIdx.x; e < n * n; e += blockDim.x) L[e] = (LT)P[e];
@@ -1645,8 +1673,25 @@ static __global__ void mcmc_repair_scatter_kernel(const int* __restrict__ count,
   lref[md] = blab[f];
 }
 
+// After every log|det| of the move is in place: a refactorised pair that the
+// next move will find under the conditioning test stays without an inverse
+// (stale, its list entry -1).  Half of the inverses of a C14H16 sweep.
+static __global__ void mcmc_repair_choose_kernel(const int* __restrict__ count, int cap, int D,
+                                                 int32_t* __restrict__ rlist, const double* __restrict__ ldabs,
+                                                 const double* __restrict__ lsign, const float* __restrict__ kap,
+                                                 double kunit, double ktol, int32_t* __restrict__ stale) {
+  const int f = blockIdx.x * blockDim.x + threadIdx.x;
+  if (f >= (*count < cap ? *count : cap)) return;
+  const int64_t md = rlist[f];
+  const bool cond = untrusted(md, D, ldabs, lsign, kap, kunit, ktol);
+  stale[md] = cond ? 1 : 0;
+  if (cond) rlist[f] = -1;
+}
+
 // Refactorisation of the flagged (walker, det) pairs of accepted walkers
-// from the cached Phi (already updated by the move): log|det|, sign and A^T.
+// from the cached Phi (already updated by the move): log|det|, sign and A^T
+// (flag 1: those that the batched list had no room for).  Without acc: A^T
+// alone, of every flagged pair.
 // A persistent grid; CTA b uses slot b of the float64 scratch (n x n matrix,
 // n pivots) and dynamic shared memory for the inverse panel.
 template <typename T, typename LT>
@@ -1655,21 +1700,24 @@ __global__ void __launch_bounds__(256) mcmc_repair_kernel(int Wn, int n, int D, 
                                                           const T* __restrict__ Phi, T* __restrict__ AT,
                                                           double* __restrict__ ldabs, double* __restrict__ lsign,
                                                           double* __restrict__ lref, LT* __restrict__ scratch,
-                                                          int32_t* __restrict__ spiv) {
+                                                          int32_t* __restrict__ spiv, int32_t* __restrict__ stale) {
   extern __shared__ unsigned char rp_smem[];
   __shared__ double s_la, s_sg;
   LT* L = scratch + (int64_t)blockIdx.x * n * n;
   int32_t* pv = spiv + (int64_t)blockIdx.x * n;
   for (int64_t md = blockIdx.x; md < (int64_t)Wn * D; md += gridDim.x) {
-    if (!acc[md / D] || flag[md] != 1) continue;
+    if ((acc && !acc[md / D]) || flag[md] != 1) continue;
     const T* P = Phi + md * n * n;
     for (int e = threadIdx.x; e < n * n; e += blockDim.x) L[e] = (LT)P[e];
     __syncthreads();
     lu_block<LT>(n, L, pv, &s_la, &s_sg);
     if (threadIdx.x == 0) {
-      ldabs[md] = s_la;
-      lsign[md] = s_sg;
-      lref[md] = s_la;
+      if (acc) {
+        ldabs[md] = s_la;
+        lsign[md] = s_sg;
+        lref[md] = s_la;
+      }
+      stale[md] = 0;
     }
     T* A = AT + md * n * n;
     if (s_sg == 0.0) {

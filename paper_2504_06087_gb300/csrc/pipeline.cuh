@@ -1260,6 +1260,7 @@ struct Runner {
     double* lref = at<double>(pl.mc_lref);
     int32_t* flag = at<int32_t>(pl.mc_flag);
     int32_t* xflag = at<int32_t>(pl.mc_xflag);
+    int32_t* stale = at<int32_t>(pl.mc_stale);
     // the state, in the value-forward buffers
     T* H0 = at<T>(pl.H0);
     T* PQ = at<T>(pl.PQ);
@@ -1295,6 +1296,7 @@ struct Runner {
       int rc = run();
       reset_status = false;
       if (rc != FIRE_OK) return rc;
+      cudaMemsetAsync(stale, 0, sizeof(int32_t) * (size_t)Wn * D, s);
       mcmc_kappa_kernel<T><<<(unsigned)((int64_t)Wn * D), 256, 0, s>>>(n, PhiS, AT, kap);
       launches += 1;
       cudaMemcpyAsync(lref, at<double>(pl.ldabs), sizeof(double) * (size_t)Wn * D, cudaMemcpyDeviceToDevice, s);
@@ -1380,20 +1382,38 @@ struct Runner {
         gemm<T>(s, X1, d, p.orb_w + (int64_t)sp * D * d * n, n, false, On, Dn, 0, 0, rngu + 2 * sp, capU, n, d, D,
                 0, (int64_t)d * n, n);
       check("mc orbitals");
-      mark("mc_ratio", 1);
-      mcmc_ratio_kernel<T><<<(unsigned)(Wn * D), 256, 0, s>>>(Wn, n, n_up, D, k, Umax, Ul, Uc, Urow, On, Fenv, Fk,
-                                                             PhiS, AT, Dl, Mt, Mlu, Mpiv, lrat, srat, k2,
-                                                             Fk2);
       {
         const int64_t npair = (int64_t)Wn * D;
-        int* xcnt = at<int>(pl.mc_xcnt);
+        int* xcnt = at<int>(pl.mc_xcnt);   // [0] pairs with exact ratios, [1] inverses to be formed
         int32_t* xlist = at<int32_t>(pl.mc_xlist);
-        // pairs whose ratio needs a float64 LU of Phi', then that LU over all
-        // SMs; only a batch beyond its capacity leaves any to the per-CTA path
+        int32_t* pend = mc.ecp || mc.swap_beta >= 0 ? nullptr : stale;   // nothing is accepted there
+        // only a batch beyond the lists' capacity leaves any pair to the per-CTA kernels
         int32_t* xover = npair > pl.xcap ? at<int32_t>(pl.mc_flag) : nullptr;
-        cudaMemsetAsync(xcnt, 0, sizeof(int), s);
+        LT* xb0 = at<LT>(pl.mc_xbatch);
+        mark("mc_inverse", 1);
+        cudaMemsetAsync(xcnt, 0, 2 * sizeof(int), s);
+        mcmc_exact_test_kernel<<<(unsigned)((npair + 127) / 128), 128, 0, s>>>(
+            npair, D, Uc, ldabs, lsign, kap, kunit, mc.kappa_tol, xflag, pend, xcnt + 1, xlist, pl.xcap, xover);
+        if (pend) {
+          int32_t* xpiv = at<int32_t>(pl.mc_xpiv);
+          mcmc_repair_build_kernel<T, LT><<<pl.xcap, 256, 0, s>>>(n, xcnt + 1, xlist, PhiS, xb0);
+          lu_batch<LT>(s, n, pl.xcap, xb0, xpiv, at<double>(pl.mc_xlab), at<double>(pl.mc_xsg), xcnt + 1);
+          inverse_warp<T>(n, pl.xcap, xb0, xpiv, AT, xcnt + 1, pl.xcap, xlist, at<double>(pl.mc_xsg));
+          launches += 2;
+          if (xover) {
+            mcmc_repair_kernel<T, LT><<<kWoodburySlots, 256, inverse_panel_smem(n, sizeof(LT)), s>>>(
+                Wn, n, D, nullptr, xover, PhiS, AT, nullptr, nullptr, nullptr, at<LT>(pl.mc_rep),
+                at<int32_t>(pl.mc_rpiv), stale);
+            launches += 1;
+          }
+        }
+        mark("mc_ratio", 2);
+        mcmc_ratio_kernel<T><<<(unsigned)(Wn * D), 256, 0, s>>>(Wn, n, n_up, D, k, Umax, Ul, Uc, Urow, On, Fenv, Fk,
+                                                               PhiS, AT, Dl, Mt, Mlu, Mpiv, lrat, srat, xflag, k2,
+                                                               Fk2);
+        // pairs whose ratio needs a float64 LU of Phi', then that LU over all SMs
         mcmc_exact_select_kernel<<<(unsigned)((npair + 127) / 128), 128, 0, s>>>(
-            npair, D, Uc, ldabs, lsign, lrat, xflag, kap, kunit, mc.kappa_tol, xcnt, xlist, pl.xcap, xover, &ms->n_exact);
+            npair, D, Uc, lsign, lrat, xflag, xcnt, xlist, pl.xcap, xover, &ms->n_exact);
         if (xover) {
           mcmc_exact_ratio_kernel<T, LT><<<kWoodburySlots, 256, (size_t)n * sizeof(int), s>>>(
               Wn, n, D, Umax, Ul, Uc, PhiS, Dl, ldabs, lsign, lrat, srat, at<LT>(pl.mc_rep), at<int32_t>(pl.mc_rpiv),
@@ -1408,7 +1428,7 @@ struct Runner {
         lu_batch<LT>(s, n, pl.xcap, xb, at<int32_t>(pl.mc_xpiv), xlab, xsg, xcnt);
         mcmc_exact_scatter_kernel<<<(pl.xcap + 255) / 256, 256, 0, s>>>(xcnt, pl.xcap, xlist, xlab, xsg, ldabs,
                                                                        lsign, lrat, srat);
-        launches += 4;
+        launches += 3;
       }
       check("mc ratio");
     };
@@ -1532,10 +1552,10 @@ struct Runner {
         }
         mcmc_repair_kernel<T, LT><<<(unsigned)(npair < kWoodburySlots ? npair : kWoodburySlots), 256,
                                     inverse_panel_smem(n, sizeof(LT)), s>>>(
-            Wn, n, D, acc, flag, PhiS, AT, ldabs, lsign, lref, at<LT>(pl.mc_rep), at<int32_t>(pl.mc_rpiv));
+            Wn, n, D, acc, flag, PhiS, AT, ldabs, lsign, lref, at<LT>(pl.mc_rep), at<int32_t>(pl.mc_rpiv), stale);
         {
           // the listed refactorisations, batched over all SMs: float64 LU of
-          // the updated Phi, then the inverse from the factors
+          // the updated Phi, then the inverses that the next move will use
           LT* xb = at<LT>(pl.mc_xbatch);
           int32_t* xpiv = at<int32_t>(pl.mc_xpiv);
           double* xlab = at<double>(pl.mc_xlab);
@@ -1544,6 +1564,8 @@ struct Runner {
           lu_batch<LT>(s, n, pl.xcap, xb, xpiv, xlab, xsg, rcnt);
           mcmc_repair_scatter_kernel<<<(pl.xcap + 255) / 256, 256, 0, s>>>(rcnt, pl.xcap, rlist, xlab, xsg, ldabs,
                                                                           lsign, lref);
+          mcmc_repair_choose_kernel<<<(pl.xcap + 255) / 256, 256, 0, s>>>(rcnt, pl.xcap, D, rlist, ldabs, lsign, kap,
+                                                                         kunit, mc.kappa_tol, stale);
           inverse_warp<T>(n, pl.xcap, xb, xpiv, AT, rcnt, pl.xcap, rlist, xsg);
         }
         launches += 5;
