@@ -156,201 +156,279 @@ __global__ void att_bwd_kernel(int Wc, int n, int n_up, int R, int dr, const T* 
   }
 }
 
-// Reduces 48 per-thread values over the CTA (blockDim multiple of 32, <= 1024)
-// into out[0..48).  `part` has room for 32 x 48 values.
+// ---------------------------------------------------------------------------
+// Backward of the filters Gamma = (a W_2) * (chi W_env), a = SiLU(x W_1 + b_1),
+// shared by the message and the electron-nucleus passes.  blockDim == d, one
+// column each; pairs go in batches of kGradPairs:
+//   forward  the caller forms Gamma's factors of every pair from the features
+//            in shared memory and leaves s_e = dGamma chi-factor and s_g =
+//            dGamma a-factor of its column in shared memory;
+//   columns  d W_2[h][c] += a_h s_e[c], d W_env[g][c] += chi_g s_g[c], the
+//            running sums in shared memory between batches (in registers beside
+//            the 48 weights of the forward they left one CTA per SM);
+//   rows     sum_c s_e[c] W_2[h][c] and sum_c s_g[c] W_env[g][c], a product of
+//            [pairs x d] with [d x 48]: a warp takes four pairs and 24 of the
+//            48 outputs, so a weight is loaded once for four pairs, and reduces
+//            its 96 sums by transpose-halving; then d W_1, d b_1 and d sigma of
+//            each pair into the CTA's sums.
+// One pair at a time, with derivative features and a 48-value CTA reduction per
+// pair, the electron-nucleus pass of C26H24 (128 walkers) took 27.3 ms and the
+// message pass 18.0 ms; now 3.8 and 4.3 ms.
+// ---------------------------------------------------------------------------
+constexpr int kGradPairs = 16;
+
 template <typename T>
-__device__ __forceinline__ void block_reduce48(T v[48], T* part, T* out) {
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  // warp transpose-reduction (recursive halving): at each step a lane keeps
-  // half of its values and adds its partner's copy of them, so lane L ends
-  // with the warp sums of values L and (L < 16) 32 + L -- 62 shuffles
-  // instead of 5 per value
-  T a[32], b[16];
-#pragma unroll
-  for (int k = 0; k < 32; ++k) a[k] = v[k];
-#pragma unroll
-  for (int k = 0; k < 16; ++k) b[k] = v[32 + k];
-#pragma unroll
-  for (int s = 16; s >= 1; s >>= 1) {
-    const bool up = (lane & s) != 0;
-#pragma unroll
-    for (int k = 0; k < s; ++k) {
-      const T send = up ? a[k] : a[k + s];
-      const T keep = up ? a[k + s] : a[k];
-      a[k] = keep + __shfl_xor_sync(0xffffffffu, send, s);
-    }
-  }
-#pragma unroll
-  for (int k = 0; k < 16; ++k) b[k] += __shfl_xor_sync(0xffffffffu, b[k], 16);
-#pragma unroll
-  for (int s = 8; s >= 1; s >>= 1) {
-    const bool up = (lane & s) != 0;
-#pragma unroll
-    for (int k = 0; k < s; ++k) {
-      const T send = up ? b[k] : b[k + s];
-      const T keep = up ? b[k + s] : b[k];
-      b[k] = keep + __shfl_xor_sync(0xffffffffu, send, s);
-    }
-  }
-  part[wid * 48 + lane] = a[0];
-  if (lane < 16) part[wid * 48 + 32 + lane] = b[0];
-  __syncthreads();
-  for (int t = threadIdx.x; t < 48; t += blockDim.x) {
-    T s = T(0);
-    for (int q = 0; q < nw; ++q) s += part[q * 48 + t];
-    out[t] = s;
-  }
-  __syncthreads();
+struct FilterGrad {
+  PairFeat<T, 1> feat[kGradPairs];
+  T dv[kGradPairs][3], r[kGradPairs];
+  T acc[5 * kEdgeHidden + kGauss];   // d W_1 (4 x H), d b_1, d sigma
+};
+// Dynamic shared memory: FilterGrad, s_e and s_g [kGradPairs][d], column sums [48][d].
+template <typename T>
+inline size_t filter_grad_smem(int d) {
+  return ((sizeof(FilterGrad<T>) + 15) & ~(size_t)15) + (size_t)(2 * kGradPairs + kEdgeHidden + kGauss) * d * sizeof(T);
 }
+template <typename T>
+struct FilterGradMem {
+  FilterGrad<T>* f;
+  T *se, *sg, *col;
+  __device__ __forceinline__ FilterGradMem(unsigned char* sm, int d) {
+    f = reinterpret_cast<FilterGrad<T>*>(sm);
+    se = reinterpret_cast<T*>(sm + ((sizeof(FilterGrad<T>) + 15) & ~(size_t)15));
+    sg = se + kGradPairs * d;
+    col = sg + kGradPairs * d;
+    const int c = threadIdx.x;
+    for (int t = 0; t < kEdgeHidden + kGauss; ++t) col[t * d + c] = T(0);
+    for (int t = c; t < 5 * kEdgeHidden + kGauss; t += blockDim.x) f->acc[t] = T(0);
+  }
+};
 
-// Filter backward shared by the message and electron-nucleus passes: given
-// dGamma_c for the pair vector delta (features in feat, see
-// pair_features_to_smem), accumulates the gradient of W2 (16 x d), W_env
-// (32 x d) in registers and of W1 (4 x H), b1, sigma either into the CTA's
-// shared accumulator acc[5H + G] (ACC: the weights are the same for every
-// pair of the CTA; layout W1 rows 0..3, b1, sigma) or by atomics into
-// gW1/gb1/gsig (per-nucleus weights).  Entry t of the 48 reduced values is
-// handled by thread t mod blockDim, the same thread for every pair, so the
-// shared accumulator needs no atomics.
-template <bool ACC, typename T, typename W>
-__device__ __forceinline__ void filter_bwd(const FL3<T>* feat, const T dv[3], T r, T cut, const W* w1,
-                                           const W* b1, const W* sigma, const T w2c[kEdgeHidden],
-                                           const T wec[kGauss], T gv, T ev, T dgam, T gW2[kEdgeHidden],
-                                           T gWe[kGauss], T* part, T* red48, T* acc, T* gW1, T* gb1, T* gsig) {
-  constexpr int H = kEdgeHidden, G = kGauss;
-  T v[48];
-#pragma unroll
-  for (int h = 0; h < H; ++h) {
-    gW2[h] += feat[h].v * dgam * ev;
-    v[h] = dgam * ev * w2c[h];
-  }
-#pragma unroll
-  for (int g = 0; g < G; ++g) {
-    gWe[g] += feat[H + g].v * dgam * gv;
-    v[H + g] = dgam * gv * wec[g];
-  }
-  block_reduce48<T>(v, part, red48);
-  for (int t = threadIdx.x; t < H + G; t += blockDim.x) {
-    if (t < H) {
-      // du_h = da_h * SiLU'(u_h), u_h = x . W1[:, h] + b1[h], x = [r, delta]
-      T u = T(b1[t]) + T(w1[t]) * r;
-      for (int k = 0; k < 3; ++k) u += T(w1[(1 + k) * H + t]) * dv[k];
-      T f, f1, f2;
-      silu3<T>(u, f, f1, f2);
-      const T du = red48[t] * f1;
-      if (ACC) {
-        acc[t] += du * r;
-        for (int k = 0; k < 3; ++k) acc[(1 + k) * H + t] += du * dv[k];
-        acc[4 * H + t] += du;
-      } else {
-        atomicAdd(&gW1[0 * H + t], du * r);
-        for (int k = 0; k < 3; ++k) atomicAdd(&gW1[(1 + k) * H + t], du * dv[k]);
-        atomicAdd(&gb1[t], du);
-      }
-    } else {
-      // chi_g = f_cut exp(-sigma_g^2 r^2): d chi_g / d sigma_g = -2 sigma_g r^2 chi_g
-      const int g = t - H;
-      const T sg = T(sigma[g]);
-      const T ds = red48[t] * (-T(2) * sg * r * r) * feat[H + g].v;
-      if (ACC) acc[5 * H + g] += ds;
-      else atomicAdd(&gsig[g], ds);
-    }
-  }
-}
-
-// Message-passing backward.  One CTA per electron (w, i), blockDim == d.
-// Inputs: dH1 = d/dh^1_i; recomputes each edge.  Outputs: dP [nb][2d]
-// (own rows), dQ [nb][2d] (atomics at j), parameter gradients of the e-e
-// filter, W^alpha_c and b^alpha.
+// The column and row sums of a batch of nb pairs (barriers inside: the
+// features, s_e and s_g must be in place before; both are free after).
 template <typename T, typename W>
-__global__ void msg_bwd_kernel(int Wc, int n, int n_up, int d, int K, const double* __restrict__ r,
-                               double cut, Params<W> p, const int32_t* __restrict__ idx,
-                               const int32_t* __restrict__ cnt, const T* __restrict__ PQ,
-                               const T* __restrict__ dH1, T* __restrict__ dP, T* __restrict__ dQ,
-                               T* __restrict__ grad, int64_t P, const int64_t* __restrict__ po) {
+__device__ __forceinline__ void filter_grad_batch(const FilterGradMem<T>& m, int nb, int d, const W* w1, const W* b1,
+                                                  const W* w2, const W* wenv, const W* sigma) {
   constexpr int H = kEdgeHidden, G = kGauss;
-  __shared__ FL3<T> feat[H + G + 4];
-  __shared__ T part[32 * 48];
-  __shared__ T red48[48];
-  __shared__ T acc[5 * H + G];
-  const int blk = blockIdx.x;
-  const int w = blk / n, i = blk % n;
   const int c = threadIdx.x;
-  const int bi = block_index(w, i, Wc, n, n_up);
-  for (int t = c; t < 5 * H + G; t += blockDim.x) acc[t] = T(0);
+  {
+    T a[H + G];
+#pragma unroll
+    for (int t = 0; t < H + G; ++t) a[t] = m.col[t * d + c];
+    for (int q = 0; q < nb; ++q) {
+      const T e = m.se[q * d + c], g = m.sg[q * d + c];
+#pragma unroll
+      for (int t = 0; t < H + G; t += 4) {
+        T f[4];
+        ld_vec<T, 4>(f, &m.f->feat[q].f[t][0]);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) a[t + i] += f[i] * (t < H ? e : g);
+      }
+    }
+#pragma unroll
+    for (int t = 0; t < H + G; ++t) m.col[t * d + c] = a[t];
+  }
+  __syncthreads();   // s_e and s_g of every column
+  constexpr int NO = (H + G) / 2, NQ = 4;   // outputs and pairs of a warp's task
+  const int lane = c & 31, nw = blockDim.x >> 5;
+  for (int task = c >> 5; task < 2 * (kGradPairs / NQ); task += nw) {
+    const int q0 = (task >> 1) * NQ, t0 = (task & 1) * NO;
+    if (q0 >= nb) continue;
+    T v[NQ * NO];
+#pragma unroll
+    for (int k = 0; k < NQ * NO; ++k) v[k] = T(0);
+    for (int k = lane; k < d; k += 32) {
+      T e[NQ], g[NQ];
+#pragma unroll
+      for (int q = 0; q < NQ; ++q) {   // rows past nb hold an earlier batch: their sums are dropped
+        e[q] = m.se[(q0 + q) * d + k];
+        g[q] = m.sg[(q0 + q) * d + k];
+      }
+#pragma unroll
+      for (int o = 0; o < NO; ++o) {
+        const int t = t0 + o;
+        const T w = T(t < H ? w2[t * d + k] : wenv[(t - H) * d + k]);
+#pragma unroll
+        for (int q = 0; q < NQ; ++q) v[q * NO + o] += w * (t < H ? e[q] : g[q]);
+      }
+    }
+    // lane L ends with the warp sums of values 32 b + L, b = 0, 1, 2
+#pragma unroll
+    for (int b = 0; b < 3; ++b) {
+      T* a = v + 32 * b;
+#pragma unroll
+      for (int s = 16; s >= 1; s >>= 1) {
+        const bool up = (lane & s) != 0;
+#pragma unroll
+        for (int k = 0; k < s; ++k) {
+          const T send = up ? a[k] : a[k + s];
+          const T keep = up ? a[k + s] : a[k];
+          a[k] = keep + __shfl_xor_sync(0xffffffffu, send, s);
+        }
+      }
+      const int id = 32 * b + lane, q = q0 + id / NO, t = t0 + id % NO;
+      if (q >= nb) continue;
+      const T rr = m.f->r[q];
+      if (t < H) {
+        // du_h = da_h * SiLU'(u_h), u_h = x . W1[:, h] + b1[h], x = [r, delta]
+        T u = T(b1[t]) + T(w1[t]) * rr;
+#pragma unroll
+        for (int k = 0; k < 3; ++k) u += T(w1[(1 + k) * H + t]) * m.f->dv[q][k];
+        T f, f1, f2;
+        silu3<T>(u, f, f1, f2);
+        const T du = a[0] * f1;
+        atomicAdd(&m.f->acc[t], du * rr);
+#pragma unroll
+        for (int k = 0; k < 3; ++k) atomicAdd(&m.f->acc[(1 + k) * H + t], du * m.f->dv[q][k]);
+        atomicAdd(&m.f->acc[4 * H + t], du);
+      } else {
+        // chi_g = f_cut exp(-sigma_g^2 r^2): d chi_g / d sigma_g = -2 sigma_g r^2 chi_g
+        const T sgm = T(sigma[t - H]);
+        atomicAdd(&m.f->acc[5 * H + t - H], a[0] * (-T(2) * sgm * rr * rr) * m.f->feat[q].f[t][0]);
+      }
+    }
+  }
+  __syncthreads();
+}
+
+// Gamma's factors of one pair and this thread's column (weights read per
+// batch: they are live in the forward part only).
+template <typename T, typename W>
+struct FilterWeights {
+  T w2[kEdgeHidden], we[kGauss];
+  __device__ __forceinline__ FilterWeights(const W* pw2, const W* pwe, int d, int c) {
+#pragma unroll
+    for (int h = 0; h < kEdgeHidden; ++h) w2[h] = T(pw2[h * d + c]);
+#pragma unroll
+    for (int g = 0; g < kGauss; ++g) we[g] = T(pwe[g * d + c]);
+  }
+  __device__ __forceinline__ void factors(const PairFeat<T, 1>& f, T& gv, T& ev) const {
+    T a[1] = {T(0)}, b[1] = {T(0)};
+    feat_dot<kEdgeHidden, 1, T>(f, 0, w2, a);
+    feat_dot<kGauss, 1, T>(f, kEdgeHidden, we, b);
+    gv = a[0];
+    ev = b[0];
+  }
+};
+
+// Message-passing backward.  One CTA per epc consecutive electrons of a walker
+// (the pairs of all of them in one list), blockDim == d.  Inputs: dH1 =
+// d/dh^1_i; recomputes each edge.  Outputs: dP [nb][2d] (own rows), dQ [nb][2d]
+// (atomics at j), parameter gradients of the e-e filter, W^alpha_c and b^alpha.
+constexpr int kGradElectrons = 8;   // largest epc
+template <typename T, typename W>
+__global__ void __launch_bounds__(256, sizeof(T) == 4 ? 2 : 1) msg_bwd_kernel(
+    int Wc, int n, int n_up, int d, int K, int epc, const double* __restrict__ r, double cut, Params<W> p,
+    const int32_t* __restrict__ idx, const int32_t* __restrict__ cnt, const T* __restrict__ PQ,
+    const T* __restrict__ dH1, T* __restrict__ dP, T* __restrict__ dQ, T* __restrict__ grad, int64_t P,
+    const int64_t* __restrict__ po) {
+  constexpr int H = kEdgeHidden, G = kGauss;
+  extern __shared__ __align__(16) unsigned char fg_smem[];
+  __shared__ int s_off[kGradElectrons + 1], s_par[kGradElectrons];
+  __shared__ int s_e[kGradPairs], s_j[kGradPairs], s_a[kGradPairs];
+  const int groups = (n + epc - 1) / epc;
+  const int w = blockIdx.x / groups, i0 = (blockIdx.x % groups) * epc;
+  const int ne = min(epc, n - i0);
+  const int c = threadIdx.x;
+  const FilterGradMem<T> m(fg_smem, d);
   const int64_t ld4 = 4 * (int64_t)d;
   T* gw = grad + (int64_t)w * P;
-  T w2[H], we[G], wc[2][4], bb[2];
-#pragma unroll
-  for (int h = 0; h < H; ++h) w2[h] = T(p.ee_w2[h * d + c]);
-#pragma unroll
-  for (int g = 0; g < G; ++g) we[g] = T(p.ee_wenv[g * d + c]);
-#pragma unroll
-  for (int a = 0; a < 2; ++a) {
-    bb[a] = T(p.msg_b[a * d + c]);
-#pragma unroll
-    for (int k = 0; k < 4; ++k) wc[a][k] = T(p.msg_w[((int64_t)a * (2 * d + 4) + 2 * d + k) * d + c]);
+  const double* rw = r + (int64_t)w * n * 3;
+  if (c == 0) {
+    int o = 0;
+    for (int e = 0; e < ne; ++e) {
+      const int32_t* ce = cnt + ((int64_t)w * n + i0 + e) * 2;
+      s_off[e] = o;
+      s_par[e] = ce[0];
+      o += ce[0] + ce[1];
+    }
+    s_off[ne] = o;
   }
-  T gW2[H], gWe[G], gWc[2][4], gB[2], dPa[2];
-#pragma unroll
-  for (int h = 0; h < H; ++h) gW2[h] = T(0);
-#pragma unroll
-  for (int g = 0; g < G; ++g) gWe[g] = T(0);
+  __syncthreads();
+  const int total = s_off[ne];
+  T gWc[2][4], gB[2], dPa[2];
 #pragma unroll
   for (int a = 0; a < 2; ++a) {
     gB[a] = dPa[a] = T(0);
 #pragma unroll
     for (int k = 0; k < 4; ++k) gWc[a][k] = T(0);
   }
-  const T delta = dH1[(int64_t)bi * d + c];
-  const int cpar = cnt[((int64_t)w * n + i) * 2], ctot = cpar + cnt[((int64_t)w * n + i) * 2 + 1];
-  const double* rw = r + (int64_t)w * n * 3;
-  const int32_t* li = idx + ((int64_t)w * n + i) * K;
-  for (int s = 0; s < ctot; ++s) {
-    const int j = li[s];
-    const int a = (s < cpar) ? 0 : 1;
-    double ddv[3] = {rw[3 * i] - rw[3 * j], rw[3 * i + 1] - rw[3 * j + 1], rw[3 * i + 2] - rw[3 * j + 2]};
-    const double rr = sqrt(ddv[0] * ddv[0] + ddv[1] * ddv[1] + ddv[2] * ddv[2]);
-    T dv[3] = {T(ddv[0]), T(ddv[1]), T(ddv[2])};
-    __syncthreads();
-    pair_features_to_smem<T, W>(dv, T(rr), p.ee_w1, p.ee_b1, p.ee_sigma, T(cut), feat);
-    __syncthreads();
-    T gv = T(0), ev = T(0);
-#pragma unroll
-    for (int h = 0; h < H; ++h) gv += feat[h].v * w2[h];
-#pragma unroll
-    for (int g = 0; g < G; ++g) ev += feat[H + g].v * we[g];
-    const T gam = gv * ev;
-    const int bj = block_index(w, j, Wc, n, n_up);
-    T z = PQ[(int64_t)bi * ld4 + (int64_t)a * d + c] + PQ[(int64_t)bj * ld4 + 2 * (int64_t)d + (int64_t)a * d + c] +
-          bb[a];
-#pragma unroll
-    for (int k = 0; k < 4; ++k) z += feat[H + G + k].v * wc[a][k];
-    T f, f1, f2;
-    silu3<T>(z, f, f1, f2);
-    const T dgam = delta * f;
-    const T dz = delta * gam * f1;
-    dPa[a] += dz;
-    atomicAdd(&dQ[(int64_t)bj * 2 * d + (int64_t)a * d + c], dz);
-    gB[a] += dz;
-#pragma unroll
-    for (int k = 0; k < 4; ++k) gWc[a][k] += feat[H + G + k].v * dz;
-    filter_bwd<true, T, W>(feat, dv, T(rr), T(cut), p.ee_w1, p.ee_b1, p.ee_sigma, w2, we, gv, ev, dgam, gW2,
-                           gWe, part, red48, acc, nullptr, nullptr, nullptr);
-  }
-  dP[(int64_t)bi * 2 * d + c] = dPa[0];
-  dP[(int64_t)bi * 2 * d + d + c] = dPa[1];
-  __syncthreads();
-  if (ctot > 0) {
-    for (int t = c; t < 5 * H + G; t += blockDim.x) {
-      if (t < 4 * H) atomicAdd(&gw[po[P_EE_W1] + t], acc[t]);
-      else if (t < 5 * H) atomicAdd(&gw[po[P_EE_B1] + t - 4 * H], acc[t]);
-      else atomicAdd(&gw[po[P_EE_SIGMA] + t - 5 * H], acc[t]);
+  int cur = -1;   // the electron whose dP is being summed
+  auto flush = [&](int e) {   // dP rows of electrons cur .. e - 1 (those without pairs stay zero)
+    for (; cur < e; ++cur) {
+      if (cur < 0) continue;
+      const int64_t bi = block_index(w, i0 + cur, Wc, n, n_up);
+      dP[bi * 2 * d + c] = dPa[0];
+      dP[bi * 2 * d + d + c] = dPa[1];
+      dPa[0] = dPa[1] = T(0);
     }
+  };
+  flush(0);
+  for (int b0 = 0; b0 < total; b0 += kGradPairs) {
+    const int nb = min(kGradPairs, total - b0);
+    if (c < nb) {
+      int e = 0;
+      while (b0 + c >= s_off[e + 1]) ++e;
+      const int s = b0 + c - s_off[e], i = i0 + e;
+      const int j = idx[((int64_t)w * n + i) * K + s];
+      const double dd[3] = {rw[3 * i] - rw[3 * j], rw[3 * i + 1] - rw[3 * j + 1], rw[3 * i + 2] - rw[3 * j + 2]};
+      s_e[c] = e;
+      s_j[c] = block_index(w, j, Wc, n, n_up);
+      s_a[c] = s < s_par[e] ? 0 : 1;
 #pragma unroll
-    for (int h = 0; h < H; ++h) atomicAdd(&gw[po[P_EE_W2] + h * d + c], gW2[h]);
+      for (int t = 0; t < 3; ++t) m.f->dv[c][t] = T(dd[t]);
+      m.f->r[c] = T(sqrt(dd[0] * dd[0] + dd[1] * dd[1] + dd[2] * dd[2]));
+    }
+    __syncthreads();
+    for (int e = c; e < nb * kPairFeat; e += blockDim.x) {
+      const int q = e / kPairFeat, k = e - q * kPairFeat;
+      m.f->feat[q].f[k][0] =
+          pair_feature<T, W>(k, m.f->dv[q], m.f->r[q], p.ee_w1, p.ee_b1, p.ee_sigma, T(cut)).v;
+    }
+    __syncthreads();
+    {
+      const FilterWeights<T, W> fw(p.ee_w2, p.ee_wenv, d, c);
+      for (int q = 0; q < nb; ++q) {
+        const int e = s_e[q], a = s_a[q];
+        if (e != cur) flush(e);
+        const int64_t bi = block_index(w, i0 + e, Wc, n, n_up), bj = s_j[q];
+        const T delta = dH1[bi * d + c];
+        T gv, ev;
+        fw.factors(m.f->feat[q], gv, ev);
+        T z = PQ[bi * ld4 + (int64_t)a * d + c] + PQ[bj * ld4 + 2 * (int64_t)d + (int64_t)a * d + c] +
+              T(p.msg_b[a * d + c]);
+        T fk[4];
+        ld_vec<T, 4>(fk, &m.f->feat[q].f[H + G][0]);
 #pragma unroll
-    for (int g = 0; g < G; ++g) atomicAdd(&gw[po[P_EE_WENV] + g * d + c], gWe[g]);
+        for (int k = 0; k < 4; ++k) z += fk[k] * T(p.msg_w[((int64_t)a * (2 * d + 4) + 2 * d + k) * d + c]);
+        T f, f1, f2;
+        silu3<T>(z, f, f1, f2);
+        const T gam = gv * ev, dgam = delta * f, dz = delta * gam * f1;
+        m.se[q * d + c] = dgam * ev;
+        m.sg[q * d + c] = dgam * gv;
+        atomicAdd(&dQ[bj * 2 * d + (int64_t)a * d + c], dz);
+        const T d0 = a ? T(0) : dz, d1 = a ? dz : T(0);
+        dPa[0] += d0;
+        dPa[1] += d1;
+        gB[0] += d0;
+        gB[1] += d1;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+          gWc[0][k] += fk[k] * d0;
+          gWc[1][k] += fk[k] * d1;
+        }
+      }
+    }
+    filter_grad_batch<T, W>(m, nb, d, p.ee_w1, p.ee_b1, p.ee_w2, p.ee_wenv, p.ee_sigma);
+  }
+  flush(ne);
+  if (total > 0) {
+    for (int t = c; t < 5 * H + G; t += blockDim.x) {
+      if (t < 4 * H) atomicAdd(&gw[po[P_EE_W1] + t], m.f->acc[t]);
+      else if (t < 5 * H) atomicAdd(&gw[po[P_EE_B1] + t - 4 * H], m.f->acc[t]);
+      else atomicAdd(&gw[po[P_EE_SIGMA] + t - 5 * H], m.f->acc[t]);
+    }
+    for (int h = 0; h < H; ++h) atomicAdd(&gw[po[P_EE_W2] + h * d + c], m.col[h * d + c]);
+    for (int g = 0; g < G; ++g) atomicAdd(&gw[po[P_EE_WENV] + g * d + c], m.col[(H + g) * d + c]);
 #pragma unroll
     for (int a = 0; a < 2; ++a) {
       atomicAdd(&gw[po[P_MSG_B] + a * d + c], gB[a]);
@@ -361,73 +439,97 @@ __global__ void msg_bwd_kernel(int Wc, int n, int n_up, int d, int K, const doub
   }
 }
 
-// Electron-nucleus filter backward: ds = d/ds_i (the filter sum).  One CTA
-// per electron, blockDim == d.
+// Electron-nucleus filter backward: ds = d/ds_i (the filter sum).  One CTA per
+// (walker, nucleus, segment of seg <= kGradSeg electrons), blockDim == d: the
+// nucleus's own weights (h^nuc_m, W_1m, b_1m) are summed within the CTA.
+constexpr int kGradSeg = 256;
 template <typename T, typename W>
-__global__ void en_bwd_kernel(int Wc, int n, int n_up, int N, int d, const double* __restrict__ r,
-                              const double* __restrict__ R, double cnuc, Params<W> p, const T* __restrict__ dS,
-                              T* __restrict__ grad, int64_t P, const int64_t* __restrict__ po) {
+__global__ void __launch_bounds__(256, sizeof(T) == 4 ? 2 : 1) en_bwd_kernel(
+    int Wc, int n, int n_up, int N, int d, int seg, const double* __restrict__ r, const double* __restrict__ R,
+    double cnuc, Params<W> p, const T* __restrict__ dS, T* __restrict__ grad, int64_t P,
+    const int64_t* __restrict__ po) {
   constexpr int H = kEdgeHidden, G = kGauss;
-  __shared__ FL3<T> feat[H + G + 4];
-  __shared__ T part[32 * 48];
-  __shared__ T red48[48];
-  const int blk = blockIdx.x;
-  const int w = blk / n, i = blk % n;
+  extern __shared__ __align__(16) unsigned char fg_smem[];
+  __shared__ int s_list[kGradSeg], s_cnt, s_b[kGradPairs];
+  const int nseg = (n + seg - 1) / seg;
+  const int m_ = (int)(blockIdx.x / nseg % N), w = (int)(blockIdx.x / nseg / N);
+  const int i0 = (int)(blockIdx.x % nseg) * seg, i1 = min(n, i0 + seg);
   const int c = threadIdx.x;
+  const FilterGradMem<T> m(fg_smem, d);
   T* gw = grad + (int64_t)w * P;
-  T w2[H], we[G], wf[4];
-#pragma unroll
-  for (int h = 0; h < H; ++h) w2[h] = T(p.en_w2[h * d + c]);
-#pragma unroll
-  for (int g = 0; g < G; ++g) we[g] = T(p.en_wenv[g * d + c]);
-#pragma unroll
-  for (int k = 0; k < 4; ++k) wf[k] = T(p.en_wfeat[k * d + c]);
-  T gW2[H], gWe[G], gWf[4];
-#pragma unroll
-  for (int h = 0; h < H; ++h) gW2[h] = T(0);
-#pragma unroll
-  for (int g = 0; g < G; ++g) gWe[g] = T(0);
+  const double Rm[3] = {R[3 * m_], R[3 * m_ + 1], R[3 * m_ + 2]};
+  const double* rw = r + (int64_t)w * n * 3;
+  const W *w1 = p.en_w1 + (int64_t)m_ * 4 * H, *b1 = p.en_b1 + (int64_t)m_ * H;
+  if (c < 32) {   // electrons of the segment within the cutoff, ascending
+    int have = 0;
+    for (int j0 = i0; j0 < i1; j0 += 32) {
+      const int i = j0 + c;
+      bool in = false;
+      if (i < i1) {
+        const double d0 = rw[3 * i] - Rm[0], d1 = rw[3 * i + 1] - Rm[1], d2 = rw[3 * i + 2] - Rm[2];
+        in = sqrt(d0 * d0 + d1 * d1 + d2 * d2) < cnuc;
+      }
+      const unsigned bal = __ballot_sync(0xffffffffu, in);
+      if (in) s_list[have + __popc(bal & ((1u << c) - 1u))] = i;
+      have += __popc(bal);
+    }
+    if (c == 0) s_cnt = have;
+  }
+  __syncthreads();
+  const int total = s_cnt;
+  if (total == 0) return;
+  T gWf[4], gE = T(0);
 #pragma unroll
   for (int k = 0; k < 4; ++k) gWf[k] = T(0);
-  const T ds = dS[(int64_t)block_index(w, i, Wc, n, n_up) * d + c];
-  const double* ri = r + ((int64_t)w * n + i) * 3;
-  bool any = false;
-  for (int m = 0; m < N; ++m) {
-    double ddv[3] = {ri[0] - R[3 * m], ri[1] - R[3 * m + 1], ri[2] - R[3 * m + 2]};
-    const double rr = sqrt(ddv[0] * ddv[0] + ddv[1] * ddv[1] + ddv[2] * ddv[2]);
-    if (!(rr < cnuc)) continue;
-    any = true;
-    T dv[3] = {T(ddv[0]), T(ddv[1]), T(ddv[2])};
+  const T emb = T(p.nuc_emb[(int64_t)m_ * d + c]);
+  for (int b0 = 0; b0 < total; b0 += kGradPairs) {
+    const int nb = min(kGradPairs, total - b0);
+    if (c < nb) {
+      const int i = s_list[b0 + c];
+      const double dd[3] = {rw[3 * i] - Rm[0], rw[3 * i + 1] - Rm[1], rw[3 * i + 2] - Rm[2]};
+      s_b[c] = block_index(w, i, Wc, n, n_up);
+#pragma unroll
+      for (int t = 0; t < 3; ++t) m.f->dv[c][t] = T(dd[t]);
+      m.f->r[c] = T(sqrt(dd[0] * dd[0] + dd[1] * dd[1] + dd[2] * dd[2]));
+    }
     __syncthreads();
-    pair_features_to_smem<T, W>(dv, T(rr), p.en_w1 + (int64_t)m * 4 * H, p.en_b1 + (int64_t)m * H, p.en_sigma,
-                                T(cnuc), feat);
+    for (int e = c; e < nb * kPairFeat; e += blockDim.x) {
+      const int q = e / kPairFeat, k = e - q * kPairFeat;
+      m.f->feat[q].f[k][0] = pair_feature<T, W>(k, m.f->dv[q], m.f->r[q], w1, b1, p.en_sigma, T(cnuc)).v;
+    }
     __syncthreads();
-    T gv = T(0), ev = T(0), fv = T(p.nuc_emb[(int64_t)m * d + c]);
+    {
+      const FilterWeights<T, W> fw(p.en_w2, p.en_wenv, d, c);
+      T wf[4];
 #pragma unroll
-    for (int h = 0; h < H; ++h) gv += feat[h].v * w2[h];
+      for (int k = 0; k < 4; ++k) wf[k] = T(p.en_wfeat[k * d + c]);
+      for (int q = 0; q < nb; ++q) {
+        const T ds = dS[(int64_t)s_b[q] * d + c];
+        T gv, ev, fk[4], fv = emb;
+        fw.factors(m.f->feat[q], gv, ev);
+        ld_vec<T, 4>(fk, &m.f->feat[q].f[H + G][0]);
 #pragma unroll
-    for (int g = 0; g < G; ++g) ev += feat[H + g].v * we[g];
+        for (int k = 0; k < 4; ++k) fv += fk[k] * wf[k];
+        const T dgam = ds * fv, dfv = ds * (gv * ev);
+        m.se[q * d + c] = dgam * ev;
+        m.sg[q * d + c] = dgam * gv;
+        gE += dfv;
 #pragma unroll
-    for (int k = 0; k < 4; ++k) fv += feat[H + G + k].v * wf[k];
-    const T gam = gv * ev;
-    const T dgam = ds * fv;
-    const T dfv = ds * gam;
-    atomicAdd(&gw[po[P_NUC_EMB] + (int64_t)m * d + c], dfv);
-#pragma unroll
-    for (int k = 0; k < 4; ++k) gWf[k] += feat[H + G + k].v * dfv;
-    filter_bwd<false, T, W>(feat, dv, T(rr), T(cnuc), p.en_w1 + (int64_t)m * 4 * H, p.en_b1 + (int64_t)m * H,
-                     p.en_sigma, w2, we, gv, ev, dgam, gW2, gWe, part, red48, nullptr,
-                     gw + po[P_EN_W1] + (int64_t)m * 4 * H, gw + po[P_EN_B1] + (int64_t)m * H,
-                     gw + po[P_EN_SIGMA]);
+        for (int k = 0; k < 4; ++k) gWf[k] += fk[k] * dfv;
+      }
+    }
+    filter_grad_batch<T, W>(m, nb, d, w1, b1, p.en_w2, p.en_wenv, p.en_sigma);
   }
-  if (any) {
-#pragma unroll
-    for (int h = 0; h < H; ++h) atomicAdd(&gw[po[P_EN_W2] + h * d + c], gW2[h]);
-#pragma unroll
-    for (int g = 0; g < G; ++g) atomicAdd(&gw[po[P_EN_WENV] + g * d + c], gWe[g]);
-#pragma unroll
-    for (int k = 0; k < 4; ++k) atomicAdd(&gw[po[P_EN_WFEAT] + k * d + c], gWf[k]);
+  atomicAdd(&gw[po[P_NUC_EMB] + (int64_t)m_ * d + c], gE);
+  for (int t = c; t < 5 * H + G; t += blockDim.x) {
+    if (t < 4 * H) atomicAdd(&gw[po[P_EN_W1] + (int64_t)m_ * 4 * H + t], m.f->acc[t]);
+    else if (t < 5 * H) atomicAdd(&gw[po[P_EN_B1] + (int64_t)m_ * H + t - 4 * H], m.f->acc[t]);
+    else atomicAdd(&gw[po[P_EN_SIGMA] + t - 5 * H], m.f->acc[t]);
   }
+  for (int h = 0; h < H; ++h) atomicAdd(&gw[po[P_EN_W2] + h * d + c], m.col[h * d + c]);
+  for (int g = 0; g < G; ++g) atomicAdd(&gw[po[P_EN_WENV] + g * d + c], m.col[(H + g) * d + c]);
+#pragma unroll
+  for (int k = 0; k < 4; ++k) atomicAdd(&gw[po[P_EN_WFEAT] + k * d + c], gWf[k]);
 }
 
 // GLU gate backward: dZg = dP * zv * SiLU'(zg), dZv = dP * SiLU(zg).

@@ -396,7 +396,19 @@ struct Runner {
       const double* r = a.r + w0 * n * 3;
       const int nb = wc * n;
       T* g = G + w0 * P;
-      cudaMemsetAsync(g, 0, sizeof(T) * (size_t)wc * P, s);
+      // every entry is written once or starts from zero and is added to: all
+      // but the orbital and envelope weights (three quarters of a C26H24 row)
+      // of a spin that has electrons, whose products write every entry
+      auto zero_cols = [&](int64_t from, int64_t to) {
+        if (to > from) cudaMemset2DAsync(g + from, sizeof(T) * P, 0, sizeof(T) * (to - from), wc, s);
+      };
+      zero_cols(0, po[P_ORB_W]);
+      zero_cols(po[P_ENV_SIGMA], P);
+      for (int sp = 0; sp < 2; ++sp)
+        if ((sp ? n_dn : n_up) == 0) {
+          zero_cols(po[P_ORB_W] + sp * Dn * d, po[P_ORB_W] + (sp + 1) * Dn * d);
+          zero_cols(po[P_ENV_PI] + sp * Dn * NE, po[P_ENV_PI] + (sp + 1) * Dn * NE);
+        }
       GradBufs<T> B;
       GradBufs<T>::carve(at<unsigned char>(pl.gradws), &B, pl.Wc, n, d, L, D, J, R, RD, NE);
       int32_t* idx = at<int32_t>(pl.idx);
@@ -406,18 +418,14 @@ struct Runner {
       int64_t* boff = at<int64_t>(pl.blk_off);
       int64_t* rng = at<int64_t>(pl.ranges);
       const double c = sys->cutoff;
-      // segments of a walker's electrons in block order: up [w n_up, +n_up), down [Wc n_up + w n_dn, +n_dn)
-      auto tn_w = [&](const T* X, int64_t ldx, int Na, const T* Y, int64_t ldy, int Nb, int64_t goff, int64_t ldc,
-                      bool acc) {
-        tn_batched<T>(s, wc, Na, Nb, n_up, X, ldx, n_up * ldx, Y, ldy, n_up * ldy, g + goff, ldc, P, acc);
-        tn_batched<T>(s, wc, Na, Nb, n_dn, X + (int64_t)wc * n_up * ldx, ldx, n_dn * ldx,
-                      Y + (int64_t)wc * n_up * ldy, ldy, n_dn * ldy, g + goff, ldc, P, true);
-        launches += 2;
+      const SpinRows el = spin_rows(wc, n_up, n_dn), wr = walker_rows();
+      auto tn_w = [&](const T* X, int64_t ldx, int Na, const T* Y, int64_t ldy, int Nb, int64_t goff, int64_t ldc) {
+        tn_batched<T>(s, wc, Na, Nb, el, X, ldx, Y, ldy, g + goff, ldc, P);
+        launches += 1;
       };
       auto colsum_w = [&](const T* Y, int64_t ldy, int Nb, int64_t goff) {
-        colsum_batched<T>(s, wc, Nb, n_up, Y, ldy, n_up * ldy, g + goff, P, true);
-        colsum_batched<T>(s, wc, Nb, n_dn, Y + (int64_t)wc * n_up * ldy, ldy, n_dn * ldy, g + goff, P, true);
-        launches += 2;
+        colsum_batched<T>(s, wc, Nb, el, Y, ldy, g + goff, P);
+        launches += 1;
       };
       // ---- forward (value rows: one row per electron block) ----
       mark("neighbors", 3);
@@ -537,19 +545,16 @@ struct Runner {
       for (int sp = 0; sp < 2; ++sp) {
         const int64_t rb = sp ? upv : 0, re = sp ? nb : upv;
         if (re <= rb) continue;
-        const int ns = sp ? n_dn : n_up;
-        for (int dd = 0; dd < D; ++dd) {
-          const int64_t wo = po[P_ORB_W] + ((int64_t)sp * D + dd) * d * n;
-          const int64_t pi_o = po[P_ENV_PI] + ((int64_t)sp * D + dd) * n * NE;
-          const T* Xs = h + rb * d;
-          tn_batched<T>(s, wc, d, n, ns, Xs, d, (int64_t)ns * d, B.dO + rb * Dn + dd * n, Dn, (int64_t)ns * Dn,
-                        g + wo, n, P, false);
-          tn_batched<T>(s, wc, n, NE, ns, B.dF + rb * Dn + dd * n, Dn, (int64_t)ns * Dn, Qf + rb * NE, NE,
-                        (int64_t)ns * NE, g + pi_o, NE, P, false);
+        const SpinRows run = one_spin(sp ? n_dn : n_up);
+        const int64_t wo = po[P_ORB_W] + (int64_t)sp * Dn * d, pi_o = po[P_ENV_PI] + (int64_t)sp * Dn * NE;
+        // all determinants of the spin: d W_d = h^T dO_d, d pi_d = dF_d^T q
+        tn_batched<T>(s, wc, d, n, run, h + rb * d, d, B.dO + rb * Dn, Dn, g + wo, n, P, D, 0, n, (int64_t)d * n);
+        tn_batched<T>(s, wc, n, NE, run, B.dF + rb * Dn, Dn, Qf + rb * NE, NE, g + pi_o, NE, P, D, n, 0,
+                      (int64_t)n * NE);
+        for (int dd = 0; dd < D; ++dd)
           gemm<T>(s, B.dO + dd * n, Dn, p.orb_w + ((int64_t)sp * D + dd) * d * n, n, true, B.dH, d, rb, re, nullptr,
                   re - rb, d, n, 1, 0, 0, 0, true);
-          launches += 3;
-        }
+        launches += 2 + D;
         gemm<T>(s, B.dF, Dn, p.env_pi + (int64_t)sp * Dn * NE, NE, false, B.dQf, NE, rb, re, nullptr, re - rb, NE,
                 (int)Dn);
         ++launches;
@@ -563,16 +568,16 @@ struct Runner {
                                   {po[P_JM2_W1], po[P_JM2_B1], po[P_JM2_W2], po[P_JM2_B2], po[P_JM2_W3], po[P_JM2_B3]}};
         for (int k = 0; k < 2; ++k) {
           jseed_kernel<T><<<wc, 256, 0, s>>>(wc, n, n_up, J, F[1], p.jm2_b3, jw3[k], k, B.df, B.dY2);
-          tn_w(B.df, 1, 1, B.JA2[k], J, J, jo[k][4], J, true);
+          tn_w(B.df, 1, 1, B.JA2[k], J, J, jo[k][4], J);
           colsum_w(B.df, 1, 1, jo[k][5]);
           silu_bwd_kernel<T, T><<<(unsigned)(((int64_t)nb * J + 255) / 256), 256, 0, s>>>(nb, J, B.dY2, J, B.JZ2[k], J,
                                                                                          jb2[k], B.dZ2, J);
-          tn_w(B.JA1[k], J, J, B.dZ2, J, J, jo[k][2], J, true);
+          tn_w(B.JA1[k], J, J, B.dZ2, J, J, jo[k][2], J);
           colsum_w(B.dZ2, J, J, jo[k][3]);
           gemm<T>(s, B.dZ2, J, jw2[k], J, true, B.dA1, J, 0, nb, nullptr, nb, J, J);
           silu_bwd_kernel<T, T><<<(unsigned)(((int64_t)nb * J + 255) / 256), 256, 0, s>>>(nb, J, B.dA1, J, B.JZ1[k], J,
                                                                                          jb1[k], B.dZ1, J);
-          tn_w(h, d, d, B.dZ1, J, J, jo[k][0], J, true);
+          tn_w(h, d, d, B.dZ1, J, J, jo[k][0], J);
           colsum_w(B.dZ1, J, J, jo[k][1]);
           gemm<T>(s, B.dZ1, J, jw1[k], J, true, B.dH, d, 0, nb, nullptr, nb, d, J, 1, 0, 0, 0, true);
           launches += 5;
@@ -585,26 +590,27 @@ struct Runner {
         cudaMemsetAsync(B.dV, 0, sizeof(T) * (size_t)wc * RD, s);
         for (int k = 0; k < 2; ++k) {
           vseed_kernel<T><<<wc, 256, 0, s>>>(J, Gv[1], p.ja2_b3, vw3[k], k, B.dfv, B.dVY2);
-          tn_batched<T>(s, wc, 1, J, 1, B.dfv, 1, 1, B.VA2[k], J, J, g + vo[k][4], J, P, true);
-          colsum_batched<T>(s, wc, 1, 1, B.dfv, 1, 1, g + vo[k][5], P, true);
+          tn_batched<T>(s, wc, 1, J, wr, B.dfv, 1, B.VA2[k], J, g + vo[k][4], J, P);
+          colsum_batched<T>(s, wc, 1, wr, B.dfv, 1, g + vo[k][5], P);
           silu_bwd_kernel<T, T><<<(unsigned)(((int64_t)wc * J + 255) / 256), 256, 0, s>>>(wc, J, B.dVY2, J, B.VZ2[k],
                                                                                          J, vb2[k], B.dVZ2, J);
-          tn_batched<T>(s, wc, J, J, 1, B.VA1[k], J, J, B.dVZ2, J, J, g + vo[k][2], J, P, true);
-          colsum_batched<T>(s, wc, J, 1, B.dVZ2, J, J, g + vo[k][3], P, true);
+          tn_batched<T>(s, wc, J, J, wr, B.VA1[k], J, B.dVZ2, J, g + vo[k][2], J, P);
+          colsum_batched<T>(s, wc, J, wr, B.dVZ2, J, g + vo[k][3], P);
           gemm<T>(s, B.dVZ2, J, vw2[k], J, true, B.dVA1, J, 0, wc, nullptr, wc, J, J);
           silu_bwd_kernel<T, T><<<(unsigned)(((int64_t)wc * J + 255) / 256), 256, 0, s>>>(wc, J, B.dVA1, J, B.VZ1[k],
                                                                                          J, vb1[k], B.dVZ1, J);
-          tn_batched<T>(s, wc, RD, J, 1, V, RD, RD, B.dVZ1, J, J, g + vo[k][0], J, P, true);
-          colsum_batched<T>(s, wc, J, 1, B.dVZ1, J, J, g + vo[k][1], P, true);
+          tn_batched<T>(s, wc, RD, J, wr, V, RD, B.dVZ1, J, g + vo[k][0], J, P);
+          colsum_batched<T>(s, wc, J, wr, B.dVZ1, J, g + vo[k][1], P);
           gemm<T>(s, B.dVZ1, J, vw1[k], J, true, B.dV, RD, 0, wc, nullptr, wc, RD, J, 1, 0, 0, 0, true);
           launches += 11;
         }
         const size_t absm = (size_t)(2 * n * R + 3 * R) * sizeof(T);
         const int bt = ((RD + 31) / 32) * 32;
         att_bwd_kernel<T><<<wc, bt, absm, s>>>(wc, n, n_up, R, dr, B.SU, ldsu, B.dV, B.dSU);
-        tn_w(B.dSU, ldsu, R, h, d, d, po[P_ATT_Q], d, true);
-        for (int rr = 0; rr < R; ++rr)
-          tn_w(h, d, d, B.dSU + R + rr * dr, ldsu, dr, po[P_ATT_WV] + (int64_t)rr * d * dr, dr, true);
+        tn_w(B.dSU, ldsu, R, h, d, d, po[P_ATT_Q], d);
+        // the R value projections side by side: columns of register r to its own [d][dr] block
+        tn_batched<T>(s, wc, d, RD, el, h, d, B.dSU + R, ldsu, g + po[P_ATT_WV], dr, P, 1, 0, 0, 0, dr,
+                      (int64_t)d * dr);
         gemm<T>(s, B.dSU, ldsu, p.att_q, d, false, B.dH, d, 0, nb, nullptr, nb, d, R, 1, 0, 0, 0, true);
         for (int rr = 0; rr < R; ++rr)
           gemm<T>(s, B.dSU + R + rr * dr, ldsu, p.att_wv + (int64_t)rr * d * dr, dr, true, B.dH, d, 0, nb, nullptr, nb,
@@ -623,7 +629,7 @@ struct Runner {
         const T* z = B.ZL + (int64_t)l * nb * d;
         silu_bwd_kernel<T, T><<<(unsigned)(((int64_t)nb * d + 255) / 256), 256, 0, s>>>(nb, d, B.dH, d, z, d,
                                                                                        p.mlp_b + (int64_t)l * d, B.dZ, d);
-        tn_w(hin, d, d, B.dZ, d, d, po[P_MLP_W] + (int64_t)l * d * d, d, true);
+        tn_w(hin, d, d, B.dZ, d, d, po[P_MLP_W] + (int64_t)l * d * d, d);
         colsum_w(B.dZ, d, d, po[P_MLP_B] + (int64_t)l * d);
         gemm<T>(s, B.dZ, d, p.mlp_w + (int64_t)l * d * d, d, true, B.dH, d, 0, nb, nullptr, nb, d, d, 1, 0, 0, 0, true);
         launches += 2;
@@ -631,12 +637,22 @@ struct Runner {
       // message passing (dH now holds d/dh^1)
       mark("bwd_msg", 0);
       cudaMemsetAsync(B.dQm, 0, sizeof(T) * (size_t)nb * 2 * d, s);
-      msg_bwd_kernel<T, T><<<nb, d, 0, s>>>(wc, n, n_up, d, K, r, c, p, idx, cnt, PQ, B.dH, B.dPm, B.dQm, g, P, pod);
+      {
+        // electrons of a CTA: as many as leave four CTAs per SM (the CTA's
+        // weight sums are added to the walker's row once)
+        int epc = (int)((int64_t)nb / (152 * 4));
+        epc = epc < 1 ? 1 : (epc > kGradElectrons ? kGradElectrons : epc);
+        if (epc > n) epc = n;
+        const unsigned ctas = (unsigned)(wc * ((n + epc - 1) / epc));
+        msg_bwd_kernel<T, T><<<ctas, d, filter_grad_smem<T>(d), s>>>(wc, n, n_up, d, K, epc, r, c, p, idx, cnt, PQ,
+                                                                     B.dH, B.dPm, B.dQm, g, P, pod);
+        launches += 1;
+      }
       cudaMemcpyAsync(B.dH0, B.dH, sizeof(T) * (size_t)nb * d, cudaMemcpyDeviceToDevice, s);
       for (int al = 0; al < 2; ++al) {
         const int64_t wa = po[P_MSG_W] + (int64_t)al * (2 * d + 4) * d;
-        tn_w(H0, d, d, B.dPm + (int64_t)al * d, 2 * d, d, wa, d, true);
-        tn_w(H0, d, d, B.dQm + (int64_t)al * d, 2 * d, d, wa + (int64_t)d * d, d, true);
+        tn_w(H0, d, d, B.dPm + (int64_t)al * d, 2 * d, d, wa, d);
+        tn_w(H0, d, d, B.dQm + (int64_t)al * d, 2 * d, d, wa + (int64_t)d * d, d);
         gemm<T>(s, B.dPm + (int64_t)al * d, 2 * d, p.msg_w + (int64_t)al * (2 * d + 4) * d, d, true, B.dH0, d, 0, nb,
                 nullptr, nb, d, d, 1, 0, 0, 0, true);
         gemm<T>(s, B.dQm + (int64_t)al * d, 2 * d, p.msg_w + (int64_t)al * (2 * d + 4) * d + (int64_t)d * d, d, true,
@@ -647,10 +663,10 @@ struct Runner {
       // GLU and LayerNorm
       mark("bwd_glu", 0);
       gemm<T>(s, B.dH0, d, p.glu_wo, d, true, B.dP5, d, 0, nb, nullptr, nb, d, d);
-      tn_w(P5, d, d, B.dH0, d, d, po[P_GLU_WO], d, true);
+      tn_w(P5, d, d, B.dH0, d, d, po[P_GLU_WO], d);
       gate_bwd_kernel<T><<<(unsigned)(((int64_t)nb * d + 255) / 256), 256, 0, s>>>(nb, d, Z5, B.dP5, B.dZ5);
-      tn_w(Y5, d, d, B.dZ5, 2 * d, d, po[P_GLU_WG], d, true);
-      tn_w(Y5, d, d, B.dZ5 + d, 2 * d, d, po[P_GLU_WV], d, true);
+      tn_w(Y5, d, d, B.dZ5, 2 * d, d, po[P_GLU_WG], d);
+      tn_w(Y5, d, d, B.dZ5 + d, 2 * d, d, po[P_GLU_WV], d);
       gemm<T>(s, B.dZ5, 2 * d, p.glu_wg, d, true, B.dY5, d, 0, nb, nullptr, nb, d, d);
       gemm<T>(s, B.dZ5 + d, 2 * d, p.glu_wv, d, true, B.dY5, d, 0, nb, nullptr, nb, d, d, 1, 0, 0, 0, true);
       ln_bwd_kernel<T, T><<<nb, d, 0, s>>>(d, S5, B.dY5, p.ln_gamma, B.dS5, B.dyx);
@@ -659,7 +675,13 @@ struct Runner {
       launches += 6;
       // electron-nucleus filters
       mark("bwd_en", 1);
-      en_bwd_kernel<T, T><<<nb, d, 0, s>>>(wc, n, n_up, N, d, r, sys->nuc_pos, sys->cutoff_nuc, p, B.dS5, g, P, pod);
+      {
+        int seg = kGradSeg;   // electrons of a CTA: shorter segments until four CTAs per SM exist
+        while (seg > kGradPairs && (int64_t)wc * N * ((n + seg - 1) / seg) < 152 * 4) seg /= 2;
+        const unsigned ctas = (unsigned)((int64_t)wc * N * ((n + seg - 1) / seg));
+        en_bwd_kernel<T, T><<<ctas, d, filter_grad_smem<T>(d), s>>>(wc, n, n_up, N, d, seg, r, sys->nuc_pos,
+                                                                    sys->cutoff_nuc, p, B.dS5, g, P, pod);
+      }
       check("bwd en");
     }
     mark("end", 0);
@@ -1638,6 +1660,8 @@ inline int set_smem_limits() {
   raise((const void*)gj_inverse_kernel<float, T>);
   raise((const void*)gj_inverse_pre_kernel<float, T>);
   raise((const void*)mcmc_att_kernel<T>);
+  raise((const void*)msg_bwd_kernel<T, T>);
+  raise((const void*)en_bwd_kernel<T, T>);
   if constexpr (sizeof(T) == 4) raise((const void*)inverse_panel_kernel<LT, T, T>);
   raise((const void*)mcmc_woodbury_kernel<T>);
   raise((const void*)mcmc_woodbury_panel_kernel<T, 4>);
