@@ -19,10 +19,13 @@ int gemm_bf16(cudaStream_t s, const void* A, int64_t lda, int64_t a_rows, const 
               int* err, int nc);
 
 // The same product with Bt rows [b_row0, b_row0 + N) of a weight block whose
-// components hold b_rows rows each (a slice of a larger packed matrix).
+// components hold b_rows rows each (a slice of a larger packed matrix) and
+// row stride ldb (0: K).  With groups > 1, group y multiplies columns
+// [y K, (y + 1) K) of A and Bt into the rows of C from y c_group_rows on.
 int gemm_bf16_rows(cudaStream_t s, const void* A, int64_t lda, int64_t a_rows, const void* Bt, int b_rows,
                    int b_row0, int N, int K, float* C, int64_t ldc, int64_t m_begin, int64_t m_end,
-                   const int64_t* m_range, int64_t m_cap, int* err, int nc);
+                   const int64_t* m_range, int64_t m_cap, int* err, int nc, int groups = 1, int64_t ldb = 0,
+                   int64_t c_group_rows = 0);
 
 // dst = nc-component bf16 K-major copy of a weight matrix (pack_bf16_kernel),
 // rows ldd >= K elements apart with zero padding (ldd = 0: K).

@@ -67,7 +67,7 @@ static bool make_map_c(CUtensorMap* m, const float* base, uint64_t cols, uint64_
 
 template <int STAGES, int NC>
 static int launch(cudaStream_t s, const CUtensorMap& ma, const CUtensorMap& mb, const CUtensorMap& mc,
-                  const TcArgs& g, int64_t m_cap, int nt) {
+                  const TcArgs& g, int64_t m_cap, int nt, int groups) {
   const size_t sm = tc_smem_bytes(STAGES, NC, g.BN);
   if (cudaFuncSetAttribute(tc_gemm_kernel<STAGES, NC>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm) !=
       cudaSuccess) {
@@ -83,7 +83,7 @@ static int launch(cudaStream_t s, const CUtensorMap& ma, const CUtensorMap& mb, 
   }
   const int64_t tiles = ((m_cap + BM - 1) / BM) * nt;
   const int grid = (int)(tiles < n_sm ? tiles : n_sm);
-  tc_gemm_kernel<STAGES, NC><<<grid, 192, sm, s>>>(ma, mb, mc, g);
+  tc_gemm_kernel<STAGES, NC><<<dim3(grid, groups), 192, sm, s>>>(ma, mb, mc, g);
   return cudaGetLastError() == cudaSuccess ? FIRE_OK : FIRE_ERR_CUDA;
 }
 
@@ -110,7 +110,11 @@ int gemm_bf16(cudaStream_t s, const void* A, int64_t lda, int64_t a_rows, const 
 
 int gemm_bf16_rows(cudaStream_t s, const void* A, int64_t lda, int64_t a_rows, const void* Bt, int b_rows,
                    int b_row0, int N, int K, float* C, int64_t ldc, int64_t m_begin, int64_t m_end,
-                   const int64_t* m_range, int64_t m_cap, int* err, int nc) {
+                   const int64_t* m_range, int64_t m_cap, int* err, int nc, int groups, int64_t ldb,
+                   int64_t c_group_rows) {
+  if (ldb <= 0) ldb = K;
+  if (groups < 1 || groups > 65535 || (groups > 1 && (lda < (int64_t)groups * K || ldb < (int64_t)groups * K)))
+    return FIRE_ERR_UNSUPPORTED;
   if (b_row0 < 0 || b_row0 + N > b_rows) return FIRE_ERR_UNSUPPORTED;
   if (N < 1 || K < BK || K % BK || m_cap <= 0 || nc < 1 || nc > 3) return FIRE_ERR_UNSUPPORTED;
   int stages = nc == 1 ? 4 : (nc == 2 ? 3 : 2);
@@ -137,23 +141,23 @@ int gemm_bf16_rows(cudaStream_t s, const void* A, int64_t lda, int64_t a_rows, c
   if (BN == 0) return FIRE_ERR_UNSUPPORTED;
   const int nt = (N + BN - 1) / BN;
   CUtensorMap ma, mb;
-  if (!make_map(&ma, A, (uint64_t)a_rows * nc, (uint64_t)K, (uint64_t)lda, BM)) return FIRE_ERR_CUDA;
-  if (!make_map(&mb, Bt, (uint64_t)b_rows * nc, (uint64_t)K, (uint64_t)K, (uint32_t)BN)) return FIRE_ERR_CUDA;
+  if (!make_map(&ma, A, (uint64_t)a_rows * nc, (uint64_t)K * groups, (uint64_t)lda, BM)) return FIRE_ERR_CUDA;
+  if (!make_map(&mb, Bt, (uint64_t)b_rows * nc, (uint64_t)K * groups, (uint64_t)ldb, (uint32_t)BN)) return FIRE_ERR_CUDA;
   // FIRE_TC_CSTORE=direct (diagnostic): every tile through the lanes' own stores
   CUtensorMap mc;
   memset(&mc, 0, sizeof(mc));
   const char* cs = getenv("FIRE_TC_CSTORE");
   const bool direct = cs && strcmp(cs, "direct") == 0;
   const int c_tma = (!direct && make_map_c(&mc, C, (uint64_t)N, (uint64_t)ldc)) ? 1 : 0;
-  TcArgs g{C, ldc, m_begin, m_end, m_range, N, K, BN, a_rows, b_rows, b_row0, err, c_tma};
-  if (nc == 1) return stages == 2 ? launch<2, 1>(s, ma, mb, mc, g, m_cap, nt)
-                                   : (stages == 3 ? launch<3, 1>(s, ma, mb, mc, g, m_cap, nt)
-                                                  : launch<4, 1>(s, ma, mb, mc, g, m_cap, nt));
-  if (nc == 2) return stages == 2 ? launch<2, 2>(s, ma, mb, mc, g, m_cap, nt)
-                                   : (stages == 3 ? launch<3, 2>(s, ma, mb, mc, g, m_cap, nt)
-                                                  : launch<4, 2>(s, ma, mb, mc, g, m_cap, nt));
-  return stages == 2 ? launch<2, 3>(s, ma, mb, mc, g, m_cap, nt)
-                     : (stages == 3 ? launch<3, 3>(s, ma, mb, mc, g, m_cap, nt) : launch<4, 3>(s, ma, mb, mc, g, m_cap, nt));
+  TcArgs g{C, ldc, m_begin, m_end, m_range, N, K, BN, a_rows, b_rows, b_row0, err, c_tma, c_group_rows};
+  if (nc == 1) return stages == 2 ? launch<2, 1>(s, ma, mb, mc, g, m_cap, nt, groups)
+                                   : (stages == 3 ? launch<3, 1>(s, ma, mb, mc, g, m_cap, nt, groups)
+                                                  : launch<4, 1>(s, ma, mb, mc, g, m_cap, nt, groups));
+  if (nc == 2) return stages == 2 ? launch<2, 2>(s, ma, mb, mc, g, m_cap, nt, groups)
+                                   : (stages == 3 ? launch<3, 2>(s, ma, mb, mc, g, m_cap, nt, groups)
+                                                  : launch<4, 2>(s, ma, mb, mc, g, m_cap, nt, groups));
+  return stages == 2 ? launch<2, 3>(s, ma, mb, mc, g, m_cap, nt, groups)
+                     : (stages == 3 ? launch<3, 3>(s, ma, mb, mc, g, m_cap, nt, groups) : launch<4, 3>(s, ma, mb, mc, g, m_cap, nt, groups));
 }
 
 // dst[c][n][k] = component c of src[k * lds + n] for a [K][N] source

@@ -18,6 +18,10 @@
 // L1 -> L2 path carries whole lines rather than a 16-byte piece of 32 rows
 // per store instruction (that request path, 76 % busy, bounded the product).
 //
+// Group y of the grid multiplies columns [y K, (y + 1) K) of A and B into the rows
+// c_group_rows y .. of C: independent products over slices of a long K axis,
+// which fill the SMs where one slice has fewer tiles than they are.
+//
 // Every mbarrier wait is bounded: after kSpinLimit polls the kernel records
 // an error in *err, stops issuing work, waits (bounded) for its own copies
 // and MMAs already in flight, frees its tensor memory and returns.
@@ -167,6 +171,7 @@ struct TcArgs {
   int64_t b_row0;                // first row of Bt inside each component
   int* err;                      // device error word (timeouts)
   int c_tma;                     // full tiles leave through the C tensor map
+  int64_t c_group_rows;          // rows of C between groups
 };
 
 // Split-bf16 products (Henry, Tang & Heinecke 2019): a value x is stored as
@@ -226,6 +231,8 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__
   fence_after_sync();
   const uint32_t tmem = tmem_slot;
   const int nk = g.K / BK;
+  const int k0 = (int)blockIdx.y * g.K;                       // this group's slice of K and rows of C
+  const int64_t c0r = (int64_t)blockIdx.y * g.c_group_rows;
 
   if (warp == 0 && lane == 0) {
     // TMA producer: runs ahead across tiles through the stage ring
@@ -244,8 +251,8 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__
         mbar_expect_tx(&full_bar[s], stage_bytes);
 #pragma unroll
         for (int c = 0; c < NC; ++c) {
-          tma_load_2d(sa + c * a_bytes, &mapA, &full_bar[s], kb * BK, (int)(c * g.a_comp_rows + m0));
-          tma_load_2d(sa + NC * a_bytes + c * b_bytes, &mapB, &full_bar[s], kb * BK, (int)(c * g.b_comp_rows + g.b_row0 + n0));
+          tma_load_2d(sa + c * a_bytes, &mapA, &full_bar[s], k0 + kb * BK, (int)(c * g.a_comp_rows + m0));
+          tma_load_2d(sa + NC * a_bytes + c * b_bytes, &mapB, &full_bar[s], k0 + kb * BK, (int)(c * g.b_comp_rows + g.b_row0 + n0));
         }
       }
     }
@@ -316,7 +323,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__
       // lane = row m0 + 32 q + lane: its 32 accumulator columns of a chunk go
       // straight from registers to its row of C (eight 128-bit stores)
       const int64_t row = m0 + 32 * q + lane;
-      float* crow = g.C + row * g.ldc + n0;
+      float* crow = g.C + (c0r + row) * g.ldc + n0;
       // full-row tiles through the tensor map: a 32-column box either lies
       // inside the tile or runs past N (clipped by the map); a box that
       // would reach into the next tile (BN not a multiple of 32) takes the
@@ -339,7 +346,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__
           fence_proxy_async_smem();
           __syncwarp();
           if (lane == 0) {
-            tma_store_2d(&mapC, stbuf + (size_t)q * kStoreBuf, n0 + c0, (int)(m0 + 32 * q));
+            tma_store_2d(&mapC, stbuf + (size_t)q * kStoreBuf, n0 + c0, (int)(c0r + m0 + 32 * q));
             bulk_commit();
           }
           continue;
