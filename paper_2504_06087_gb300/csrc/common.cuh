@@ -62,6 +62,19 @@ __device__ __forceinline__ void ld_vec(T (&v)[VN], const T* p) {
   }
 }
 
+// c += a * b for a pair of accumulators: one packed instruction for float32 (two
+// lanes, each rounded like fmaf), which leaves the issue slots of the other
+// half to the shared-memory loads.
+__device__ __forceinline__ void fma_pair(float& c0, float& c1, float a, float b0, float b1) {
+  asm("{\n .reg .b64 x, y, z;\n mov.b64 x, {%2, %2};\n mov.b64 y, {%3, %4};\n mov.b64 z, {%0, %1};\n"
+      " fma.rn.f32x2 z, x, y, z;\n mov.b64 {%0, %1}, z;\n}"
+      : "+f"(c0), "+f"(c1) : "f"(a), "f"(b0), "f"(b1));
+}
+__device__ __forceinline__ void fma_pair(double& c0, double& c1, double a, double b0, double b1) {
+  c0 = fma(a, b0, c0);
+  c1 = fma(a, b1, c1);
+}
+
 // SiLU and its first two derivatives: s = logistic(x),
 // f = x s, f' = s (1 + x (1 - s)), f'' = s (1 - s) (2 + x (1 - 2 s)).
 template <typename T>

@@ -69,12 +69,13 @@ constexpr int kPairFeat = kEdgeHidden + kGauss + 4;
 
 // Features of one pair in shared memory.  NC = 1: the values, so a thread
 // reads four features with one 128-bit broadcast.  NC = 5: value, Laplacian
-// and three tangents of a feature side by side (an array per component, read
-// four features at a time, measured 2-6 % slower: the sums issue as many
-// multiply-adds, and the loads are not what bounds them).
+// and three tangents of a feature side by side, in float32 on 32 bytes: two
+// loads and, with packed multiply-adds on (value, Laplacian) and the first two
+// tangents, three multiply-adds per feature instead of five of each.
 template <typename T, int NC>
 struct alignas(16) PairFeat {
-  T f[kPairFeat][NC];
+  static constexpr int S = NC == 5 && sizeof(T) == 4 ? 8 : NC;
+  T f[kPairFeat][S];
 };
 template <int NC, typename T>
 __device__ __forceinline__ void put_feature(PairFeat<T, NC>& o, int k, const FL3<T>& v) {
@@ -96,11 +97,37 @@ __device__ __forceinline__ void feat_dot(const PairFeat<T, NC>& q, int k0, const
 #pragma unroll
       for (int i = 0; i < 4; ++i) acc[0] += v[i] * w[k + i];
     }
+  } else if constexpr (sizeof(T) == 4) {
+#pragma unroll
+    for (int k = 0; k < COUNT; ++k) {
+      T v[4];
+      ld_vec<T, 4>(v, &q.f[k0 + k][0]);
+      const T z = q.f[k0 + k][4];
+      fma_pair(acc[0], acc[1], w[k], v[0], v[1]);
+      fma_pair(acc[2], acc[3], w[k], v[2], v[3]);
+      acc[4] = fma(z, w[k], acc[4]);
+    }
   } else {
 #pragma unroll
     for (int k = 0; k < COUNT; ++k)
 #pragma unroll
       for (int c = 0; c < NC; ++c) acc[c] += q.f[k0 + k][c] * w[k];
+  }
+}
+// Item e of nbat kPairFeat features as (pair q, feature k), the hidden units
+// of all pairs first, then the Gaussians, then e-bar: a warp's items are of one
+// kind (with a pair's features in a row every warp ran all three formulas).
+__device__ __forceinline__ void feature_item(int e, int nbat, int& q, int& k) {
+  const int nh = nbat * kEdgeHidden, ng = nbat * kGauss;
+  if (e < nh) {
+    q = e / kEdgeHidden;
+    k = e % kEdgeHidden;
+  } else if (e < nh + ng) {
+    q = (e - nh) / kGauss;
+    k = kEdgeHidden + (e - nh) % kGauss;
+  } else {
+    q = (e - nh - ng) / 4;
+    k = kEdgeHidden + kGauss + (e - nh - ng) % 4;
   }
 }
 template <typename T>
@@ -172,7 +199,8 @@ __global__ void __launch_bounds__(kFilterThreads<T>) en_filter_kernel(int Wc, in
     }
     __syncthreads();
     for (int e = threadIdx.x; e < nbat * kPairFeat; e += blockDim.x) {
-      const int q = e / kPairFeat, k = e - q * kPairFeat;
+      int q, k;
+      feature_item(e, nbat, q, k);
       const int m = s_m[q];
       put_feature<NC, T>(featb[q], k,
                          pair_feature<T, W>(k, s_dv[q], s_r[q], p.en_w1 + (int64_t)m * 4 * H,
@@ -391,7 +419,8 @@ __global__ void __launch_bounds__(kFilterThreads<T>) msg_kernel(int Wc, int n, i
     }
     __syncthreads();
     for (int e = threadIdx.x; e < nbat * kPairFeat; e += blockDim.x) {
-      const int q = e / kPairFeat, k = e - q * kPairFeat;
+      int q, k;
+      feature_item(e, nbat, q, k);
       put_feature<NC, T>(featb[q], k, pair_feature<T, W>(k, s_dv[q], s_r[q], p.ee_w1, p.ee_b1, p.ee_sigma, T(cut)));
     }
     __syncthreads();

@@ -32,19 +32,6 @@ struct GemmArgs {
   int va, vb, vc;                // 16-byte loads of A and of B, 16-byte stores of C
 };
 
-// c += a * b for a pair of columns: one packed instruction for float32 (two
-// lanes, each rounded like fmaf), which leaves the issue slots of the other
-// half to the shared-memory loads.
-__device__ __forceinline__ void fma_pair(float& c0, float& c1, float a, float b0, float b1) {
-  asm("{\n .reg .b64 x, y, z;\n mov.b64 x, {%2, %2};\n mov.b64 y, {%3, %4};\n mov.b64 z, {%0, %1};\n"
-      " fma.rn.f32x2 z, x, y, z;\n mov.b64 {%0, %1}, z;\n}"
-      : "+f"(c0), "+f"(c1) : "f"(a), "f"(b0), "f"(b1));
-}
-__device__ __forceinline__ void fma_pair(double& c0, double& c1, double a, double b0, double b1) {
-  c0 = fma(a, b0, c0);
-  c1 = fma(a, b1, c1);
-}
-
 // One BM x BN tile per CTA; a thread owns TM x TN outputs as groups of at most
 // four consecutive rows and columns, so a warp's shared loads are 128-bit
 // broadcasts without bank conflicts.  The next BK-deep slab is in registers

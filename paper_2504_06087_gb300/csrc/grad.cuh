@@ -380,7 +380,8 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 2 : 1) msg_bwd_kernel(
     }
     __syncthreads();
     for (int e = c; e < nb * kPairFeat; e += blockDim.x) {
-      const int q = e / kPairFeat, k = e - q * kPairFeat;
+      int q, k;
+      feature_item(e, nb, q, k);
       m.f->feat[q].f[k][0] =
           pair_feature<T, W>(k, m.f->dv[q], m.f->r[q], p.ee_w1, p.ee_b1, p.ee_sigma, T(cut)).v;
     }
@@ -494,7 +495,8 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 2 : 1) en_bwd_kernel(
     }
     __syncthreads();
     for (int e = c; e < nb * kPairFeat; e += blockDim.x) {
-      const int q = e / kPairFeat, k = e - q * kPairFeat;
+      int q, k;
+      feature_item(e, nb, q, k);
       m.f->feat[q].f[k][0] = pair_feature<T, W>(k, m.f->dv[q], m.f->r[q], w1, b1, p.en_sigma, T(cnuc)).v;
     }
     __syncthreads();

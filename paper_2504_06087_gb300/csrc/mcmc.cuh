@@ -356,7 +356,8 @@ struct MsgBatch {
   template <typename W>
   __device__ __forceinline__ void features(int cnt, const Params<W>& p, double cut) {
     for (int e = threadIdx.x; e < cnt * kPairFeat; e += blockDim.x) {
-      const int q = e / kPairFeat, k = e - q * kPairFeat;
+      int q, k;
+      feature_item(e, cnt, q, k);
       if (Q[q]) feat[q].f[k][0] = pair_feature<T, W>(k, dv[q], r[q], p.ee_w1, p.ee_b1, p.ee_sigma, T(cut)).v;
     }
   }
