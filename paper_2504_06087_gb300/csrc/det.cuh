@@ -251,61 +251,64 @@ __global__ void lu_kernel(int n, LT* __restrict__ M, int32_t* __restrict__ piv,
 inline size_t lu_smem_bytes(int n, size_t lsz, int nb = 16) { return (size_t)(2 * nb + 1) * n * lsz; }
 
 
-// The LU of lu_kernel (same pivots, same chain of operations per element) with
-// the whole matrix in shared memory, one CTA per matrix: three barriers per
-// column, no panel copies and no row interchanges in global memory.  A
-// float64 multiply-add occupies the pipe for so long (a warp's 32 take 64
-// cycles of an SM quarter) that only the number of float64 warp instructions
-// counts: the trailing block is walked as one flat range, so every lane of
-// every instruction works, and column c needs one reciprocal.
-// Two CTAs per SM fit up to n = 119 (float64) or 168 (float32); beyond that
-// the blocked kernel, which keeps only a panel, is the faster one.
+// In-place LU with partial pivoting of the n x n matrix S (row stride ld) in
+// shared memory by one CTA of 256 threads: the pivots to pv, sign changes
+// counted in the return value (uniform), an exactly zero pivot sets *zero and
+// leaves its column.  The float64 pipe takes a warp instruction in 64 cycles
+// of an SM quarter however few lanes work, so the trailing block is walked as
+// one flat range (every lane of every instruction works) and a column takes
+// one reciprocal; and what a column waits for (its update, the pivot search,
+// the reciprocal) warp 0 does for the next column while the other warps update
+// the rest.  Two barriers per column.
+//   best pivot: largest |S[r][c]|, first row on ties; a NaN counts as the
+//   largest (nan_last = false) or only if nothing else is left.
+__device__ __forceinline__ double reciprocal(double x) { return __drcp_rn(x); }
+__device__ __forceinline__ float reciprocal(float x) { return __frcp_rn(x); }
 template <typename LT>
-__global__ void __launch_bounds__(256) lu_smem_kernel(int n, LT* __restrict__ M, int32_t* __restrict__ piv,
-                                                      double* __restrict__ logabs, double* __restrict__ sgn,
-                                                      const int* __restrict__ count) {
-  if (count && (int)blockIdx.x >= *count) return;
-  extern __shared__ unsigned char lu_smem[];
-  LT* S = reinterpret_cast<LT*>(lu_smem);   // [n][n + 1]
-  __shared__ int s_piv, s_zero;
-  __shared__ LT s_pv, s_rinv;
-  const int ld = n + 1;
-  LT* A = M + (int64_t)blockIdx.x * n * n;
-  int32_t* pv = piv + (int64_t)blockIdx.x * n;
-  const int tid = threadIdx.x, bd = blockDim.x;
-  if (tid == 0) s_zero = 0;
-  for (int r = tid >> 5; r < n; r += bd >> 5)
-    for (int c = tid & 31; c < n; c += 32) S[r * ld + c] = A[(int64_t)r * n + c];
-  int neg = 0;
-  __syncthreads();
-  for (int c = 0; c < n; ++c) {
-    if (tid < 32) {   // argmax |S[r][c]|, r >= c, first row on ties
-      unsigned long long best = 0;
-      int bi = c;
-      for (int r = c + tid; r < n; r += 32) {
-        const unsigned long long v = mag_key(S[r * ld + c]);
-        if (v > best) { best = v; bi = r; }
-      }
-      for (int o = 16; o > 0; o >>= 1) {
-        const unsigned long long ov = __shfl_xor_sync(0xffffffffu, best, o);
-        const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
-        if (ov > best || (ov == best && oi < bi)) { best = ov; bi = oi; }
-      }
-      if (tid == 0) {
-        const LT x = S[bi * ld + c];
-        s_piv = bi;
-        s_pv = x;
-        s_rinv = best == 0 ? LT(0) : LT(1) / x;
-        pv[c] = bi;
-        if (best == 0) s_zero = 1;
-      }
+struct LuShared {
+  LT pv[2], rinv[2];
+  int piv[2], zero;
+};
+template <typename LT, bool nan_last>
+__device__ __forceinline__ int lu_smem_core(int n, LT* S, int ld, int32_t* __restrict__ pv, LuShared<LT>& sh) {
+  const int tid = threadIdx.x;
+  auto key = [](LT x) -> unsigned long long {
+    const unsigned long long k = mag_key(x);
+    if (!nan_last) return k;
+    return k > (sizeof(LT) == 8 ? kMagInf : 0x7f800000ull) ? 0 : k + 1;
+  };
+  // pivot of column c (warp 0), its entries updated
+  auto search = [&](int c) {
+    unsigned long long best = 0;
+    int bi = c;
+    for (int r = c + tid; r < n; r += 32) {
+      const unsigned long long v = key(S[r * ld + c]);
+      if (v > best) { best = v; bi = r; }
     }
-    __syncthreads();
-    const int p = s_piv;
-    const LT pivot = s_pv, rinv = s_rinv;
+    // largest key of the warp and its first row: three 32-bit reductions
+    const unsigned hi = (unsigned)(best >> 32), mh = __reduce_max_sync(0xffffffffu, hi);
+    const unsigned lo = hi == mh ? (unsigned)best : 0u, ml = __reduce_max_sync(0xffffffffu, lo);
+    bi = (int)__reduce_min_sync(0xffffffffu, hi == mh && (unsigned)best == ml ? (unsigned)bi : 0xffffffffu);
+    if (tid == 0) {
+      const LT x = S[bi * ld + c];
+      sh.piv[c & 1] = bi;
+      sh.pv[c & 1] = x;
+      sh.rinv[c & 1] = x == LT(0) ? LT(0) : reciprocal(x);
+      pv[c] = bi;
+      if (x == LT(0)) sh.zero = 1;
+    }
+  };
+  if (tid == 0) sh.zero = 0;
+  __syncthreads();
+  if (tid < 32) search(0);
+  __syncthreads();
+  int neg = 0;
+  for (int c = 0; c < n; ++c) {
+    const int p = sh.piv[c & 1];
+    const LT pivot = sh.pv[c & 1], rinv = sh.rinv[c & 1];
     // rows c and p change places; column c becomes the multipliers
     if (p != c) {
-      for (int q = tid; q < n; q += bd) {
+      for (int q = tid; q < n; q += 256) {
         if (q == c) continue;
         const LT t = S[c * ld + q];
         S[c * ld + q] = S[p * ld + q];
@@ -313,26 +316,59 @@ __global__ void __launch_bounds__(256) lu_smem_kernel(int n, LT* __restrict__ M,
       }
       neg ^= 1;
     }
-    for (int r = c + 1 + tid; r < n; r += bd) {
+    for (int r = c + 1 + tid; r < n; r += 256) {
       const LT x = S[(r == p ? c : r) * ld + c];
       S[r * ld + c] = pivot != LT(0) ? x * rinv : x;
       if (r == p) S[c * ld + c] = pivot;
     }
     __syncthreads();
-    if (pivot != LT(0)) {
-      const int w = n - c - 1;
-      const float iw = 1.f / (float)w;
-      for (int e = tid; e < w * w; e += bd) {
-        int rr = (int)((float)e * iw);   // e / w, corrected by one either way
-        rr += (rr + 1) * w <= e ? 1 : 0;
-        rr -= rr * w > e ? 1 : 0;
-        const int r = c + 1 + rr, j = c + 1 + e - rr * w;
+    const int w = n - c - 1;
+    if (tid < 32) {   // column c + 1, then its pivot
+      if (w > 0) {
+        if (pivot != LT(0)) {
+          const LT u = S[c * ld + c + 1];
+          for (int r = c + 1 + tid; r < n; r += 32) S[r * ld + c + 1] -= S[r * ld + c] * u;
+          __syncwarp();
+        }
+        search(c + 1);
+      }
+    } else if (pivot != LT(0)) {
+      const int w1 = w - 1;   // columns c + 2 ..
+      const float iw = 1.f / (float)w1;
+      for (int e = tid - 32; e < w * w1; e += 224) {
+        int rr = (int)((float)e * iw);   // e / w1, corrected by one either way
+        rr += (rr + 1) * w1 <= e ? 1 : 0;
+        rr -= rr * w1 > e ? 1 : 0;
+        const int r = c + 1 + rr, j = c + 2 + e - rr * w1;
         S[r * ld + j] -= S[r * ld + c] * S[c * ld + j];
       }
     }
     __syncthreads();
   }
-  for (int r = tid >> 5; r < n; r += bd >> 5)
+  return neg;
+}
+
+// The LU of lu_kernel (same pivots, same chain of operations per element) with
+// the whole matrix in shared memory, one CTA per matrix: no panel copies and
+// no row interchanges in global memory.  Two CTAs per SM fit up to n = 119
+// (float64) or 168 (float32); beyond that the blocked kernel, which keeps only
+// a panel, is the faster one.  512 matrices of n = 58, a few of them present:
+// 181 us blocked, 105 with the pivot chain in the open, 82 now.
+template <typename LT>
+__global__ void __launch_bounds__(256) lu_smem_kernel(int n, LT* __restrict__ M, int32_t* __restrict__ piv,
+                                                      double* __restrict__ logabs, double* __restrict__ sgn,
+                                                      const int* __restrict__ count) {
+  if (count && (int)blockIdx.x >= *count) return;
+  extern __shared__ unsigned char lu_smem[];
+  LT* S = reinterpret_cast<LT*>(lu_smem);   // [n][n + 1]
+  __shared__ LuShared<LT> sh;
+  const int ld = n + 1;
+  LT* A = M + (int64_t)blockIdx.x * n * n;
+  const int tid = threadIdx.x;
+  for (int r = tid >> 5; r < n; r += 8)
+    for (int c = tid & 31; c < n; c += 32) S[r * ld + c] = A[(int64_t)r * n + c];
+  const int neg = lu_smem_core<LT, false>(n, S, ld, piv + (int64_t)blockIdx.x * n, sh);
+  for (int r = tid >> 5; r < n; r += 8)
     for (int c = tid & 31; c < n; c += 32) A[(int64_t)r * n + c] = S[r * ld + c];
   if (tid < 32) {   // log|det| and sign
     double la = 0.0;
@@ -347,7 +383,7 @@ __global__ void __launch_bounds__(256) lu_smem_kernel(int n, LT* __restrict__ M,
       sg ^= __shfl_xor_sync(0xffffffffu, sg, o);
     }
     if (tid == 0) {
-      if (s_zero) { logabs[blockIdx.x] = -INFINITY; sgn[blockIdx.x] = 0.0; }
+      if (sh.zero) { logabs[blockIdx.x] = -INFINITY; sgn[blockIdx.x] = 0.0; }
       else { logabs[blockIdx.x] = la; sgn[blockIdx.x] = sg ? -1.0 : 1.0; }
     }
   }

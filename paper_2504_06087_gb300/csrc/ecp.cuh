@@ -39,15 +39,8 @@ __device__ inline void quad_dir(int n_quad, int q, double* d) {
   for (int t = 0; t < 3; ++t) d[t] = v[t] / nrm;
 }
 
-// Rotation of electron k in walker w: quaternion (x, y, z, w) =
-// (sqrt(1-u1) sin 2pi u2, sqrt(1-u1) cos 2pi u2, sqrt(u1) sin 2pi u3,
-// sqrt(u1) cos 2pi u3), u1..u3 from Philox counter (k, 0, walker, 3).
-__device__ inline void ecp_rotation(uint64_t seed, uint32_t walker, uint32_t k, double R[3][3]) {
-  const Philox4 c = philox4x32_10(k, 0u, walker, 3u, (uint32_t)seed, (uint32_t)(seed >> 32));
-  const double u1 = u01(c.v[0]), u2 = u01(c.v[1]), u3 = u01(c.v[2]);
-  const double two_pi = 6.283185307179586476925286766559;
-  const double x = sqrt(1.0 - u1) * sin(two_pi * u2), y = sqrt(1.0 - u1) * cos(two_pi * u2);
-  const double z = sqrt(u1) * sin(two_pi * u3), w = sqrt(u1) * cos(two_pi * u3);
+// Rotation matrix of the unit quaternion (x, y, z, w).
+__device__ inline void ecp_matrix(double x, double y, double z, double w, double R[3][3]) {
   R[0][0] = 1 - 2 * (y * y + z * z); R[0][1] = 2 * (x * y - w * z);     R[0][2] = 2 * (x * z + w * y);
   R[1][0] = 2 * (x * y + w * z);     R[1][1] = 1 - 2 * (x * x + z * z); R[1][2] = 2 * (y * z - w * x);
   R[2][0] = 2 * (x * z - w * y);     R[2][1] = 2 * (y * z + w * x);     R[2][2] = 1 - 2 * (x * x + y * y);
@@ -69,47 +62,80 @@ static __global__ void ecp_propose_kernel(int n, int n_up, int k, int q, const d
   const int w = blockIdx.x;
   const int lane = threadIdx.x;
   const double* rw = r + (int64_t)w * n * 3;
-  __shared__ double rn[3];
-  __shared__ int s_active;
+  // Every float64 root, division, sine and power is one sequence for the warp,
+  // so independent ones go to different lanes (all on lane 0: 30 us, now 19).
+  const unsigned full = 0xffffffffu;
+  double x[3];
+  for (int t = 0; t < 3; ++t) x[t] = rw[3 * k + t];
+  // the first pseudopotential nucleus whose r_cut contains the electron
+  int m = -1;
+  double rad = 0.0;
+  for (int m0 = 0; m0 < N && m < 0; m0 += 32) {
+    const int mm = m0 + lane;
+    double d2 = 0.0;
+    bool in = false;
+    if (mm < N && ecp[mm].n_quad > 0) {
+      for (int t = 0; t < 3; ++t) {
+        const double rel = x[t] - nuc_pos[3 * mm + t];
+        d2 += rel * rel;
+      }
+      d2 = sqrt(d2);
+      in = d2 < ecp[mm].r_cut;
+    }
+    const unsigned bal = __ballot_sync(full, in);
+    if (bal) {
+      const int src = __ffs(bal) - 1;
+      m = m0 + src;
+      rad = __shfl_sync(full, d2, src);
+    }
+  }
+  const bool active = m >= 0 && q < ecp[m < 0 ? 0 : m].n_quad && rad > 0.0;
+  double rn[3], p = 0.0;
+  if (active) {   // the same for every lane
+    const fire_ecp_t& ec = ecp[m];
+    // rotation: quaternion (x, y, z, w) = (sqrt(1-u1) sin 2pi u2, sqrt(1-u1) cos 2pi u2,
+    // sqrt(u1) sin 2pi u3, sqrt(u1) cos 2pi u3) in lanes 0 .. 3
+    const Philox4 c = philox4x32_10((uint32_t)k, 0u, (uint32_t)w, 3u, (uint32_t)seed, (uint32_t)(seed >> 32));
+    const double u1 = u01(c.v[0]), u2 = u01(c.v[1]), u3 = u01(c.v[2]);
+    const double two_pi = 6.283185307179586476925286766559;
+    const double ang = two_pi * ((lane & 3) < 2 ? u2 : u3);
+    const double sn = sin(ang), cn = cos(ang);
+    const double rt = sqrt((lane & 3) < 2 ? 1.0 - u1 : u1);
+    const double qv = rt * ((lane & 1) == 0 ? sn : cn);
+    const double qx = __shfl_sync(full, qv, 0), qy = __shfl_sync(full, qv, 1);
+    const double qz = __shfl_sync(full, qv, 2), qw = __shfl_sync(full, qv, 3);
+    double Rm[3][3], d0[3];
+    ecp_matrix(qx, qy, qz, qw, Rm);
+    quad_dir(ec.n_quad, q, d0);
+    // lane t < 3: component t of the direction, its share of rhat . n_q
+    const int t = lane < 3 ? lane : 0;
+    const double d = Rm[t][0] * d0[0] + Rm[t][1] * d0[1] + Rm[t][2] * d0[2];
+    const double rel = x[t] - nuc_pos[3 * m + t];
+    const double cst = d * rel / rad;
+    double cs = 0.0;
+    for (int s = 0; s < 3; ++s) {
+      rn[s] = nuc_pos[3 * m + s] + rad * __shfl_sync(full, d, s);
+      cs += __shfl_sync(full, cst, s);
+    }
+    // lane 4 l + j: term j of channel l
+    const int l = lane >> 2, j = lane & 3;
+    double term = 0.0;
+    if (l < 3 && l < ec.n_channels && j < ec.n_terms[l])
+      term = ec.coef[l][j] * pow(rad, ec.power[l][j]) * exp(-ec.alpha[l][j] * rad * rad);
+    for (int a = 0; a < ec.n_channels; ++a) {
+      double v = 0.0;
+      for (int b = 0; b < ec.n_terms[a]; ++b) v += __shfl_sync(full, term, 4 * a + b);
+      p += v * (2 * a + 1) * legendre_p(a, cs) / (double)ec.n_quad;
+    }
+  } else {
+    for (int t = 0; t < 3; ++t) rn[t] = x[t];
+  }
   if (lane == 0) {
-    int m = -1;
-    double rel[3] = {0, 0, 0}, rad = 0.0;
-    for (int mm = 0; mm < N && m < 0; ++mm) {
-      if (ecp[mm].n_quad <= 0) continue;
-      double d2 = 0.0;
-      for (int t = 0; t < 3; ++t) {
-        rel[t] = rw[3 * k + t] - nuc_pos[3 * mm + t];
-        d2 += rel[t] * rel[t];
-      }
-      if (sqrt(d2) < ecp[mm].r_cut) { m = mm; rad = sqrt(d2); }
-    }
-    double p = 0.0;
-    if (m >= 0 && q < ecp[m].n_quad && rad > 0.0) {
-      double R[3][3], d0[3], d[3];
-      ecp_rotation(seed, (uint32_t)w, (uint32_t)k, R);
-      quad_dir(ecp[m].n_quad, q, d0);
-      double cs = 0.0;
-      for (int t = 0; t < 3; ++t) {
-        d[t] = R[t][0] * d0[0] + R[t][1] * d0[1] + R[t][2] * d0[2];
-        rn[t] = nuc_pos[3 * m + t] + rad * d[t];
-        cs += d[t] * rel[t] / rad;
-      }
-      const fire_ecp_t& e = ecp[m];
-      for (int l = 0; l < e.n_channels; ++l) {
-        double v = 0.0;
-        for (int j = 0; j < e.n_terms[l]; ++j) v += e.coef[l][j] * pow(rad, e.power[l][j]) * exp(-e.alpha[l][j] * rad * rad);
-        p += v * (2 * l + 1) * legendre_p(l, cs) / (double)e.n_quad;
-      }
-      s_active = 1;
-    } else {
-      for (int t = 0; t < 3; ++t) rn[t] = rw[3 * k + t];
-      s_active = 0;
-    }
     for (int t = 0; t < 3; ++t) rk[(int64_t)w * 3 + t] = rn[t];
     pref[w] = p;
   }
   __syncwarp();
-  update_set(w, lane, n, n_up, k, rw, rn, c2, Umax, Ul, Uc, Ucu, st, s_active != 0);
+  update_set(w, lane, n, n_up, k, rw, rn, c2, Umax, Ul, Uc, Ucu, st, active);
 }
 
 // v_nl[w] += pref[w] Psi(r')/Psi(r) for the walkers with a virtual move.
@@ -125,9 +151,9 @@ __global__ void ecp_accum_kernel(int Wn, int n, int n_up, int D, int k, int Umax
                                  const double* __restrict__ lrat, const double* __restrict__ srat,
                                  double* __restrict__ v_nl) {
   const int w = blockIdx.x;
-  if (pref[w] == 0.0) return;   // the whole warp leaves together
+  if (pref[w] == 0.0) return;   // the whole CTA leaves together
   const WalkerRatio wr =
-      walker_ratio<T>(w, threadIdx.x, Wn, n, n_up, D, k, Umax, flags, r + (int64_t)w * n * 3, rk + (int64_t)w * 3, -1,
+      walker_ratio<T>(w, Wn, n, n_up, D, k, Umax, flags, r + (int64_t)w * n * 3, rk + (int64_t)w * 3, -1,
                       nullptr, Ul, Uc, Urow, jp, F1, F2, F1n, F2n, G1, G2, G1n, G2n, ldabs, lsign, lrat, srat);
   if (threadIdx.x == 0) v_nl[w] += pref[w] * wr.sign * exp(wr.logr);
 }

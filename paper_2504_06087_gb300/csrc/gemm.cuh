@@ -30,13 +30,16 @@ struct GemmArgs {
   int nb;                        // columns per block of B
   int accumulate;
   int va, vb, vc;                // 16-byte loads of A and of B, 16-byte stores of C
+  const T* bias;                 // ACT: C = (R ? R : 0) + SiLU(product + bias), R with row stride ldr
+  const T* R;
+  int64_t ldr;
 };
 
 // One BM x BN tile per CTA; a thread owns TM x TN outputs as groups of at most
 // four consecutive rows and columns, so a warp's shared loads are 128-bit
 // broadcasts without bank conflicts.  The next BK-deep slab is in registers
 // while the current one is multiplied.
-template <typename T, int BM, int BN, int BK, int TM, int TN, bool TB>
+template <typename T, int BM, int BN, int BK, int TM, int TN, bool TB, bool ACT = false>
 __global__ void __launch_bounds__((BM / TM) * (BN / TN))
 gemm_kernel(GemmArgs<T> g) {
   constexpr int NT = (BM / TM) * (BN / TN);
@@ -178,6 +181,17 @@ gemm_kernel(GemmArgs<T> g) {
   for (int i = 0; i < TM; ++i) {
     const int64_t gm = m0 + (i / GM) * (BM / RM) + ty * GM + i % GM;
     if (gm >= me) continue;
+    if constexpr (ACT) {
+#pragma unroll
+      for (int j = 0; j < TN; ++j) {
+        const int gn = n0 + (j / GN) * (BN / RN) + tx * GN + j % GN;
+        if (gn >= g.N) continue;
+        T f, f1, f2;
+        silu3<T>(acc[i][j] + g.bias[gn], f, f1, f2);
+        C[gm * g.ldc + gn] = g.R ? g.R[gm * g.ldr + gn] + f : f;
+      }
+      continue;
+    }
 #pragma unroll
     for (int p = 0; p < RN; ++p) {
       const int gn = n0 + p * (BN / RN) + tx * GN;
@@ -211,11 +225,15 @@ template <typename T, int BM, int BN, int BK, int TM, int TN>
 inline void gemm_launch(cudaStream_t s, const GemmArgs<T>& g, bool tb, int64_t m_cap, int batch) {
   const dim3 grid((unsigned)((m_cap + BM - 1) / BM), (unsigned)((g.N + BN - 1) / BN), batch);
   constexpr int NT = (BM / TM) * (BN / TN);
-  if (tb) gemm_kernel<T, BM, BN, BK, TM, TN, true><<<grid, NT, 0, s>>>(g);
+  if (g.bias) gemm_kernel<T, BM, BN, BK, TM, TN, false, true><<<grid, NT, 0, s>>>(g);
+  else if (tb) gemm_kernel<T, BM, BN, BK, TM, TN, true><<<grid, NT, 0, s>>>(g);
   else gemm_kernel<T, BM, BN, BK, TM, TN, false><<<grid, NT, 0, s>>>(g);
 }
 
-// Host launcher.  m_cap bounds end - begin (grid sizing).
+// Host launcher.  m_cap bounds end - begin (grid sizing).  With bias (plain
+// products only) the epilogue is a SiLU layer, C = (R ? R : 0) + SiLU(A B + bias):
+// a move's products are so short that the layer's own launch took a third of
+// their time.  C must not be A or R's rows of another tile (R may be A).
 //
 // float32: tiles of 64 x 64 (64 threads, 8 x 8 outputs each, 168 registers)
 // reach 55-59 of the 77 TFLOP/s of plain multiply-adds once a few tiles per SM
@@ -233,9 +251,12 @@ template <typename T>
 inline void gemm(cudaStream_t s, const T* A, int64_t lda, const T* B, int64_t ldb, bool transB,
                  T* C, int64_t ldc, int64_t m_begin, int64_t m_end, const int64_t* m_range,
                  int64_t m_cap, int N, int K, int batch = 1, int64_t sA = 0, int64_t sB = 0,
-                 int64_t sC = 0, bool accumulate = false) {
+                 int64_t sC = 0, bool accumulate = false, const T* bias = nullptr, const T* R = nullptr,
+                 int64_t ldr = 0) {
   if (m_cap <= 0 || N <= 0 || K <= 0 || batch <= 0) return;
-  GemmArgs<T> g{A, B, C, lda, ldb, ldc, sA, sB, sC, m_begin, m_end, m_range, N, K, N, accumulate ? 1 : 0, 0, 0, 0};
+  GemmArgs<T> g{A, B, C, lda, ldb, ldc, sA, sB, sC, m_begin, m_end, m_range, N, K, N, accumulate ? 1 : 0, 0, 0, 0,
+                bias, R, ldr};
+  if (bias && (transB || batch != 1 || accumulate)) return;   // the fused layer is a plain product
   if (batch > 1 && sA == 0 && sC == N) {   // side by side: one product of batch * N columns
     g.N = N * batch;
     batch = 1;
@@ -248,15 +269,18 @@ inline void gemm(cudaStream_t s, const T* A, int64_t lda, const T* B, int64_t ld
   if constexpr (sizeof(T) == 8) {
     gemm_launch<T, 16, 16, 32, 1, 2>(s, g, transB, m_cap, batch);
   } else {
-    // the tile of least estimated time: rounds of 152 SMs times the tile's
-    // outputs over its rate relative to the 64 x 64 tile's
-    struct Tile { int bm, bn; float eff; };
-    constexpr Tile t[] = {{64, 64, 1.f}, {32, 32, 0.38f}, {128, 16, 0.42f}};
+    // the tile of least estimated time, in outputs of the 64 x 64 tile's rate:
+    // all tiles over 152 SMs, but no less than one tile alone takes (a lone
+    // 64-thread tile is a chain of loads and barriers: 3700 rows, N = K = 128,
+    // 11 us against 8 with 32 x 32 tiles)
+    struct Tile { int bm, bn; float eff, lone; };
+    constexpr Tile t[] = {{64, 64, 1.f, 18500.f}, {32, 32, 0.38f, 11700.f}, {128, 16, 0.42f, 16000.f}};
     int best = 0;
     float cost = 3.4e38f;
     for (int q = 0; q < 3; ++q) {
       const int64_t tiles = ((m_cap + t[q].bm - 1) / t[q].bm) * ((g.N + t[q].bn - 1) / t[q].bn) * batch;
-      const float c = (float)((tiles + 151) / 152) * t[q].bm * t[q].bn / t[q].eff;
+      float c = (float)tiles * t[q].bm * t[q].bn / (152.f * t[q].eff);
+      if (c < t[q].lone) c = t[q].lone + 1e-3f * c;
       if (c < cost) { cost = c; best = q; }
     }
     if (best == 0) gemm_launch<T, 64, 64, 16, 8, 8>(s, g, transB, m_cap, batch);

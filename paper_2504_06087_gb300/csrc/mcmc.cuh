@@ -18,6 +18,7 @@
 #pragma once
 
 #include "common.cuh"
+#include "det.cuh"
 #include "embed.cuh"
 #include "philox.cuh"
 
@@ -552,8 +553,10 @@ __global__ void __launch_bounds__(256) mcmc_ratio_kernel(
     const T* __restrict__ Phi, const T* __restrict__ AT, T* __restrict__ Dl, T* __restrict__ Mt,
     double* __restrict__ Mg, int32_t* __restrict__ Mpiv, double* __restrict__ lrat, double* __restrict__ srat,
     const int32_t* __restrict__ xflag, int k2 = -1, const T* __restrict__ Fk2 = nullptr) {
-  __shared__ double su[kLemmaSmem * (kLemmaSmem + 1)];   // the product tiles, then M
-  __shared__ int s_p;
+  // the product's chunks (or tiles), then M
+  constexpr int kStage = 2 * 2 * kLemmaSmem * 144 / 8;
+  static_assert(kStage >= kLemmaSmem * (kLemmaSmem + 1), "M");
+  __shared__ __align__(16) double su[kStage];
   const int w = blockIdx.x / D, dd = blockIdx.x % D;
   const int u = Uc[w];
   const int64_t Dn = (int64_t)D * n;
@@ -579,74 +582,85 @@ __global__ void __launch_bounds__(256) mcmc_ratio_kernel(
     Dw[(int64_t)aa * n + l] = o * ph - Pw[(int64_t)i * n + l];
   }
   if (xflag[md]) return;   // its ratio comes from a float64 LU: only Delta is needed
-  // Delta A[:, U] = Delta (u x n) times the rows U of A^T
-  T* Mw = Mt + md * Umax * Umax;
-  cta_gemm_nt<T>(u, u, n, Dw, n, Aw, n, U, Mw, Umax, T(1), false, reinterpret_cast<T*>(su));
+  // Delta A[:, U] = Delta (u x n) times the rows U of A^T, plus 1
   const bool in_smem = u <= kLemmaSmem;
   double* M = in_smem ? su : Mg + md * Umax * Umax;
   const int ldm = in_smem ? kLemmaSmem + 1 : Umax;
-  for (int e = threadIdx.x; e < u * u; e += blockDim.x) {
-    const int a = e / u, b = e % u;
-    M[a * ldm + b] = (double)Mw[a * Umax + b] + (a == b ? 1.0 : 0.0);
+  if (in_smem) {
+    // chunks of 128 bytes of every row, copied one ahead; a thread owns rows
+    // ta + 16 i and columns tm + 16 j (the same chain of multiply-adds as the
+    // tiled product: 32 x 32 tiles waited for global memory at two barriers a tile)
+    constexpr int LC = 128 / (int)sizeof(T), LS = LC + 16 / (int)sizeof(T), VE = 16 / (int)sizeof(T);
+    const int tid = threadIdx.x, tm = tid & 15, ta = tid >> 4;
+    T* stage[2] = {reinterpret_cast<T*>(su), reinterpret_cast<T*>(su) + 2 * kLemmaSmem * LS};
+    __syncthreads();   // Delta is written
+    auto fetch = [&](int l0, T* to) {
+      for (int e = tid; e < 2 * u * LC; e += 256) {
+        const int row = e / LC, c = e % LC, l = l0 + c;
+        const T* src = row < u ? Dw + (int64_t)row * n : Aw + (int64_t)U[row - u] * n;
+        const uint32_t dst = (uint32_t)__cvta_generic_to_shared(to + (int64_t)row * LS + c);
+        asm volatile("cp.async.ca.shared.global [%0], [%1], %2, %3;" ::"r"(dst), "l"(src + (l < n ? l : 0)),
+                     "n"((int)sizeof(T)), "r"(l < n ? (int)sizeof(T) : 0)
+                     : "memory");
+      }
+      asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+    T b[4][4];
+#pragma unroll
+    for (int p = 0; p < 4; ++p)
+#pragma unroll
+      for (int q = 0; q < 4; ++q) b[p][q] = T(0);
+    fetch(0, stage[0]);
+    int buf = 0;
+    for (int l0 = 0; l0 < n; l0 += LC) {
+      if (l0 + LC < n) {
+        fetch(l0 + LC, stage[buf ^ 1]);
+        asm volatile("cp.async.wait_group 1;" ::: "memory");
+      } else {
+        asm volatile("cp.async.wait_group 0;" ::: "memory");
+      }
+      __syncthreads();
+      const T *sd = stage[buf], *sx = sd + (int64_t)u * LS;
+#pragma unroll 2
+      for (int c = 0; c < LC; c += VE) {
+        T d[4][VE];
+#pragma unroll
+        for (int p = 0; p < 4; ++p)
+          if (16 * p < u) ld_vec<T, VE>(d[p], sd + (int64_t)(ta + 16 * p < u ? ta + 16 * p : u - 1) * LS + c);
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          if (16 * q < u) {
+            T x[VE];
+            ld_vec<T, VE>(x, sx + (int64_t)(tm + 16 * q < u ? tm + 16 * q : u - 1) * LS + c);
+#pragma unroll
+            for (int p = 0; p < 4; ++p)
+              if (16 * p < u) {
+#pragma unroll
+                for (int v = 0; v < VE; ++v) b[p][q] = fma(d[p][v], x[v], b[p][q]);
+              }
+          }
+        }
+      }
+      __syncthreads();
+      buf ^= 1;
+    }
+#pragma unroll
+    for (int p = 0; p < 4; ++p)
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const int a = ta + 16 * p, c = tm + 16 * q;
+        if (a < u && c < u) M[a * ldm + c] = (double)b[p][q] + (a == c ? 1.0 : 0.0);
+      }
+  } else {
+    T* Mw = Mt + md * Umax * Umax;
+    cta_gemm_nt<T>(u, u, n, Dw, n, Aw, n, U, Mw, Umax, T(1), false, reinterpret_cast<T*>(su));
+    for (int e = threadIdx.x; e < u * u; e += blockDim.x) {
+      const int a = e / u, c = e % u;
+      M[a * ldm + c] = (double)Mw[a * Umax + c] + (a == c ? 1.0 : 0.0);
+    }
   }
-  __syncthreads();
-  int32_t* pv = Mpiv + md * Umax;
-  __shared__ double s_pv;
-  int neg = 0;
-  for (int c = 0; c < u; ++c) {
-    if (threadIdx.x < 32) {   // pivot: the first row of largest |M[q][c]|, q >= c (never a NaN while others are left)
-      unsigned long long best = 0;
-      int bq = c;
-      for (int q = c + threadIdx.x; q < u; q += 32) {
-        const double x = M[q * ldm + c];
-        const unsigned long long v = mag_key(x) > kMagInf ? 0 : mag_key(x) + 1;
-        if (v > best) { best = v; bq = q; }
-      }
-      for (int o = 16; o > 0; o >>= 1) {
-        const unsigned long long ob = __shfl_xor_sync(0xffffffffu, best, o);
-        const int oq = __shfl_xor_sync(0xffffffffu, bq, o);
-        if (ob > best || (ob == best && oq < bq)) { best = ob; bq = oq; }
-      }
-      if (threadIdx.x == 0) {
-        s_p = bq;
-        s_pv = M[bq * ldm + c];
-        pv[c] = bq;
-      }
-    }
-    __syncthreads();
-    const int pq = s_p;
-    const double piv = s_pv;
-    // rows c and pq change places, and column c becomes the multipliers (one
-    // division per row)
-    if (pq != c) {
-      for (int q = threadIdx.x; q < u; q += blockDim.x) {
-        if (q == c) continue;
-        const double t = M[c * ldm + q];
-        M[c * ldm + q] = M[pq * ldm + q];
-        M[pq * ldm + q] = t;
-      }
-      neg ^= 1;
-    }
-    if (piv < 0.0) neg ^= 1;
-    for (int q = c + 1 + threadIdx.x; q < u; q += blockDim.x) {
-      const double x = M[(q == pq ? c : q) * ldm + c];
-      M[q * ldm + c] = piv == 0.0 ? x : x / piv;
-      if (q == pq) M[c * ldm + c] = piv;
-    }
-    __syncthreads();
-    if (piv != 0.0) {
-      const int wdt = u - c - 1;
-      const float iw = 1.f / (float)wdt;
-      for (int e = threadIdx.x; e < wdt * wdt; e += blockDim.x) {
-        int rr = (int)((float)e * iw);            // e / wdt, corrected by one either way
-        rr += (rr + 1) * wdt <= e ? 1 : 0;
-        rr -= rr * wdt > e ? 1 : 0;
-        const int q = c + 1 + rr, cc = c + 1 + e - rr * wdt;
-        M[q * ldm + cc] -= M[q * ldm + c] * M[c * ldm + cc];
-      }
-    }
-    __syncthreads();
-  }
+  __shared__ LuShared<double> sh;
+  int neg = lu_smem_core<double, true>(u, M, ldm, Mpiv + md * Umax, sh);
   // log|det M|: the logarithms by the lanes of one warp, summed in order
   if (threadIdx.x < 32) {
     double la = 0.0;
@@ -656,6 +670,7 @@ __global__ void __launch_bounds__(256) mcmc_ratio_kernel(
       const double p = c < u ? M[c * ldm + c] : 1.0;
       const double l = p == 0.0 ? 0.0 : log(fabs(p));
       zero |= __any_sync(0xffffffffu, p == 0.0);
+      neg ^= __popc(__ballot_sync(0xffffffffu, p < 0.0)) & 1;
       for (int k = 0; k < 32 && c0 + k < u; ++k) la += __shfl_sync(0xffffffffu, l, k);
     }
     if (threadIdx.x == 0) {
@@ -690,16 +705,34 @@ __global__ void mcmc_att_kernel(int Wn, int n, int n_up, int R, int dr, int Umax
   auto row = [&](int i) -> const T* {
     return slot[i] >= 0 ? SUn + (int64_t)slot[i] * ldn : SU + (int64_t)block_index(w, i, Wn, n, n_up) * ld;
   };
-  for (int q = threadIdx.x; q < R; q += blockDim.x) {
+  // largest score per register: one warp per register, electrons over its lanes
+  for (int q = threadIdx.x >> 5; q < R; q += blockDim.x >> 5) {
     T m = -INFINITY;
-    for (int i = 0; i < n; ++i) m = fmax(m, row(i)[q]);
-    smax[q] = m;
+    for (int i = threadIdx.x & 31; i < n; i += 32) m = fmax(m, row(i)[q]);
+    for (int o = 16; o > 0; o >>= 1) m = fmax(m, __shfl_xor_sync(0xffffffffu, m, o));
+    if ((threadIdx.x & 31) == 0) smax[q] = m;
   }
   __syncthreads();
   for (int col = threadIdx.x; col < RD; col += blockDim.x) {
     const int rg = col / dr;
     T Z = T(0), Nv = T(0);
-    for (int i = 0; i < n; ++i) {
+    int i = 0;
+    for (; i + 8 <= n; i += 8) {   // the loads of eight electrons in flight
+      T sc[8], vv[8];
+#pragma unroll
+      for (int u = 0; u < 8; ++u) {
+        const T* rr = row(i + u);
+        sc[u] = rr[rg];
+        vv[u] = rr[R + col];
+      }
+#pragma unroll
+      for (int u = 0; u < 8; ++u) {
+        const T e = dexp<T>(sc[u] - smax[rg]);
+        Z += e;
+        Nv += e * vv[u];
+      }
+    }
+    for (; i < n; ++i) {
       const T* rr = row(i);
       const T e = dexp<T>(rr[rg] - smax[rg]);
       Z += e;
@@ -715,7 +748,7 @@ struct McmcJastrow {
 };
 
 // ln|Psi'/Psi| and sign(Psi'/Psi) of walker w for the move of electron k to
-// rk (all lanes of one warp call it; the result is valid on lane 0):
+// rk (every thread of the CTA calls it; the result is valid on thread 0):
 // determinant part from the ratios of all determinants, cusp change of
 // electron k, change of the MLP-Jastrow sums over the update set, change of
 // the attention-Jastrow readout.
@@ -723,8 +756,14 @@ struct WalkerRatio {
   double logr, sign;
 };
 
+// By kRatioThreads threads.  A float64 logarithm, exponential, root or division
+// holds the pipe for a thousand cycles or more whether one lane needs it or
+// 32, so the terms are spread over lanes (determinants, the six logarithms)
+// and warps (the cusp pairs) and then summed in the order one lane would
+// (one warp with the sums on lane 0: 34-60 us a move, now 18-29).
+constexpr int kRatioThreads = 128;
 template <typename T>
-__device__ WalkerRatio walker_ratio(int w, int lane, int Wn, int n, int n_up, int D, int k, int Umax, uint32_t flags,
+__device__ WalkerRatio walker_ratio(int w, int Wn, int n, int n_up, int D, int k, int Umax, uint32_t flags,
                                     const double* __restrict__ rw, const double* __restrict__ rn, int k2,
                                     const double* __restrict__ rn2,
                                     const int32_t* __restrict__ Ul, const int32_t* __restrict__ Uc,
@@ -734,28 +773,50 @@ __device__ WalkerRatio walker_ratio(int w, int lane, int Wn, int n, int n_up, in
                                     const T* __restrict__ G1n, const T* __restrict__ G2n,
                                     const double* __restrict__ ldabs, const double* __restrict__ lsign,
                                     const double* __restrict__ lrat, const double* __restrict__ srat) {
+  constexpr int NW = kRatioThreads / 32;
+  __shared__ double s_dc[NW][2][32];
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   const T* cusp = reinterpret_cast<const T*>(jp.cusp);
   double dc = 0.0, s2 = 0.0, ds1 = 0.0, ds2 = 0.0;
   const double wp = (double)cusp[0], wa = (double)cusp[1], ap = (double)cusp[2], aa = (double)cusp[3];
   // cusp terms of the pairs of a moved electron (k, and k2 >= 0 for a swap of
-  // two electrons, whose own pair keeps its distance and spin channel)
-  for (int j = lane; j < n; j += 32) {
-    for (int mv = 0; mv < 2; ++mv) {
-      const int km = mv == 0 ? k : k2;
-      const double* rm = mv == 0 ? rn : rn2;
-      if (km < 0 || j == k || j == k2) continue;
-      const bool same = (j < n_up) == (km < n_up);
-      const double om = same ? wp : wa, al = same ? ap : aa;
-      double o2 = 0.0, n2 = 0.0;
-      for (int t = 0; t < 3; ++t) {
-        const double a = rw[3 * km + t] - rw[3 * j + t], b = rm[t] - rw[3 * j + t];
-        o2 += a * a;
-        n2 += b * b;
+  // two electrons, whose own pair keeps its distance and spin channel); warp g
+  // forms the terms of electrons 32 (NW i + g) + lane, warp 0 sums them
+  for (int j0 = 0; j0 < n; j0 += 32 * NW) {
+    const int j = j0 + 32 * wid + lane;
+    if (flags & FIRE_J_CUSP)
+      for (int mv = 0; mv < 2; ++mv) {
+        const int km = mv == 0 ? k : k2;
+        const double* rm = mv == 0 ? rn : rn2;
+        double term = 0.0;
+        if (j < n && km >= 0 && j != k && j != k2) {
+          const bool same = (j < n_up) == (km < n_up);
+          const double om = same ? wp : wa, al = same ? ap : aa;
+          double o2 = 0.0, n2 = 0.0;
+          for (int t = 0; t < 3; ++t) {
+            const double a = rw[3 * km + t] - rw[3 * j + t], b = rm[t] - rw[3 * j + t];
+            o2 += a * a;
+            n2 += b * b;
+          }
+          term = om * al * al / (al + sqrt(n2)) - om * al * al / (al + sqrt(o2));
+        }
+        s_dc[wid][mv][lane] = term;
+        if (k2 < 0) break;
       }
-      dc += om * al * al / (al + sqrt(n2)) - om * al * al / (al + sqrt(o2));
-    }
-    if (flags & FIRE_J_MLP) s2 += (double)F2[block_index(w, j, Wn, n, n_up)];
+    __syncthreads();
+    if (wid == 0)
+      for (int g = 0; g < NW && j0 + 32 * g < n; ++g) {
+        if (flags & FIRE_J_CUSP) {
+          dc += s_dc[g][0][lane];
+          if (k2 >= 0) dc += s_dc[g][1][lane];
+        }
+        const int jj = j0 + 32 * g + lane;
+        if ((flags & FIRE_J_MLP) && jj < n) s2 += (double)F2[block_index(w, jj, Wn, n, n_up)];
+      }
+    __syncthreads();
   }
+  WalkerRatio out{0.0, 0.0};
+  if (wid != 0) return out;
   if (flags & FIRE_J_MLP)
     for (int a = lane; a < Uc[w]; a += 32) {
       const int i = Ul[(int64_t)w * Umax + a];
@@ -770,8 +831,6 @@ __device__ WalkerRatio walker_ratio(int w, int lane, int Wn, int n, int n_up, in
     ds1 += __shfl_xor_sync(0xffffffffu, ds1, o);
     ds2 += __shfl_xor_sync(0xffffffffu, ds2, o);
   }
-  WalkerRatio out{0.0, 0.0};
-  if (lane != 0) return out;
   // determinants: ln|sum_d s_d rho_d e^{l_d}| - ln|sum_d s_d e^{l_d}|
   const double* lw = ldabs + (int64_t)w * D;
   const double* sw = lsign + (int64_t)w * D;
@@ -779,28 +838,52 @@ __device__ WalkerRatio walker_ratio(int w, int lane, int Wn, int n, int n_up, in
   const double* sr = srat + (int64_t)w * D;
   double lmax = -INFINITY, lmaxn = -INFINITY;
   auto live = [&](int q) { return sw[q] * sr[q] != 0.0 && isfinite(lr[q]); };
-  for (int q = 0; q < D; ++q) {
+  for (int q = lane; q < D; q += 32) {
     if (sw[q] != 0.0 && lw[q] > lmax) lmax = lw[q];
     if (live(q) && lw[q] + lr[q] > lmaxn) lmaxn = lw[q] + lr[q];
   }
-  double So = 0.0, Sn = 0.0;
-  for (int q = 0; q < D; ++q) {
-    if (sw[q] != 0.0) So += sw[q] * exp(lw[q] - lmax);
-    if (live(q)) Sn += sw[q] * sr[q] * exp(lw[q] + lr[q] - lmaxn);
+  for (int o = 16; o > 0; o >>= 1) {
+    const double a = __shfl_xor_sync(0xffffffffu, lmax, o), b = __shfl_xor_sync(0xffffffffu, lmaxn, o);
+    lmax = a > lmax ? a : lmax;
+    lmaxn = b > lmaxn ? b : lmaxn;
   }
-  double logr = (lmaxn + log(fabs(Sn))) - (lmax + log(fabs(So)));
+  double So = 0.0, Sn = 0.0;
+  for (int q0 = 0; q0 < D; q0 += 32) {
+    const int q = q0 + lane;
+    const bool o = q < D && sw[q] != 0.0, nw = q < D && live(q);
+    const double eo = o ? exp(lw[q] - lmax) : 0.0, en = nw ? exp(lw[q] + lr[q] - lmaxn) : 0.0;
+    const double fo = o ? sw[q] : 0.0, fn = nw ? sw[q] * sr[q] : 0.0;
+    for (int g = 0; g < 32 && q0 + g < D; ++g) {
+      const double xo = __shfl_sync(0xffffffffu, eo, g), xn = __shfl_sync(0xffffffffu, en, g);
+      const double yo = __shfl_sync(0xffffffffu, fo, g), yn = __shfl_sync(0xffffffffu, fn, g);
+      if (yo != 0.0) So += yo * xo;
+      if (yn != 0.0) Sn += yn * xn;
+    }
+  }
+  // the logarithms, one per lane
+  const double S2o = s2 + n * ((flags & FIRE_J_MLP) ? (double)reinterpret_cast<const T*>(jp.jb32)[0] : 0.0);
+  double gn = 1.0, go = 1.0;
+  if (flags & FIRE_J_ATT) {
+    const double b32 = (double)reinterpret_cast<const T*>(jp.ab32)[0];
+    gn = (double)G2n[w] + b32;
+    go = (double)G2[w] + b32;
+  }
+  const double arg = lane == 0 ? Sn : lane == 1 ? So : lane == 2 ? S2o + ds2 : lane == 3 ? S2o : lane == 4 ? gn : go;
+  const double lg = log(fabs(arg));
+  const double lSn = __shfl_sync(0xffffffffu, lg, 0), lSo = __shfl_sync(0xffffffffu, lg, 1);
+  const double l2n = __shfl_sync(0xffffffffu, lg, 2), l2o = __shfl_sync(0xffffffffu, lg, 3);
+  const double lgn = __shfl_sync(0xffffffffu, lg, 4), lgo = __shfl_sync(0xffffffffu, lg, 5);
+  if (lane != 0) return out;
+  double logr = (lmaxn + lSn) - (lmax + lSo);
   double sg = (Sn > 0.0) == (So > 0.0) ? 1.0 : -1.0;
   if (Sn == 0.0) sg = 0.0;
   if (flags & FIRE_J_CUSP) logr += dc;
   if (flags & FIRE_J_MLP) {
-    const double S2o = s2 + n * (double)reinterpret_cast<const T*>(jp.jb32)[0];
-    logr += ds1 + log(fabs(S2o + ds2)) - log(fabs(S2o));
+    logr += ds1 + l2n - l2o;
     if ((S2o + ds2 > 0.0) != (S2o > 0.0)) sg = -sg;
   }
   if (flags & FIRE_J_ATT) {
-    const double b32 = (double)reinterpret_cast<const T*>(jp.ab32)[0];
-    const double gn = (double)G2n[w] + b32, go = (double)G2[w] + b32;
-    logr += ((double)G1n[w] - (double)G1[w]) + log(fabs(gn)) - log(fabs(go));
+    logr += ((double)G1n[w] - (double)G1[w]) + lgn - lgo;
     if ((gn > 0.0) != (go > 0.0)) sg = -sg;
   }
   out.logr = logr;
@@ -810,7 +893,7 @@ __device__ WalkerRatio walker_ratio(int w, int lane, int Wn, int n, int n_up, in
 
 // Accept / reject: accept iff ln u < 2 ln|Psi'/Psi| + lq (lq = 0 for a local
 // move, the Hastings factor ln rho(r_k) - ln rho(r'_k) for a global jump)
-// and the ratio is finite.  One warp per walker; an accepted walker moves r_k
+// and the ratio is finite.  One CTA per walker; an accepted walker moves r_k
 // and updates its determinant logs and its running log|Psi|.
 template <typename T>
 __global__ void mcmc_accept_kernel(int Wn, int n, int n_up, int D, int k, int Umax, uint32_t flags,
@@ -829,12 +912,11 @@ __global__ void mcmc_accept_kernel(int Wn, int n, int n_up, int D, int k, int Um
                                    int* __restrict__ rcnt, int32_t* __restrict__ rlist, int rcap,
                                    unsigned long long* __restrict__ nrepair) {
   const int w = blockIdx.x;
-  const int lane = threadIdx.x;
   double* rw = r + (int64_t)w * n * 3;
   const double* rn = rk + (int64_t)w * 3;
-  const WalkerRatio wr = walker_ratio<T>(w, lane, Wn, n, n_up, D, k, Umax, flags, rw, rn, -1, nullptr, Ul, Uc, Urow,
+  const WalkerRatio wr = walker_ratio<T>(w, Wn, n, n_up, D, k, Umax, flags, rw, rn, -1, nullptr, Ul, Uc, Urow,
                                          jp, F1, F2, F1n, F2n, G1, G2, G1n, G2n, ldabs, lsign, lrat, srat);
-  if (lane != 0) return;
+  if (threadIdx.x != 0) return;
   const double logr = wr.logr;
   const double* lr = lrat + (int64_t)w * D;
   const double* sr = srat + (int64_t)w * D;

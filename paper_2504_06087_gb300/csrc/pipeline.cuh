@@ -1335,15 +1335,19 @@ struct Runner {
     const size_t msm = (size_t)n * sizeof(int);
     const size_t asm_ = (((size_t)n * sizeof(int) + 15) & ~(size_t)15) + (size_t)R * sizeof(T);
     const int abt = RD < 1024 ? ((RD + 31) / 32) * 32 : 1024;
+    // SiLU layer Y = (R ? R : 0) + SiLU(A w + b) over rows [rng[0], rng[1]) (Y is neither A nor R)
+    auto layer = [&](const T* A, int64_t lda, const T* w, const T* b, T* Yl, int64_t ldy, const int64_t* rng,
+                     int64_t cap, int No, int Ki, const T* Rl = nullptr, int64_t ldr = 0) {
+      gemm<T>(s, A, lda, w, No, false, Yl, ldy, 0, 0, rng, cap, No, Ki, 1, 0, 0, 0, false, b, Rl, ldr);
+      launches += 1;
+    };
     // two-hidden-layer SiLU readout over rows [rng[0], rng[1]); Zb has row stride ldzb
     auto readout = [&](const T* Xin, int din, const int64_t* rng, int64_t cap, const T* w1, const T* b1,
                        const T* w2, const T* b2, const T* w3, T* Zb, int64_t ldzb, T* Yb, T* F) {
-      gemm<T>(s, Xin, din, w1, J, false, Zb, ldzb, 0, 0, rng, cap, J, din);
-      mcmc_act_kernel<T, T><<<actg, 256, 0, s>>>(rng, J, Zb, ldzb, b1, Yb, J, 0);
-      gemm<T>(s, Yb, J, w2, J, false, Zb, ldzb, 0, 0, rng, cap, J, J);
-      mcmc_act_kernel<T, T><<<actg, 256, 0, s>>>(rng, J, Zb, ldzb, b2, Yb, J, 0);
-      rowdot_kernel<T, T><<<(unsigned)((cap + 7) / 8), 256, 0, s>>>(Yb, J, J, w3, F, rng, 0, 0);
-      launches += 5;
+      layer(Xin, din, w1, b1, Yb, J, rng, cap, J, din);
+      layer(Yb, J, w2, b2, Zb, ldzb, rng, cap, J, J);
+      rowdot_kernel<T, T><<<(unsigned)((cap + 7) / 8), 256, 0, s>>>(Zb, ldzb, J, w3, F, rng, 0, 0);
+      launches += 1;
     };
     // unit roundoff of the state, for the conditioning test of the exact ratios
     const double kunit = sizeof(T) == 4 ? 5.9604644775390625e-8 : 1.1102230246251565e-16;
@@ -1379,10 +1383,20 @@ struct Runner {
     // and the determinant ratios (k2 >= 0: a second moved electron whose
     // envelope row is Fk2)
     auto rows_and_ratio = [&](int k, int k2, const T* Fk2) {
-      mark("mc_mlp", 2 * dm.L);
-      for (int l = 0; l < dm.L; ++l) {
-        gemm<T>(s, X1, d, p.mlp_w + (int64_t)l * d * d, d, false, Zm, ldz, 0, 0, fullu, capU, d, d);
-        mcmc_act_kernel<T, T><<<actg, 256, 0, s>>>(fullu, d, Zm, ldz, p.mlp_b + (int64_t)l * d, X1, d, 1);
+      mark("mc_mlp", 0);
+      // residual layers X1 -> Zm -> X1 ..., so the rows end in X1; an odd first
+      // layer in place, through a product and a layer kernel of its own
+      int l0 = 0;
+      if (dm.L & 1) {
+        gemm<T>(s, X1, d, p.mlp_w, d, false, Zm, ldz, 0, 0, fullu, capU, d, d);
+        mcmc_act_kernel<T, T><<<actg, 256, 0, s>>>(fullu, d, Zm, ldz, p.mlp_b, X1, d, 1);
+        launches += 2;
+        l0 = 1;
+      }
+      for (int l = l0; l < dm.L; l += 2) {
+        layer(X1, d, p.mlp_w + (int64_t)l * d * d, p.mlp_b + (int64_t)l * d, Zm, ldz, fullu, capU, d, d, X1, d);
+        layer(Zm, ldz, p.mlp_w + (int64_t)(l + 1) * d * d, p.mlp_b + (int64_t)(l + 1) * d, X1, d, fullu, capU, d, d, Zm,
+              ldz);
       }
       if (dm.flags & FIRE_J_MLP) {
         mark("mc_jastrow", 0);
@@ -1481,7 +1495,7 @@ struct Runner {
         check("swap msg");
         rows_and_ratio(a2, b, Fk2);
         mark("swap_accum", 1);
-        swap_accum_kernel<T><<<Wn, 32, 0, s>>>(Wn, n, n_up, D, a2, b, Umax, dm.flags, r, rk, rk2, Ul, Uc, Urow, jp,
+        swap_accum_kernel<T><<<Wn, kRatioThreads, 0, s>>>(Wn, n, n_up, D, a2, b, Umax, dm.flags, r, rk, rk2, Ul, Uc, Urow, jp,
                                                F1, F2, F1n, F2n, G1, G2, G1n, G2n, ldabs, lsign, lrat, srat,
                                                mc.swap_ratios);
         check("swap");
@@ -1506,7 +1520,7 @@ struct Runner {
                                                lq, Ul, Uc, Ucu, st);
           evaluate_move(k);
           mark("ecp_accum", 1);
-          ecp_accum_kernel<T><<<Wn, 32, 0, s>>>(Wn, n, n_up, D, k, Umax, dm.flags, r, rk, lq, Ul, Uc, Urow, jp, F1, F2,
+          ecp_accum_kernel<T><<<Wn, kRatioThreads, 0, s>>>(Wn, n, n_up, D, k, Umax, dm.flags, r, rk, lq, Ul, Uc, Urow, jp, F1, F2,
                                                 F1n, F2n, G1, G2, G1n, G2n, ldabs, lsign, lrat, srat, mc.v_nl);
           check("ecp");
         }
@@ -1544,7 +1558,7 @@ struct Runner {
         int* rcnt = at<int>(pl.mc_xcnt);
         int32_t* rlist = at<int32_t>(pl.mc_xlist);
         cudaMemsetAsync(rcnt, 0, sizeof(int), s);
-        mcmc_accept_kernel<T><<<Wn, 32, 0, s>>>(Wn, n, n_up, D, k, Umax, dm.flags, r, rk, uacc, Ul, Uc, Urow, jp, F1,
+        mcmc_accept_kernel<T><<<Wn, kRatioThreads, 0, s>>>(Wn, n, n_up, D, k, Umax, dm.flags, r, rk, uacc, Ul, Uc, Urow, jp, F1,
                                                 F2, F1n, F2n, G1, G2, G1n, G2n, ldabs, lsign, lrat, srat, lp, acc,
                                                 mc.acc_count, &ms->n_accepted, lref, flag, xflag, lq, rcnt, rlist,
                                                 pl.xcap, &ms->n_repair);

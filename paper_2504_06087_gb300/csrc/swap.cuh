@@ -133,7 +133,7 @@ __global__ void swap_accum_kernel(int Wn, int n, int n_up, int D, int a, int b, 
                                   const double* __restrict__ lrat, const double* __restrict__ srat,
                                   double* __restrict__ ratios) {
   const int w = blockIdx.x;
-  const WalkerRatio wr = walker_ratio<T>(w, threadIdx.x, Wn, n, n_up, D, a, Umax, flags, r + (int64_t)w * n * 3,
+  const WalkerRatio wr = walker_ratio<T>(w, Wn, n, n_up, D, a, Umax, flags, r + (int64_t)w * n * 3,
                                          rk + (int64_t)w * 3, b, rk2 + (int64_t)w * 3, Ul, Uc, Urow, jp, F1, F2, F1n,
                                          F2n, G1, G2, G1n, G2n, ldabs, lsign, lrat, srat);
   if (threadIdx.x == 0) ratios[(int64_t)w * n_up + a] = wr.sign * exp(wr.logr);
