@@ -469,6 +469,14 @@ int fire_selftest_simt_gemm(int32_t dtype, int64_t M, int32_t N, int32_t K, int3
                             int32_t accumulate, const void* A, int64_t lda, const void* B, int64_t ldb,
                             int64_t sB, void* C, int64_t ldc, int64_t sC, void* stream);
 
+/* Diagnostic: the same product as a SiLU layer, C = (R ? R : 0) + SiLU(A B +
+ * bias) for A[M][K], B[K][N], bias[N], R[M][N] (R may be NULL; ldr is read only
+ * with it).  With `one` the residual sum is a single multiply-add, without it
+ * product and sum are rounded one by one.  FIRE_ERR_INVALID_ARG as above. */
+int fire_selftest_simt_layer(int32_t dtype, int64_t M, int32_t N, int32_t K, int32_t one, const void* A, int64_t lda,
+                             const void* B, const void* bias, const void* R, int64_t ldr, void* C, int64_t ldc,
+                             void* stream);
+
 /* Size of the workspace that fire_local_energy_static() owns (32 MiB). */
 #define FIRE_STATIC_WORKSPACE_BYTES (32u * 1024u * 1024u)
 

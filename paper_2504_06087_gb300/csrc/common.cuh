@@ -75,6 +75,12 @@ __device__ __forceinline__ void fma_pair(double& c0, double& c1, double a, doubl
   c1 = fma(a, b1, c1);
 }
 
+// A sum and a product that are never contracted into one multiply-add.
+__device__ __forceinline__ float add_rn(float a, float b) { return __fadd_rn(a, b); }
+__device__ __forceinline__ double add_rn(double a, double b) { return __dadd_rn(a, b); }
+__device__ __forceinline__ float mul_rn(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ double mul_rn(double a, double b) { return __dmul_rn(a, b); }
+
 // SiLU and its first two derivatives: s = logistic(x),
 // f = x s, f' = s (1 + x (1 - s)), f'' = s (1 - s) (2 + x (1 - 2 s)).
 template <typename T>

@@ -33,6 +33,7 @@ struct GemmArgs {
   const T* bias;                 // ACT: C = (R ? R : 0) + SiLU(product + bias), R with row stride ldr
   const T* R;
   int64_t ldr;
+  int one;                       // ACT: R is added to x * logistic(x) in one rounding or in two
 };
 
 // One BM x BN tile per CTA; a thread owns TM x TN outputs as groups of at most
@@ -183,12 +184,38 @@ gemm_kernel(GemmArgs<T> g) {
     if (gm >= me) continue;
     if constexpr (ACT) {
 #pragma unroll
-      for (int j = 0; j < TN; ++j) {
-        const int gn = n0 + (j / GN) * (BN / RN) + tx * GN + j % GN;
-        if (gn >= g.N) continue;
-        T f, f1, f2;
-        silu3<T>(acc[i][j] + g.bias[gn], f, f1, f2);
-        C[gm * g.ldc + gn] = g.R ? g.R[gm * g.ldr + gn] + f : f;
+      for (int p = 0; p < RN; ++p) {
+        const int gn = n0 + p * (BN / RN) + tx * GN;
+        T* o = C + gm * g.ldc + gn;
+        const T* rr = g.R ? g.R + gm * g.ldr + gn : nullptr;
+        const bool whole = g.vc && gn + GN <= g.N;   // (R is as aligned as C then)
+        T y[GN];
+        if (whole && rr) ld_vec<T, GN>(y, rr);
+        else
+#pragma unroll
+          for (int j = 0; j < GN; ++j) y[j] = rr && gn + j < g.N ? rr[j] : T(0);
+#pragma unroll
+        for (int j = 0; j < GN; ++j) {
+          const T x = acc[i][p * GN + j] + (gn + j < g.N ? g.bias[gn + j] : T(0));
+          const T sg = T(1) / (T(1) + dexp<T>(-x));
+          const T f = mul_rn(x, sg);
+          y[j] = !rr ? f : g.one ? fma(x, sg, y[j]) : add_rn(y[j], f);
+        }
+        if (whole) {
+          constexpr int W = VE < GN ? VE : GN;
+          struct alignas(W * sizeof(T)) Vec { T x[W]; };
+#pragma unroll
+          for (int q = 0; q < GN; q += W) {
+            Vec u;
+#pragma unroll
+            for (int j = 0; j < W; ++j) u.x[j] = y[q + j];
+            *reinterpret_cast<Vec*>(o + q) = u;
+          }
+        } else {
+#pragma unroll
+          for (int j = 0; j < GN; ++j)
+            if (gn + j < g.N) o[j] = y[j];
+        }
       }
       continue;
     }
@@ -233,7 +260,10 @@ inline void gemm_launch(cudaStream_t s, const GemmArgs<T>& g, bool tb, int64_t m
 // Host launcher.  m_cap bounds end - begin (grid sizing).  With bias (plain
 // products only) the epilogue is a SiLU layer, C = (R ? R : 0) + SiLU(A B + bias):
 // a move's products are so short that the layer's own launch took a third of
-// their time.  C must not be A or R's rows of another tile (R may be A).
+// their time.  C must not be A or R's rows of another tile (R may be A).  With
+// `one` the residual sum is a single multiply-add, as in mcmc_act_kernel;
+// without it product and sum are rounded one by one, as in fl_act4_kernel: a
+// row comes out the same whichever kernel took its layer.
 //
 // float32: tiles of 64 x 64 (64 threads, 8 x 8 outputs each, 168 registers)
 // reach 55-59 of the 77 TFLOP/s of plain multiply-adds once a few tiles per SM
@@ -252,10 +282,10 @@ inline void gemm(cudaStream_t s, const T* A, int64_t lda, const T* B, int64_t ld
                  T* C, int64_t ldc, int64_t m_begin, int64_t m_end, const int64_t* m_range,
                  int64_t m_cap, int N, int K, int batch = 1, int64_t sA = 0, int64_t sB = 0,
                  int64_t sC = 0, bool accumulate = false, const T* bias = nullptr, const T* R = nullptr,
-                 int64_t ldr = 0) {
+                 int64_t ldr = 0, int one = 0) {
   if (m_cap <= 0 || N <= 0 || K <= 0 || batch <= 0) return;
   GemmArgs<T> g{A, B, C, lda, ldb, ldc, sA, sB, sC, m_begin, m_end, m_range, N, K, N, accumulate ? 1 : 0, 0, 0, 0,
-                bias, R, ldr};
+                bias, R, ldr, one};
   if (bias && (transB || batch != 1 || accumulate)) return;   // the fused layer is a plain product
   if (batch > 1 && sA == 0 && sC == N) {   // side by side: one product of batch * N columns
     g.N = N * batch;
@@ -265,7 +295,7 @@ inline void gemm(cudaStream_t s, const T* A, int64_t lda, const T* B, int64_t ld
   auto al = [](const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; };
   g.va = al(A) && lda % VE == 0 && K % VE == 0 && sA % VE == 0;
   g.vb = al(B) && ldb % VE == 0 && sB % VE == 0 && (transB ? K : N) % VE == 0;
-  g.vc = al(C) && ldc % VE == 0 && sC % VE == 0;
+  g.vc = al(C) && ldc % VE == 0 && sC % VE == 0 && (!R || (al(R) && ldr % VE == 0));
   if constexpr (sizeof(T) == 8) {
     gemm_launch<T, 16, 16, 32, 1, 2>(s, g, transB, m_cap, batch);
   } else {

@@ -93,8 +93,9 @@ static __global__ void nbr_reverse_kernel(int n, int n_up, int K, const int32_t*
   }
 }
 
-// Exclusive scan of block row counts -> blk_off[0..nb]; ranges[0..3] =
-// {up_begin, up_end, down_begin, down_end} rows.  One CTA of 1024 threads.
+// Exclusive scan of block row counts -> blk_off[0..nb]; ranges[0..5] =
+// {up_begin, up_end, down_begin, down_end, 0, total} rows.  One CTA of 1024
+// threads.
 static __global__ void blk_scan_kernel(int nb, int nb_up, const int64_t* __restrict__ rows,
                                 int64_t* __restrict__ off, int64_t* __restrict__ ranges,
                                 DevStatus* st) {
@@ -130,6 +131,24 @@ static __global__ void blk_scan_kernel(int nb, int nb_up, const int64_t* __restr
     ranges[1] = mid;
     ranges[2] = mid;
     ranges[3] = part[T - 1];
+    ranges[4] = 0;
+    ranges[5] = part[T - 1];
+  }
+}
+
+// The same layout for value rows alone: block b is row b.
+static __global__ void blk_unit_kernel(int nb, int nb_up, int64_t* __restrict__ off, int64_t* __restrict__ ranges,
+                                       DevStatus* st) {
+  const int t = blockIdx.x * blockDim.x + threadIdx.x;
+  for (int b = t; b <= nb; b += gridDim.x * blockDim.x) off[b] = b;
+  if (t == 0) {
+    ranges[0] = 0;
+    ranges[1] = nb_up;
+    ranges[2] = nb_up;
+    ranges[3] = nb;
+    ranges[4] = 0;
+    ranges[5] = nb;
+    st->rows_total += nb;
   }
 }
 

@@ -346,6 +346,12 @@ struct Runner {
     fl_act_kernel<T, T><<<nblk, 256, 0, s>>>(ncol, off, stride, Z, ldz, bias, Y, ldy, residual, Yb, ync, ycs, yall);
   }
 
+  // Y = (R ? R : 0) + SiLU(A w + b) over rows [0, rows) (Y is neither A nor R)
+  void value_layer(const T* A, int64_t lda, const T* w, const T* b, T* Y, int64_t ldy, int64_t rows, int No, int Ki,
+                   const T* R = nullptr, int64_t ldr = 0) {
+    gemm<T>(s, A, lda, w, No, false, Y, ldy, 0, rows, nullptr, rows, No, Ki, 1, 0, 0, 0, false, b, R, ldr);
+  }
+
   // SiLU-MLP readout with two hidden layers over ragged blocks (rows of X
   // given by blk offsets or a fixed stride) -> per-row scalar F.
   void mlp_readout(const T* Xin, const __nv_bfloat16* Xinb, int64_t ldx, int din, const int64_t* range,
@@ -356,6 +362,13 @@ struct Runner {
     const int J = dm.J;
     if (a_rows < 0) a_rows = capA;   // rows between the bf16 components of Xinb and Yb
     if (nc < 0) nc = nc_jas;
+    const int max_rows = off ? (int)pl.rows_per_el : (int)stride;
+    if (!w1b && !w2b && max_rows == 1) {   // value rows, SIMT: row b is block b
+      value_layer(Xin, ldx, w1, b1, Y, ldy, nblk, J, din);
+      gemm<T>(s, Y, ldy, w2, J, false, Z, ldz, 0, nblk, nullptr, nblk, J, J);
+      fl_act_dot_kernel<T, T><<<nblk, 256, (size_t)8 * sizeof(T), s>>>(J, nullptr, 1, Z, ldz, b2, w3, F, 1);
+      return;
+    }
     row_gemm(Xin, Xinb, ldx, a_rows, w1, w1b, J, Z, ldz, range, rb, re, cap, J, din, nc);
     // the hidden layer feeds a tensor-core product through Yb: of the float
     // rows only the value rows (read again in fp32) are stored; should the
@@ -367,7 +380,6 @@ struct Runner {
       gemm<T>(s, Y, ldy, w2, J, false, Z, ldz, rb, re, range, cap, J, J);
     }
     // last activation fused with the readout vector: F = act(Z + b2) . w3
-    const int max_rows = off ? (int)pl.rows_per_el : (int)stride;
     fl_act_dot_kernel<T, T><<<nblk, 256, (size_t)8 * max_rows * sizeof(T), s>>>(J, off, stride, Z, ldz, b2, w3, F,
                                                                                max_rows);
   }
@@ -428,10 +440,9 @@ struct Runner {
         launches += 1;
       };
       // ---- forward (value rows: one row per electron block) ----
-      mark("neighbors", 3);
+      mark("neighbors", 2);
       nbr_build_kernel<<<wc, 256, (size_t)n * 3 * sizeof(double), s>>>(wc, n, n_up, r, c * c, K, idx, cnt, brow, st, 0);
-      nbr_reverse_kernel<<<wc, 256, 0, s>>>(n, n_up, K, idx, cnt, rev);
-      blk_scan_kernel<<<1, 1024, 0, s>>>(nb, wc * n_up, brow, boff, rng, st);
+      blk_unit_kernel<<<nb / 4096 + 1, 256, 0, s>>>(nb, wc * n_up, boff, rng, st);
       T* S5 = at<T>(pl.S5);
       T* Y5 = at<T>(pl.Y5);
       T* Z5 = at<T>(pl.Z5);
@@ -784,11 +795,15 @@ struct Runner {
       int64_t* rng = at<int64_t>(pl.ranges);
       const double c = sys->cutoff;
       // 1. neighbour lists and the ragged row layout
-      mark("neighbors", 3);
+      mark("neighbors", deriv ? 3 : 2);
       nbr_build_kernel<<<wc, 256, (size_t)n * 3 * sizeof(double), s>>>(wc, n, n_up, r, c * c, K, idx, cnt,
                                                                         brow, st, deriv);
-      nbr_reverse_kernel<<<wc, 256, 0, s>>>(n, n_up, K, idx, cnt, rev);
-      blk_scan_kernel<<<1, 1024, 0, s>>>(nb, wc * n_up, brow, boff, rng, st);
+      if (deriv) {
+        nbr_reverse_kernel<<<wc, 256, 0, s>>>(n, n_up, K, idx, cnt, rev);
+        blk_scan_kernel<<<1, 1024, 0, s>>>(nb, wc * n_up, brow, boff, rng, st);
+      } else {
+        blk_unit_kernel<<<nb / 4096 + 1, 256, 0, s>>>(nb, wc * n_up, boff, rng, st);
+      }
       // float forms with aligned rows: the tangent electrons sorted into the
       // contraction buckets by neighbourhood size
       const char* cenv = getenv("FIRE_CONTRACT");
@@ -810,18 +825,18 @@ struct Runner {
         launches += 1;
       }
       check("nbr");
-      // the chunk's row total and largest neighbour count, read back once:
-      // they size the grids and the contraction tiles exactly
-      int64_t rows_chunk = 0;
+      // the chunk's row total and largest neighbour count, read back once: they
+      // size the grids and the contraction tiles exactly.  Value rows alone are
+      // one per block: nothing to read back (and nothing to wait for).
+      int64_t rows_chunk = nb;
       int32_t kreq = 0;
-      cudaMemcpyAsync(&rows_chunk, rng + 3, sizeof(int64_t), cudaMemcpyDeviceToHost, s);
-      cudaMemcpyAsync(&kreq, &st->k_required, sizeof(int32_t), cudaMemcpyDeviceToHost, s);
-      if (cudaStreamSynchronize(s) != cudaSuccess) return FIRE_ERR_CUDA;
+      if (deriv) {
+        cudaMemcpyAsync(&rows_chunk, rng + 3, sizeof(int64_t), cudaMemcpyDeviceToHost, s);
+        cudaMemcpyAsync(&kreq, &st->k_required, sizeof(int32_t), cudaMemcpyDeviceToHost, s);
+        if (cudaStreamSynchronize(s) != cudaSuccess) return FIRE_ERR_CUDA;
+      }
       const int64_t cap = rows_chunk > 0 ? rows_chunk : 1;
-      int64_t* fullr = at<int64_t>(pl.ranges) + 4;
-      // fullr = {0, total}: written by a tiny copy below
-      cudaMemcpyAsync(fullr, rng, sizeof(int64_t), cudaMemcpyDeviceToDevice, s);
-      cudaMemcpyAsync(fullr + 1, rng + 3, sizeof(int64_t), cudaMemcpyDeviceToDevice, s);
+      const int64_t* fullr = rng + 4;   // {0, rows of the chunk}
 
       // 2. initial embeddings h^0 (5 rows per electron)
       T* S5 = at<T>(pl.S5);
@@ -905,7 +920,20 @@ struct Runner {
       vr_cap = (int64_t)pl.Wc * dm.n;
       vr_kmax = dm.d;
       const int64_t ldb = pl.ld_big;
-      for (int l = 0; l < dm.L; ++l) {
+      // value rows of the SIMT forms: pairs of layers X -> Z -> X with the SiLU in
+      // the products' epilogues (an odd first layer in place)
+      const bool vsimt = !deriv && !pl.wbf16;
+      if (vsimt && (dm.L & 1)) {
+        mark("mlp_gemm", 2);
+        gemm<T>(s, X, d, p.mlp_w, d, false, Z, ldb, 0, nb, nullptr, nb, d, d);
+        fl_act(d, boff, 0, Z, ldb, p.mlp_b, X, d, 1, nullptr, 0, 0, 1, nb);
+      }
+      for (int l = dm.L & 1; vsimt && l < dm.L; l += 2) {
+        mark("mlp_gemm", 2);
+        value_layer(X, d, p.mlp_w + (int64_t)l * d * d, p.mlp_b + (int64_t)l * d, Z, ldb, nb, d, d, X, d);
+        value_layer(Z, ldb, p.mlp_w + (int64_t)(l + 1) * d * d, p.mlp_b + (int64_t)(l + 1) * d, X, d, nb, d, d, Z, ldb);
+      }
+      for (int l = 0; l < (vsimt ? 0 : dm.L); ++l) {
         mark("mlp_gemm", 1);
         row_gemm(X, Xb, d, capA, p.mlp_w + (int64_t)l * d * d, wbm(0, pl.wb_mlp + kMaxSplit * (int64_t)l * d * d),
                  d, Z, ldb, fullr, 0, 0, cap, d, d, nc_mlp);
@@ -1338,7 +1366,7 @@ struct Runner {
     // SiLU layer Y = (R ? R : 0) + SiLU(A w + b) over rows [rng[0], rng[1]) (Y is neither A nor R)
     auto layer = [&](const T* A, int64_t lda, const T* w, const T* b, T* Yl, int64_t ldy, const int64_t* rng,
                      int64_t cap, int No, int Ki, const T* Rl = nullptr, int64_t ldr = 0) {
-      gemm<T>(s, A, lda, w, No, false, Yl, ldy, 0, 0, rng, cap, No, Ki, 1, 0, 0, 0, false, b, Rl, ldr);
+      gemm<T>(s, A, lda, w, No, false, Yl, ldy, 0, 0, rng, cap, No, Ki, 1, 0, 0, 0, false, b, Rl, ldr, 1);
       launches += 1;
     };
     // two-hidden-layer SiLU readout over rows [rng[0], rng[1]); Zb has row stride ldzb
@@ -1643,6 +1671,15 @@ inline int set_smem_limits() {
   int dev = 0, maxopt = 0;
   if (cudaGetDevice(&dev) != cudaSuccess) return FIRE_ERR_CUDA;
   cudaDeviceGetAttribute(&maxopt, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+  // the last kernel raised below tells whether all of them are, in the
+  // device's current context (25 attribute queries and 50 settings a call
+  // cost a small call 25 us of host time before its first launch)
+  const void* last = (const void*)gj_inverse_pre_kernel<float, T>;
+  {
+    cudaFuncAttributes at;
+    if (cudaFuncGetAttributes(&at, last) != cudaSuccess) return FIRE_ERR_CUDA;
+    if (at.maxDynamicSharedSizeBytes >= maxopt - (int)at.sharedSizeBytes) return FIRE_OK;
+  }
   int rc = FIRE_OK;
   auto raise = [&](const void* fn) {
     cudaFuncAttributes at;
@@ -1672,7 +1709,6 @@ inline int set_smem_limits() {
   raise((const void*)lu_kernel<LT, 32>);
   raise((const void*)att_pool_kernel<T>);
   raise((const void*)gj_inverse_kernel<float, T>);
-  raise((const void*)gj_inverse_pre_kernel<float, T>);
   raise((const void*)mcmc_att_kernel<T>);
   raise((const void*)msg_bwd_kernel<T, T>);
   raise((const void*)en_bwd_kernel<T, T>);
@@ -1683,6 +1719,7 @@ inline int set_smem_limits() {
   raise((const void*)mcmc_woodbury_panel_kernel<T, 12>);
   raise((const void*)mcmc_repair_kernel<T, LT>);
   raise((const void*)inverse_warp_kernel<LT, T>);
+  if (rc == FIRE_OK) raise(last);
   cudaError_t e = cudaGetLastError();
   if (rc != FIRE_OK || e != cudaSuccess) set_last_error("smem limits", cudaGetErrorString(e));
   return rc;

@@ -84,3 +84,19 @@ extern "C" int fire_selftest_simt_gemm(int32_t dtype, int64_t M, int32_t N, int3
                       K, batch, 0, sB, sC, accumulate != 0);
   return cudaGetLastError() == cudaSuccess ? FIRE_OK : FIRE_ERR_CUDA;
 }
+
+extern "C" int fire_selftest_simt_layer(int32_t dtype, int64_t M, int32_t N, int32_t K, int32_t one, const void* A,
+                                        int64_t lda, const void* B, const void* bias, const void* R, int64_t ldr,
+                                        void* C, int64_t ldc, void* stream) {
+  if ((dtype != 0 && dtype != 1) || M < 1 || N < 1 || K < 1 || lda < K || ldc < N || !A || !B || !bias || !C ||
+      (R && ldr < N))
+    return FIRE_ERR_INVALID_ARG;
+  cudaStream_t s = (cudaStream_t)stream;
+  if (dtype == 0)
+    fire::gemm<double>(s, (const double*)A, lda, (const double*)B, N, false, (double*)C, ldc, 0, M, nullptr, M, N, K, 1,
+                       0, 0, 0, false, (const double*)bias, (const double*)R, ldr, one != 0);
+  else
+    fire::gemm<float>(s, (const float*)A, lda, (const float*)B, N, false, (float*)C, ldc, 0, M, nullptr, M, N, K, 1, 0,
+                      0, 0, false, (const float*)bias, (const float*)R, ldr, one != 0);
+  return cudaGetLastError() == cudaSuccess ? FIRE_OK : FIRE_ERR_CUDA;
+}

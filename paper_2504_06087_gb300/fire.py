@@ -125,6 +125,9 @@ SIGNATURES = {
                                                ctypes.c_int32, ctypes.c_int32, ctypes.c_int32, VP, ctypes.c_int64, VP,
                                                ctypes.c_int64, ctypes.c_int64, VP, ctypes.c_int64, ctypes.c_int64,
                                                VP]),
+    "fire_selftest_simt_layer": (ctypes.c_int, [ctypes.c_int32, ctypes.c_int64, ctypes.c_int32, ctypes.c_int32,
+                                                ctypes.c_int32, VP, ctypes.c_int64, VP, VP, VP, ctypes.c_int64, VP,
+                                                ctypes.c_int64, VP]),
     "fire_selftest_fma_rate": (ctypes.c_int, [ctypes.c_int32, ctypes.c_int64, ctypes.c_int32, VP, VP]),
     "fire_spring_workspace_size": (ctypes.c_size_t, [ctypes.c_int64, ctypes.c_int64]),
     "fire_spring_step": (ctypes.c_int, [ctypes.c_int64, ctypes.c_int64, VP, ctypes.c_int64, VP, VP, ctypes.c_double,

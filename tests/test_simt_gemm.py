@@ -47,3 +47,37 @@ def test_simt_gemm_matches_float64_product(dtype, M, N, K, batch, tb, off, acc):
     bound = 1.01 * (K + acc) * (u + 2.0 ** -53) * mag
     assert ((C[:, :batch * N].double() - ref).abs() <= bound).all()
     assert torch.equal(C[:, batch * N:], C0[:, batch * N:])   # nothing beyond the columns
+
+
+# M, N, K, residual, one, offset of R and C (elements: unaligned rows take scalar loads and stores)
+LAYERS = [
+    (1, 1, 1, 0, 0, 0), (33, 30, 17, 1, 0, 0), (64, 64, 64, 1, 1, 0), (65, 62, 64, 1, 1, 1), (300, 128, 128, 0, 0, 0),
+    (257, 128, 96, 1, 0, 0), (20011, 256, 64, 1, 1, 0), (20011, 180, 33, 1, 0, 1), (40000, 17, 33, 1, 1, 0),
+]
+
+
+@pytest.mark.parametrize("dtype", [torch.float32, torch.float64])
+@pytest.mark.parametrize("M,N,K,res,one,off", LAYERS)
+def test_simt_layer_matches_float64_layer(dtype, M, N, K, res, one, off):
+    """The product's bound carried through SiLU (its slope is below 1.1), plus
+    the rounding of bias, logistic (exp, sum, quotient), product and sum."""
+    g = torch.Generator(device="cpu").manual_seed(3 * M + N + K)
+    rnd = lambda *q: torch.randn(*q, generator=g, dtype=torch.float64).to(dtype).cuda()
+    A, B, b = rnd(M, K), rnd(K, N), rnd(N)
+    R, C = (rnd(off + M * (N + 4))[off:].view(M, N + 4) for _ in range(2))
+    C0 = C.clone()
+    vp = ctypes.c_void_p
+    rc = fire.lib().fire_selftest_simt_layer(
+        0 if dtype == torch.float64 else 1, M, N, K, one, vp(A.data_ptr()), K, vp(B.data_ptr()), vp(b.data_ptr()),
+        vp(R.data_ptr()) if res else None, R.stride(0), vp(C.data_ptr()), C.stride(0),
+        vp(torch.cuda.current_stream().cuda_stream))
+    assert rc == 0
+    torch.cuda.synchronize()
+    x = A.double() @ B.double() + b.double()
+    f = x * torch.sigmoid(x)
+    ref = f + R[:, :N].double() if res else f
+    u = (2.0 ** -53 if dtype == torch.float64 else 2.0 ** -24) + 2.0 ** -53
+    mag = A.double().abs() @ B.double().abs() + b.double().abs()
+    bound = 1.1 * 1.01 * (K + 2) * u * mag + 10 * u * f.abs() + 2 * u * ref.abs() + 1e-30
+    assert ((C[:, :N].double() - ref).abs() <= bound).all()
+    assert torch.equal(C[:, N:], C0[:, N:])
