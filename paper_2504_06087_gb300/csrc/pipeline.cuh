@@ -1671,10 +1671,11 @@ inline int set_smem_limits() {
   int dev = 0, maxopt = 0;
   if (cudaGetDevice(&dev) != cudaSuccess) return FIRE_ERR_CUDA;
   cudaDeviceGetAttribute(&maxopt, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-  // the last kernel raised below tells whether all of them are, in the
-  // device's current context (25 attribute queries and 50 settings a call
-  // cost a small call 25 us of host time before its first launch)
-  const void* last = (const void*)gj_inverse_pre_kernel<float, T>;
+  // the last kernel raised below (one that no other form raises) tells whether
+  // all of this form's are, in the device's current context (25 attribute
+  // queries and 50 settings a call cost a small call 25 us of host time before
+  // its first launch)
+  const void* last = (const void*)inverse_warp_kernel<LT, T>;
   {
     cudaFuncAttributes at;
     if (cudaFuncGetAttributes(&at, last) != cudaSuccess) return FIRE_ERR_CUDA;
@@ -1718,7 +1719,7 @@ inline int set_smem_limits() {
   raise((const void*)mcmc_woodbury_panel_kernel<T, 8>);
   raise((const void*)mcmc_woodbury_panel_kernel<T, 12>);
   raise((const void*)mcmc_repair_kernel<T, LT>);
-  raise((const void*)inverse_warp_kernel<LT, T>);
+  raise((const void*)gj_inverse_pre_kernel<float, T>);
   if (rc == FIRE_OK) raise(last);
   cudaError_t e = cudaGetLastError();
   if (rc != FIRE_OK || e != cudaSuccess) set_last_error("smem limits", cudaGetErrorString(e));
