@@ -901,15 +901,27 @@ contract_kernel(int Wc, int n, int n_up, int K, int mcap, int dd, int D, const i
   }
 }
 
-// Four consecutive elements p[l .. l+3] (zero beyond n; 128-bit load when
-// the row slice is 16-byte aligned, i.e. n % 4 == 0).
-__device__ __forceinline__ float4 ld_row4(const float* __restrict__ p, int l, int n, bool vec) {
-  if (vec) return l < n ? __ldg(reinterpret_cast<const float4*>(p + l)) : make_float4(0.f, 0.f, 0.f, 0.f);
-  float4 v;
-  v.x = l < n ? __ldg(p + l) : 0.f;
-  v.y = l + 1 < n ? __ldg(p + l + 1) : 0.f;
-  v.z = l + 2 < n ? __ldg(p + l + 2) : 0.f;
-  v.w = l + 3 < n ? __ldg(p + l + 3) : 0.f;
+// Four consecutive elements p[l .. l+3] (zero beyond n), l < n a multiple of
+// 4, by loads of vw elements: 4 where n % 4 == 0 (every row slice is 16-byte
+// aligned then), 2 where n is even, else 1.
+__device__ __forceinline__ float4 ld_row4(const float* __restrict__ p, int l, int n, int vw) {
+  if (vw == 4) return __ldg(reinterpret_cast<const float4*>(p + l));
+  float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+  if (vw == 2) {
+    const float2 a = __ldg(reinterpret_cast<const float2*>(p + l));
+    v.x = a.x;
+    v.y = a.y;
+    if (l + 2 < n) {
+      const float2 b = __ldg(reinterpret_cast<const float2*>(p + l + 2));
+      v.z = b.x;
+      v.w = b.y;
+    }
+    return v;
+  }
+  v.x = __ldg(p + l);
+  if (l + 1 < n) v.y = __ldg(p + l + 1);
+  if (l + 2 < n) v.z = __ldg(p + l + 2);
+  if (l + 3 < n) v.w = __ldg(p + l + 3);
   return v;
 }
 
@@ -918,10 +930,13 @@ __device__ __forceinline__ float4 ld_row4(const float* __restrict__ p, int l, in
 // NT threads per (walker, tangent electron n'); thread tile = 3 members x 3
 // coordinates (9 rows of T) x 4 member columns of A, so every orbital l costs
 // four 128-bit shared loads for 36 FMAs.  Orbitals go in chunks of 32: each
-// staging item (member k, 4 orbitals) reads 128-bit slices of k's three O
-// rows, its envelope row and its row of A^T and writes the T quads
-// (x = 0, 1, 2, pad) member-contiguous, so neither the gathers nor the shared
-// stores conflict.  Neighbourhood sizes are bucketed: a CTA whose member
+// staging item (member k, 4 orbitals) reads slices of k's three O rows, its
+// envelope row and its row of A^T and writes the T quads (x = 0, 1, 2, pad)
+// member-contiguous.  Eight lanes take the eight slices of one row: with the
+// members on neighbouring lanes and scalar loads for n % 4 != 0 every load
+// instruction touched 32 rows, and their L1 wavefronts, about five times the
+// multiply-adds' shared loads, bounded the kernel (n = 58, 512 walkers, 8
+// determinants: 7.98 ms, now 5.45).  Neighbourhood sizes are bucketed: a CTA whose member
 // count m lies outside [mlo, mhi] exits at once, so one launch per bucket
 // sizes its tiles and shared memory for that bucket only.
 //   MP = member slots of the bucket (>= every tile's member and column, multiple of 4)
@@ -992,7 +1007,7 @@ contract2_kernel(int Wc, int n, int n_up, int K, int mlo, int mhi, int dd, int D
   const float* Aw = AT + ((int64_t)w * D + dd) * n * n;
   const int bnp = block_index(w, np, Wc, n, n_up);
   const int64_t onp = blk_off[bnp] * ldo;
-  const bool vec = (n & 3) == 0 && (ldo & 3) == 0;
+  const int vec = ((n | (int)ldo) & 3) == 0 ? 4 : (((n | (int)ldo) & 1) == 0 ? 2 : 1);
 
   // sum_l LapPhi_{n' l} A_{l n'}: the Laplacian row of n' against A's column n'
   float lt = 0.f;
@@ -1017,10 +1032,13 @@ contract2_kernel(int Wc, int n, int n_up, int K, int mlo, int mhi, int dd, int D
 
   for (int l0 = 0; l0 < n; l0 += LC) {
     __syncthreads();   // the previous chunk is consumed
-    // staging items (member k, orbitals l0 + 4 q4 .. + 3), members fastest
+    // staging items (member k, orbitals l0 + 4 q4 .. + 3), orbitals fastest;
+    // slices beyond n are neither staged nor multiplied
+    const int lc = min(LC, n - l0);
     for (int e = tid; e < kfill * (LC / 4); e += NT) {
-      const int k = e % kfill, q4 = e / kfill;
+      const int k = e / (LC / 4), q4 = e % (LC / 4);
       const int l = l0 + 4 * q4;
+      if (l >= n) continue;
       float4 t0 = make_float4(0.f, 0.f, 0.f, 0.f), t1 = t0, t2 = t0, av = t0;
       if (k < m) {
         const float4 ph = ld_row4(Fenv + fo[k], l, n, vec);
@@ -1063,7 +1081,7 @@ contract2_kernel(int Wc, int n, int n_up, int K, int mlo, int mhi, int dd, int D
         const float* tp = Ts + 12 * kg;
         const float* ap = As + 4 * cg;
 #pragma unroll 4
-        for (int q = 0; q < LC; ++q) {
+        for (int q = 0; q < lc; ++q) {
           const float4 a0 = *reinterpret_cast<const float4*>(tp + q * ST);
           const float4 a1 = *reinterpret_cast<const float4*>(tp + q * ST + 4);
           const float4 a2 = *reinterpret_cast<const float4*>(tp + q * ST + 8);
