@@ -140,7 +140,9 @@ typedef struct {
 
 /* Network hyper-parameters (Supplementary table "Hyperparameters"). */
 typedef struct {
-  int32_t width;             /* hidden width d (multiple of 8, <= 1024)         */
+  int32_t width;             /* hidden width d: a multiple of 32 up to 512 (FP32,
+                                BF16_FP64) or 256 (FP64, and the gradient in
+                                every form); wider: FIRE_ERR_UNSUPPORTED         */
   int32_t n_layers;          /* depth L of the embedding MLP h = MLP(h^1)       */
   int32_t n_det;             /* determinants N_det                              */
   int32_t n_env;             /* exponential envelopes per nucleus               */

@@ -276,12 +276,20 @@ static size_t budget_bytes() {
   return (size_t)(mb * 1024.0 * 1024.0);
 }
 
+// Widest network that the kernels of a call can be launched for: those with
+// one thread per column hold a column's weights in registers.
+static int max_width(int prec, int op) {
+  if (op == FIRE_OP_GRAD_LOGPSI) return kGradThreads;
+  return prec == FIRE_PREC_FP64 ? kFilterThreads<double> : kFilterThreads<float>;
+}
+
 int make_plan(const fire_system_t* sys, const fire_arch_t* ar, int64_t W, int prec, int k_cap, int op,
               Plan* pl) {
   int rc = check_system(sys, ar);
   if (rc) return rc;
   if (W < 1 || k_cap < 1 || k_cap > 1024) return FIRE_ERR_INVALID_ARG;
   if (prec < 0 || prec > 2) return FIRE_ERR_INVALID_ARG;
+  if (ar->width > max_width(prec, op)) return FIRE_ERR_UNSUPPORTED;
   // Metropolis moves of both reduced forms run in float32
   if (op == FIRE_OP_MCMC && prec == FIRE_PREC_BF16_FP64) prec = FIRE_PREC_FP32;
   memset(pl, 0, sizeof(Plan));

@@ -61,7 +61,10 @@ constexpr int kPairBatch = 16;
 // Largest nucleus count of the batched electron-nucleus filter.
 constexpr int kMaxNuc = 512;
 // Widest CTA (one thread per column) whose registers the filter kernels have
-// to fit: 128 a thread in float32, 255 in float64.
+// to fit: 128 a thread in float32, 255 in float64 (registers are given to the
+// four quarters of an SM in whole warps, so a CTA of 9 warps takes as many as
+// one of 12: the next width in float64 would leave 168 a thread, which spills).
+// The plan refuses wider networks (max_width).
 template <typename T>
 constexpr int kFilterThreads = sizeof(T) == 4 ? 512 : 256;
 // Filter features of a pair, hidden units first, then Gaussians, then e-bar.

@@ -176,6 +176,8 @@ __global__ void att_bwd_kernel(int Wc, int n, int n_up, int R, int dr, const T* 
 // message pass 18.0 ms; now 3.8 and 4.3 ms.
 // ---------------------------------------------------------------------------
 constexpr int kGradPairs = 16;
+// Widest CTA of the two kernels (two of them per SM in float32).
+constexpr int kGradThreads = 256;
 
 template <typename T>
 struct FilterGrad {
@@ -316,7 +318,7 @@ struct FilterWeights {
 // (atomics at j), parameter gradients of the e-e filter, W^alpha_c and b^alpha.
 constexpr int kGradElectrons = 8;   // largest epc
 template <typename T, typename W>
-__global__ void __launch_bounds__(256, sizeof(T) == 4 ? 2 : 1) msg_bwd_kernel(
+__global__ void __launch_bounds__(kGradThreads, sizeof(T) == 4 ? 2 : 1) msg_bwd_kernel(
     int Wc, int n, int n_up, int d, int K, int epc, const double* __restrict__ r, double cut, Params<W> p,
     const int32_t* __restrict__ idx, const int32_t* __restrict__ cnt, const T* __restrict__ PQ,
     const T* __restrict__ dH1, T* __restrict__ dP, T* __restrict__ dQ, T* __restrict__ grad, int64_t P,
@@ -445,7 +447,7 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 2 : 1) msg_bwd_kernel(
 // nucleus's own weights (h^nuc_m, W_1m, b_1m) are summed within the CTA.
 constexpr int kGradSeg = 256;
 template <typename T, typename W>
-__global__ void __launch_bounds__(256, sizeof(T) == 4 ? 2 : 1) en_bwd_kernel(
+__global__ void __launch_bounds__(kGradThreads, sizeof(T) == 4 ? 2 : 1) en_bwd_kernel(
     int Wc, int n, int n_up, int N, int d, int seg, const double* __restrict__ r, const double* __restrict__ R,
     double cnuc, Params<W> p, const T* __restrict__ dS, T* __restrict__ grad, int64_t P,
     const int64_t* __restrict__ po) {
