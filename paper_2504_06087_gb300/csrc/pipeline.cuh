@@ -1311,6 +1311,14 @@ struct Runner {
     int32_t* flag = at<int32_t>(pl.mc_flag);
     int32_t* xflag = at<int32_t>(pl.mc_xflag);
     int32_t* stale = at<int32_t>(pl.mc_stale);
+    // pairs that the lists of exact ratios, refactorisations and late inverses
+    // hold; FIRE_MCMC_LIST (diagnostic) shortens them, so that the kernels that
+    // take the pairs beyond can be tested on small batches
+    int xcap = pl.xcap;
+    if (const char* e = getenv("FIRE_MCMC_LIST")) {
+      const int v = atoi(e);
+      if (v >= 1 && v < xcap) xcap = v;
+    }
     // the state, in the value-forward buffers
     T* H0 = at<T>(pl.H0);
     T* PQ = at<T>(pl.PQ);
@@ -1452,17 +1460,17 @@ struct Runner {
         int32_t* xlist = at<int32_t>(pl.mc_xlist);
         int32_t* pend = mc.ecp || mc.swap_beta >= 0 ? nullptr : stale;   // nothing is accepted there
         // only a batch beyond the lists' capacity leaves any pair to the per-CTA kernels
-        int32_t* xover = npair > pl.xcap ? at<int32_t>(pl.mc_flag) : nullptr;
+        int32_t* xover = npair > xcap ? at<int32_t>(pl.mc_flag) : nullptr;
         LT* xb0 = at<LT>(pl.mc_xbatch);
         mark("mc_inverse", 1);
         cudaMemsetAsync(xcnt, 0, 2 * sizeof(int), s);
         mcmc_exact_test_kernel<<<(unsigned)((npair + 127) / 128), 128, 0, s>>>(
-            npair, D, Uc, ldabs, lsign, kap, kunit, mc.kappa_tol, xflag, pend, xcnt + 1, xlist, pl.xcap, xover);
+            npair, D, Uc, ldabs, lsign, kap, kunit, mc.kappa_tol, xflag, pend, xcnt + 1, xlist, xcap, xover);
         if (pend) {
           int32_t* xpiv = at<int32_t>(pl.mc_xpiv);
-          mcmc_repair_build_kernel<T, LT><<<pl.xcap, 256, 0, s>>>(n, xcnt + 1, xlist, PhiS, xb0);
-          lu_batch<LT>(s, n, pl.xcap, xb0, xpiv, at<double>(pl.mc_xlab), at<double>(pl.mc_xsg), xcnt + 1);
-          inverse_warp<T>(n, pl.xcap, xb0, xpiv, AT, xcnt + 1, pl.xcap, xlist, at<double>(pl.mc_xsg));
+          mcmc_repair_build_kernel<T, LT><<<xcap, 256, 0, s>>>(n, xcnt + 1, xlist, PhiS, xb0);
+          lu_batch<LT>(s, n, xcap, xb0, xpiv, at<double>(pl.mc_xlab), at<double>(pl.mc_xsg), xcnt + 1);
+          inverse_warp<T>(n, xcap, xb0, xpiv, AT, xcnt + 1, xcap, xlist, at<double>(pl.mc_xsg));
           launches += 2;
           if (xover) {
             mcmc_repair_kernel<T, LT><<<kWoodburySlots, 256, inverse_panel_smem(n, sizeof(LT)), s>>>(
@@ -1477,7 +1485,7 @@ struct Runner {
                                                                Fk2);
         // pairs whose ratio needs a float64 LU of Phi', then that LU over all SMs
         mcmc_exact_select_kernel<<<(unsigned)((npair + 127) / 128), 128, 0, s>>>(
-            npair, D, Uc, lsign, lrat, xflag, xcnt, xlist, pl.xcap, xover, &ms->n_exact);
+            npair, D, Uc, lsign, lrat, xflag, xcnt, xlist, xcap, xover, &ms->n_exact);
         if (xover) {
           mcmc_exact_ratio_kernel<T, LT><<<kWoodburySlots, 256, (size_t)n * sizeof(int), s>>>(
               Wn, n, D, Umax, Ul, Uc, PhiS, Dl, ldabs, lsign, lrat, srat, at<LT>(pl.mc_rep), at<int32_t>(pl.mc_rpiv),
@@ -1487,10 +1495,10 @@ struct Runner {
         LT* xb = at<LT>(pl.mc_xbatch);
         double* xlab = at<double>(pl.mc_xlab);
         double* xsg = at<double>(pl.mc_xsg);
-        mcmc_exact_build_kernel<T, LT><<<pl.xcap, 256, (size_t)n * sizeof(int), s>>>(n, D, Umax, xcnt, xlist, Ul, Uc,
+        mcmc_exact_build_kernel<T, LT><<<xcap, 256, (size_t)n * sizeof(int), s>>>(n, D, Umax, xcnt, xlist, Ul, Uc,
                                                                                      PhiS, Dl, xb);
-        lu_batch<LT>(s, n, pl.xcap, xb, at<int32_t>(pl.mc_xpiv), xlab, xsg, xcnt);
-        mcmc_exact_scatter_kernel<<<(pl.xcap + 255) / 256, 256, 0, s>>>(xcnt, pl.xcap, xlist, xlab, xsg, ldabs,
+        lu_batch<LT>(s, n, xcap, xb, at<int32_t>(pl.mc_xpiv), xlab, xsg, xcnt);
+        mcmc_exact_scatter_kernel<<<(xcap + 255) / 256, 256, 0, s>>>(xcnt, xcap, xlist, xlab, xsg, ldabs,
                                                                        lsign, lrat, srat);
         launches += 3;
       }
@@ -1589,7 +1597,7 @@ struct Runner {
         mcmc_accept_kernel<T><<<Wn, kRatioThreads, 0, s>>>(Wn, n, n_up, D, k, Umax, dm.flags, r, rk, uacc, Ul, Uc, Urow, jp, F1,
                                                 F2, F1n, F2n, G1, G2, G1n, G2n, ldabs, lsign, lrat, srat, lp, acc,
                                                 mc.acc_count, &ms->n_accepted, lref, flag, xflag, lq, rcnt, rlist,
-                                                pl.xcap, &ms->n_repair);
+                                                xcap, &ms->n_repair);
         mcmc_rows_kernel<T><<<(unsigned)capU, 128, 0, s>>>(
             Wn, n, n_up, d, (int)Dn, RD, k, Umax, pl.ld_big, RD1, (dm.flags & FIRE_J_MLP) ? 1 : 0,
             (dm.flags & FIRE_J_ATT) ? 1 : 0, acc, Ul, Uc, Urow, F1n, F2n, F1, F2, SUn, SU, h0k, H0, PQk, PQ, Fk,
@@ -1624,13 +1632,13 @@ struct Runner {
           int32_t* xpiv = at<int32_t>(pl.mc_xpiv);
           double* xlab = at<double>(pl.mc_xlab);
           double* xsg = at<double>(pl.mc_xsg);
-          mcmc_repair_build_kernel<T, LT><<<pl.xcap, 256, 0, s>>>(n, rcnt, rlist, PhiS, xb);
-          lu_batch<LT>(s, n, pl.xcap, xb, xpiv, xlab, xsg, rcnt);
-          mcmc_repair_scatter_kernel<<<(pl.xcap + 255) / 256, 256, 0, s>>>(rcnt, pl.xcap, rlist, xlab, xsg, ldabs,
+          mcmc_repair_build_kernel<T, LT><<<xcap, 256, 0, s>>>(n, rcnt, rlist, PhiS, xb);
+          lu_batch<LT>(s, n, xcap, xb, xpiv, xlab, xsg, rcnt);
+          mcmc_repair_scatter_kernel<<<(xcap + 255) / 256, 256, 0, s>>>(rcnt, xcap, rlist, xlab, xsg, ldabs,
                                                                           lsign, lref);
-          mcmc_repair_choose_kernel<<<(pl.xcap + 255) / 256, 256, 0, s>>>(rcnt, pl.xcap, D, rlist, ldabs, lsign, kap,
+          mcmc_repair_choose_kernel<<<(xcap + 255) / 256, 256, 0, s>>>(rcnt, xcap, D, rlist, ldabs, lsign, kap,
                                                                          kunit, mc.kappa_tol, stale);
-          inverse_warp<T>(n, pl.xcap, xb, xpiv, AT, rcnt, pl.xcap, rlist, xsg);
+          inverse_warp<T>(n, xcap, xb, xpiv, AT, rcnt, xcap, rlist, xsg);
         }
         launches += 5;
         check("mc update");
