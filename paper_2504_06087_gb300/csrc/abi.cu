@@ -212,7 +212,7 @@ static size_t layout(Plan& pl, int64_t Wc) {
     TAKE(mc_stat, sizeof(McmcStat));
     TAKE(mc_wdrift, Wc * 8);
     TAKE(mc_lref, Wc * D * 8);         // log|det| of each matrix at its last factorisation
-    TAKE(mc_stale, Wc * D * 4);        // 1: refactorised, its inverse not formed yet
+    TAKE(mc_stale, Wc * D * 4);        // 1: refactorised under the conditioning test, without an inverse
     TAKE(mc_kap, Wc * D * 4);          // condition estimate of each matrix at the last refresh
     TAKE(mc_ecp, (int64_t)dm.N * (int64_t)sizeof(fire_ecp_t));   // pseudopotential table
     // the batched float64 LU of the exact ratios of ill-conditioned determinants

@@ -1596,30 +1596,17 @@ __device__ __forceinline__ bool untrusted(int64_t md, int D, const double* __res
 
 // Before a move: xflag = 2 for the pairs under the conditioning test, else 0
 // (walkers without a move, i.e. with an empty update set, are not tested).  A
-// determinant refactorised under the test has no inverse (stale): while it
-// stays there its ratios come from float64 LUs, which need none, and an
-// accepted move refactorises it again.  One that the lemma is going to use
-// after all gets its inverse now: it is listed, and marked in over where the
-// list (cap) is full.
-// One thread per pair.
+// determinant refactorised under the test has no inverse (stale): its ratios
+// come from float64 LUs, which need none, until an accepted move refactorises
+// it again.  One thread per pair.
 static __global__ void mcmc_exact_test_kernel(int64_t npair, int D, const int32_t* __restrict__ Uc,
                                               const double* __restrict__ ldabs, const double* __restrict__ lsign,
                                               const float* __restrict__ kap, double kunit, double ktol,
-                                              int32_t* __restrict__ xflag, int32_t* __restrict__ stale,
-                                              int* __restrict__ scount, int32_t* __restrict__ slist, int cap,
-                                              int32_t* __restrict__ over) {
+                                              const int32_t* __restrict__ stale, int32_t* __restrict__ xflag) {
   const int64_t md = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (md >= npair) return;
-  const bool cond = Uc[md / D] > 0 && untrusted(md, D, ldabs, lsign, kap, kunit, ktol);
+  const bool cond = Uc[md / D] > 0 && (stale[md] || untrusted(md, D, ldabs, lsign, kap, kunit, ktol));
   xflag[md] = cond ? 2 : 0;
-  int full = 0;
-  if (stale && stale[md] && !cond) {
-    stale[md] = 0;
-    const int slot = atomicAdd(scount, 1);
-    if (slot < cap) slist[slot] = (int32_t)md;
-    else full = 1;
-  }
-  if (over) over[md] = full;
 }
 
 // Lists the pairs whose ratio comes from a float64 LU of Phi' = Phi with the
@@ -1731,8 +1718,7 @@ static __global__ void mcmc_exact_scatter_kernel(const int* __restrict__ count, 
 // 2): a float64 copy of the cached Phi (already updated by the move) for the
 // LU, then log|det|, sign and the reference log|det| of the new factors, then
 // A^T from them, but not for those that the next move takes under the
-// conditioning test (mcmc_repair_choose_kernel).  The same copy and LU serve
-// the inverses formed later.  CTAs beyond the count leave.
+// conditioning test (mcmc_repair_choose_kernel).  CTAs beyond the count leave.
 template <typename T, typename LT>
 __global__ void __launch_bounds__(256) mcmc_repair_build_kernel(int n, const int* __restrict__ count,
                                                                 const int32_t* __restrict__ rlist,
@@ -1758,7 +1744,9 @@ static __global__ void mcmc_repair_scatter_kernel(const int* __restrict__ count,
 
 // After every log|det| of the move is in place: a refactorised pair that the
 // next move will find under the conditioning test stays without an inverse
-// (stale, its list entry -1).  Half of the inverses of a C14H16 sweep.
+// (stale, its list entry -1).  The walker's logs stay as they are until it
+// accepts a move, which refactorises the pair, so nothing reads the inverse
+// in between.  Half of the inverses of a C14H16 sweep.
 static __global__ void mcmc_repair_choose_kernel(const int* __restrict__ count, int cap, int D,
                                                  int32_t* __restrict__ rlist, const double* __restrict__ ldabs,
                                                  const double* __restrict__ lsign, const float* __restrict__ kap,
@@ -1773,8 +1761,7 @@ static __global__ void mcmc_repair_choose_kernel(const int* __restrict__ count, 
 
 // Refactorisation of the flagged (walker, det) pairs of accepted walkers
 // from the cached Phi (already updated by the move): log|det|, sign and A^T
-// (flag 1: those that the batched list had no room for).  Without acc: A^T
-// alone, of every flagged pair.
+// (flag 1: those that the batched list had no room for).
 // A persistent grid; CTA b uses slot b of the float64 scratch (n x n matrix,
 // n pivots) and dynamic shared memory for the inverse panel.
 template <typename T, typename LT>
@@ -1789,17 +1776,15 @@ __global__ void __launch_bounds__(256) mcmc_repair_kernel(int Wn, int n, int D, 
   LT* L = scratch + (int64_t)blockIdx.x * n * n;
   int32_t* pv = spiv + (int64_t)blockIdx.x * n;
   for (int64_t md = blockIdx.x; md < (int64_t)Wn * D; md += gridDim.x) {
-    if ((acc && !acc[md / D]) || flag[md] != 1) continue;
+    if (!acc[md / D] || flag[md] != 1) continue;
     const T* P = Phi + md * n * n;
     for (int e = threadIdx.x; e < n * n; e += blockDim.x) L[e] = (LT)P[e];
     __syncthreads();
     lu_block<LT>(n, L, pv, &s_la, &s_sg);
     if (threadIdx.x == 0) {
-      if (acc) {
-        ldabs[md] = s_la;
-        lsign[md] = s_sg;
-        lref[md] = s_la;
-      }
+      ldabs[md] = s_la;
+      lsign[md] = s_sg;
+      lref[md] = s_la;
       stale[md] = 0;
     }
     T* A = AT + md * n * n;

@@ -1311,8 +1311,8 @@ struct Runner {
     int32_t* flag = at<int32_t>(pl.mc_flag);
     int32_t* xflag = at<int32_t>(pl.mc_xflag);
     int32_t* stale = at<int32_t>(pl.mc_stale);
-    // pairs that the lists of exact ratios, refactorisations and late inverses
-    // hold; FIRE_MCMC_LIST (diagnostic) shortens them, so that the kernels that
+    // pairs that the lists of exact ratios and refactorisations hold;
+    // FIRE_MCMC_LIST (diagnostic) shortens them, so that the kernels that
     // take the pairs beyond can be tested on small batches
     int xcap = pl.xcap;
     if (const char* e = getenv("FIRE_MCMC_LIST")) {
@@ -1456,30 +1456,14 @@ struct Runner {
       check("mc orbitals");
       {
         const int64_t npair = (int64_t)Wn * D;
-        int* xcnt = at<int>(pl.mc_xcnt);   // [0] pairs with exact ratios, [1] inverses to be formed
+        int* xcnt = at<int>(pl.mc_xcnt);
         int32_t* xlist = at<int32_t>(pl.mc_xlist);
-        int32_t* pend = mc.ecp || mc.swap_beta >= 0 ? nullptr : stale;   // nothing is accepted there
         // only a batch beyond the lists' capacity leaves any pair to the per-CTA kernels
         int32_t* xover = npair > xcap ? at<int32_t>(pl.mc_flag) : nullptr;
-        LT* xb0 = at<LT>(pl.mc_xbatch);
-        mark("mc_inverse", 1);
-        cudaMemsetAsync(xcnt, 0, 2 * sizeof(int), s);
-        mcmc_exact_test_kernel<<<(unsigned)((npair + 127) / 128), 128, 0, s>>>(
-            npair, D, Uc, ldabs, lsign, kap, kunit, mc.kappa_tol, xflag, pend, xcnt + 1, xlist, xcap, xover);
-        if (pend) {
-          int32_t* xpiv = at<int32_t>(pl.mc_xpiv);
-          mcmc_repair_build_kernel<T, LT><<<xcap, 256, 0, s>>>(n, xcnt + 1, xlist, PhiS, xb0);
-          lu_batch<LT>(s, n, xcap, xb0, xpiv, at<double>(pl.mc_xlab), at<double>(pl.mc_xsg), xcnt + 1);
-          inverse_warp<T>(n, xcap, xb0, xpiv, AT, xcnt + 1, xcap, xlist, at<double>(pl.mc_xsg));
-          launches += 2;
-          if (xover) {
-            mcmc_repair_kernel<T, LT><<<kWoodburySlots, 256, inverse_panel_smem(n, sizeof(LT)), s>>>(
-                Wn, n, D, nullptr, xover, PhiS, AT, nullptr, nullptr, nullptr, at<LT>(pl.mc_rep),
-                at<int32_t>(pl.mc_rpiv), stale);
-            launches += 1;
-          }
-        }
-        mark("mc_ratio", 2);
+        cudaMemsetAsync(xcnt, 0, sizeof(int), s);
+        mark("mc_ratio", 3);
+        mcmc_exact_test_kernel<<<(unsigned)((npair + 127) / 128), 128, 0, s>>>(npair, D, Uc, ldabs, lsign, kap, kunit,
+                                                                              mc.kappa_tol, stale, xflag);
         mcmc_ratio_kernel<T><<<(unsigned)(Wn * D), 256, 0, s>>>(Wn, n, n_up, D, k, Umax, Ul, Uc, Urow, On, Fenv, Fk,
                                                                PhiS, AT, Dl, Mt, Mlu, Mpiv, lrat, srat, xflag, k2,
                                                                Fk2);
