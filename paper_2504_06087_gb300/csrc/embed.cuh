@@ -28,22 +28,8 @@ __device__ __forceinline__ void fl3_mul(const FL3<T>& a, const FL3<T>& b, FL3<T>
   o.l = a.l * b.v + T(2) * cross + a.v * b.l;
 }
 
-// Filter features of one pair vector into shared memory:
-// feat[0..H) hidden units, feat[H..H+G) Gaussians chi_g, feat[H+G..H+G+4) e-bar.
-template <typename T, typename W>
-__device__ __forceinline__ void pair_features_to_smem(const T dv[3], T r, const W* w1, const W* b1,
-                                                      const W* sigma, T cut, FL3<T>* feat) {
-  const int H = kEdgeHidden, G = kGauss;
-  for (int k = threadIdx.x; k < H + G + 4; k += blockDim.x) {
-    FL3<T> o;
-    if (k < H) pair_hidden<T, W>(dv, r, w1, b1, k, H, o);
-    else if (k < H + G) pair_chi<T>(dv, r, T(sigma[k - H]), cut, o);
-    else pair_ebar<T>(dv, r, k - H - G, o);
-    feat[k] = o;
-  }
-}
-
-// Feature k of one pair (the layout of pair_features_to_smem).
+// Filter feature k of one pair vector: hidden units 0 .. H-1, Gaussians chi_g
+// H .. H+G-1, then the four of e-bar.
 template <typename T, typename W>
 __device__ __forceinline__ FL3<T> pair_feature(int k, const T dv[3], T r, const W* w1, const W* b1,
                                                const W* sigma, T cut) {
