@@ -1001,7 +1001,6 @@ struct Runner {
         convert_kernel<LT, T><<<1024, 256, 0, s>>>((int64_t)wc * D * n * n, LUb, at<T>(pl.PhiS));
         launches += 1;
       }
-      const size_t lusm = lu_smem_bytes(n, sizeof(LT));
       // slogdet: when the inverse does not come from these factors (float
       // forms: Gauss-Jordan on a float copy of Phi; value-only calls), the
       // float64 LU may run on a second stream (FIRE_LU_SIDE=1) and join before
@@ -1013,7 +1012,7 @@ struct Runner {
       auto launch_lu_side = [&]() {
         cudaEventRecord(ev_fork, s);
         cudaStreamWaitEvent(s2, ev_fork, 0);
-        lu_kernel<LT, 16><<<wc * D, 256, lusm, s2>>>(n, LUb, piv, ldabs, lsign);
+        lu_batch<LT>(s2, n, wc * D, LUb, piv, ldabs, lsign);
         cudaEventRecord(ev_join, s2);
       };
       mark("lu", 1);

@@ -75,3 +75,13 @@ def test_log_determinant(n, prec):
     err = np.abs(out["logabs"].cpu().numpy() - la)
     t = 1e-10 if prec == "fp64" else 1e-5
     assert (err <= np.maximum(t * np.maximum(np.abs(la), 1.0), n * kappa * u)).all(), err
+
+
+@pytest.mark.parametrize("n", [58, 119, 120])
+def test_second_stream_factorises_alike(n, monkeypatch):
+    """FIRE_LU_SIDE moves the float64 LU to another stream: the same kernel, the same bits."""
+    s, arch, p, r = _model(n)
+    f = fire.Fire(s, arch, p, "bf16", k_cap=n)
+    ref = f.logpsi(r)["logabs"].cpu().numpy()
+    monkeypatch.setenv("FIRE_LU_SIDE", "1")
+    np.testing.assert_array_equal(f.logpsi(r)["logabs"].cpu().numpy(), ref)
