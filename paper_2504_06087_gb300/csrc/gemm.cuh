@@ -14,6 +14,7 @@
 #pragma once
 
 #include "common.cuh"
+#include "plan.h"
 
 namespace fire {
 
@@ -300,7 +301,7 @@ inline void gemm(cudaStream_t s, const T* A, int64_t lda, const T* B, int64_t ld
     gemm_launch<T, 16, 16, 32, 1, 2>(s, g, transB, m_cap, batch);
   } else {
     // the tile of least estimated time, in outputs of the 64 x 64 tile's rate:
-    // all tiles over 152 SMs, but no less than one tile alone takes (a lone
+    // all tiles over the SMs, but no less than one tile alone takes (a lone
     // 64-thread tile is a chain of loads and barriers: 3700 rows, N = K = 128,
     // 11 us against 8 with 32 x 32 tiles)
     struct Tile { int bm, bn; float eff, lone; };
@@ -309,7 +310,7 @@ inline void gemm(cudaStream_t s, const T* A, int64_t lda, const T* B, int64_t ld
     float cost = 3.4e38f;
     for (int q = 0; q < 3; ++q) {
       const int64_t tiles = ((m_cap + t[q].bm - 1) / t[q].bm) * ((g.N + t[q].bn - 1) / t[q].bn) * batch;
-      float c = (float)tiles * t[q].bm * t[q].bn / (152.f * t[q].eff);
+      float c = (float)tiles * t[q].bm * t[q].bn / ((float)kSMs * t[q].eff);
       if (c < t[q].lone) c = t[q].lone + 1e-3f * c;
       if (c < cost) { cost = c; best = q; }
     }

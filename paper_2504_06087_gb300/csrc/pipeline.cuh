@@ -651,7 +651,7 @@ struct Runner {
       {
         // electrons of a CTA: as many as leave four CTAs per SM (the CTA's
         // weight sums are added to the walker's row once)
-        int epc = (int)((int64_t)nb / (152 * 4));
+        int epc = (int)((int64_t)nb / (kSMs * 4));
         epc = epc < 1 ? 1 : (epc > kGradElectrons ? kGradElectrons : epc);
         if (epc > n) epc = n;
         const unsigned ctas = (unsigned)(wc * ((n + epc - 1) / epc));
@@ -688,7 +688,7 @@ struct Runner {
       mark("bwd_en", 1);
       {
         int seg = kGradSeg;   // electrons of a CTA: shorter segments until four CTAs per SM exist
-        while (seg > kGradPairs && (int64_t)wc * N * ((n + seg - 1) / seg) < 152 * 4) seg /= 2;
+        while (seg > kGradPairs && (int64_t)wc * N * ((n + seg - 1) / seg) < kSMs * 4) seg /= 2;
         const unsigned ctas = (unsigned)((int64_t)wc * N * ((n + seg - 1) / seg));
         en_bwd_kernel<T, T><<<ctas, d, filter_grad_smem<T>(d), s>>>(wc, n, n_up, N, d, seg, r, sys->nuc_pos,
                                                                     sys->cutoff_nuc, p, B.dS5, g, P, pod);
@@ -1365,7 +1365,7 @@ struct Runner {
     if (rc != FIRE_OK) return rc;
 
     const double c = sys->cutoff;
-    const unsigned actg = 152 * 8;
+    const unsigned actg = kSMs * 8;
     const McmcJastrow jp{p.cusp, p.jm2_b3, p.ja2_b3};
     const size_t msm = (size_t)n * sizeof(int);
     const size_t asm_ = (((size_t)n * sizeof(int) + 15) & ~(size_t)15) + (size_t)R * sizeof(T);

@@ -8,6 +8,10 @@
 
 namespace fire {
 
+// SMs of a GB300: the host rules that choose tiles, groups and grids count
+// with it.
+constexpr int kSMs = 152;
+
 struct Dims {
   int n, n_up, N, d, L, D, E, G, H, J, R, dr, K;
   uint32_t flags;
@@ -65,7 +69,7 @@ constexpr int kOrbGroup = 4;
 
 // CTAs (and scratch slots) of the Woodbury update: a persistent grid over
 // the (walker, determinant) pairs, 4 per SM.
-constexpr int kWoodburySlots = 152 * 4;
+constexpr int kWoodburySlots = kSMs * 4;
 
 // Device counters of a Metropolis call.
 struct McmcStat {

@@ -25,6 +25,7 @@
 #include <stdint.h>
 
 #include "../../include/fire.h"
+#include "plan.h"
 #include "tc_api.h"
 
 namespace fire {
@@ -49,14 +50,14 @@ struct Layout {
 
 // Chunks per product launch: the fewest that keep nine tenths of the SMs (a
 // CTA of 128 x 128 outputs each) busy to the last round, within 512 MB of
-// packed rows.  N = 1024 (64 tiles of a chunk on 152 SMs): 7.
+// packed rows.  N = 1024 (64 tiles of a chunk): 7.
 inline int chunk_groups(int64_t N, int64_t pc, int64_t nchunk) {
   const int64_t tiles = ((N + 127) / 128) * ((N + 127) / 128);
   int best = 1;
   double eff = 0.0;
-  for (int64_t g = 1; g <= 152 && g <= nchunk && (g == 1 || g * kNC * N * pc * 2 <= (512ll << 20)); ++g) {
+  for (int64_t g = 1; g <= kSMs && g <= nchunk && (g == 1 || g * kNC * N * pc * 2 <= (512ll << 20)); ++g) {
     const int64_t t = tiles * g;
-    const double e = (double)t / (double)((t + 151) / 152 * 152);
+    const double e = (double)t / (double)((t + kSMs - 1) / kSMs * kSMs);
     if (e > eff) { eff = e; best = (int)g; }
     if (e >= 0.9) break;
   }
@@ -584,7 +585,7 @@ extern "C" int fire_spring_step(int64_t n_walkers, int64_t n_params, const float
   colmean_kernel<<<(unsigned)((P + 255) / 256), 256, 0, s>>>(N, P, O, ldo, mean);
   double* scal = reinterpret_cast<double*>(w + L.scal);   // abar, mu, mean . dprev, sum x
   if (cudaMemsetAsync(scal, 0, 32, s) != cudaSuccess) return FIRE_ERR_CUDA;
-  if (delta_prev) meandot_kernel<<<152, 256, 0, s>>>(P, mean, delta_prev, scal + 2);
+  if (delta_prev) meandot_kernel<<<fire::kSMs, 256, 0, s>>>(P, mean, delta_prev, scal + 2);
   // Gram matrix over chunks of the parameter axis, L.groups of them per launch
   // (the last chunks alone where the axis does not fill a group)
   const int vec = ldo % 4 == 0 && (reinterpret_cast<uintptr_t>(O) & 15) == 0;
@@ -607,12 +608,12 @@ extern "C" int fire_spring_step(int64_t n_walkers, int64_t n_params, const float
   // exact centring in float64: Obar Obar^T = P G P
   double* a = reinterpret_cast<double*>(w + L.a);
   rowmean_kernel<<<(unsigned)((N + 7) / 8), 256, 0, s>>>(N, Np, K, a);
-  center_kernel<<<608, 1024, 0, s>>>(N, Np, K, a, scal);
+  center_kernel<<<4 * fire::kSMs, 1024, 0, s>>>(N, Np, K, a, scal);
   if (gram) cudaMemcpy2DAsync(gram, (size_t)N * 8, K, (size_t)Np * 8, (size_t)N * 8, (size_t)N,
                               cudaMemcpyDeviceToDevice, s);
   rhs_kernel<<<1, 1024, 0, s>>>(N, Np, e_loc, delta_prev ? rowdot : nullptr, scal + 2, eta, lambda, b, K,
                                 scal + 1);
-  lift_kernel<<<608, 256, 0, s>>>(N, Np, K, scal + 1);
+  lift_kernel<<<4 * fire::kSMs, 256, 0, s>>>(N, Np, K, scal + 1);
   // float64 Cholesky of K + lambda I, then the two triangular solves
   const int nb = (int)(Np / kB);
   const size_t usm = 2 * (size_t)kB * (kB + 1) * 8;
