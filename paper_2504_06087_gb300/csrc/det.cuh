@@ -485,7 +485,13 @@ __global__ void __launch_bounds__(384, 1) gj_inverse_kernel(int n, const IT* __r
             if (ov > best || (ov == best && oi < bi)) { best = ov; bi = oi; }
           }
           if (tid == 0) {
-            if (bi >= n) bi = 0;   // singular: any row, the result is not finite
+            // a column without a finite entry left (an exactly singular matrix
+            // after its zero pivot): any unused row, so that piv and stp stay
+            // permutations; the result is not finite
+            if (bi >= n) {
+              bi = 0;
+              while (used[bi]) ++bi;   // fewer than n rows are used before step k
+            }
             piv[k] = bi;
             stp[bi] = k;
             used[bi] = 1;
