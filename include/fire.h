@@ -146,8 +146,8 @@ typedef struct {
   int32_t n_layers;          /* depth L of the embedding MLP h = MLP(h^1)       */
   int32_t n_det;             /* determinants N_det                              */
   int32_t n_env;             /* exponential envelopes per nucleus               */
-  int32_t n_gauss;           /* Gaussians d_0 of the radial filters (<= 64)     */
-  int32_t edge_hidden;       /* hidden width of the filter MLP (<= 64)          */
+  int32_t n_gauss;           /* Gaussians d_0 of the radial filters (32)        */
+  int32_t edge_hidden;       /* hidden width of the filter MLP (16)             */
   int32_t jastrow_width;     /* hidden width of the Jastrow MLPs (0 = width)    */
   int32_t n_reg;             /* attention registers                             */
   int32_t d_reg;             /* register dimension                              */

@@ -351,7 +351,7 @@ __device__ __forceinline__ int lu_smem_core(int n, LT* S, int ld, int32_t* __res
 // The LU of lu_kernel (same pivots, same chain of operations per element) with
 // the whole matrix in shared memory, one CTA per matrix: no panel copies and
 // no row interchanges in global memory.  Two CTAs per SM fit up to n = 119
-// (float64) or 168 (float32); beyond that the blocked kernel, which keeps only
+// (float64) or 169 (float32); beyond that the blocked kernel, which keeps only
 // a panel, is the faster one.  512 matrices of n = 58, a few of them present:
 // 181 us blocked, 105 with the pivot chain in the open, 82 now.
 template <typename LT>
